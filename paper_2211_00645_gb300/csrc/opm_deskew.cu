@@ -1,10 +1,15 @@
 // Full-volume deskew (Fig. 2c remap with linear interpolation between scan
 // planes).  Output-write bound: every voxel is written once with streaming
-// stores.  Each thread walks a run of output columns j of one row k and keeps
-// the current pair of raw planes in registers, so a raw vector is fetched once
-// per plane step rather than once per voxel.  A lane owns two half-vectors of
-// columns 32*HALF apart, so that every store instruction of a warp covers one
-// contiguous span of 32*HALF elements.
+// stores.  Each warp walks a run of kRunJ output columns j of one row k and
+// keeps the current pair of raw planes in registers, so a raw vector is
+// fetched once per plane step rather than once per voxel.  The run's planes
+// and weights are worked out by the warp's lanes side by side, one column
+// each, and handed round by shuffles; the plane after the current pair is
+// already on its way when the walk steps onto it.
+// A lane owns NH vectors of H columns x, 32 H apart, so that every load and
+// store instruction of a warp covers one contiguous span.
+#include <algorithm>
+
 #include "opm_common.cuh"
 
 namespace opm {
@@ -13,149 +18,206 @@ namespace {
 
 constexpr int kThreadsX = 32;  // lanes along x
 constexpr int kThreadsY = 4;   // j-runs per CTA
-constexpr int kRunJ = 32;      // output columns per thread
+constexpr int kRunJ = 32;      // output columns per warp, one per lane for the plane table
 
-template <typename T, int N, typename Acc>
-__device__ __forceinline__ void load_half(const T* __restrict__ p, bool vec, int lim, Acc (&out)[N]) {
-  static_assert(sizeof(T) * N == 8, "8-byte half vectors");
-  if (vec) {
+// H raw elements as loaded: 8 or 16 bytes, or a single element.
+template <typename T, int H>
+struct RawVec {
+  static_assert(H == 1 || sizeof(T) * H == 8 || sizeof(T) * H == 16, "8- or 16-byte vectors");
+  uint32_t w[(sizeof(T) * H + 3) / 4];
+};
+
+template <typename T, int H>
+__device__ __forceinline__ void load_raw(const T* __restrict__ p, RawVec<T, H>& out) {
+  if constexpr (sizeof(T) * H == 16) {
+    const uint4 u = __ldg(reinterpret_cast<const uint4*>(p));
+    out.w[0] = u.x, out.w[1] = u.y, out.w[2] = u.z, out.w[3] = u.w;
+  } else if constexpr (sizeof(T) * H == 8) {
     const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
-    const T* e = reinterpret_cast<const T*>(&u);
-#pragma unroll
-    for (int i = 0; i < N; ++i) out[i] = static_cast<Acc>(e[i]);
+    out.w[0] = u.x, out.w[1] = u.y;
   } else {
-#pragma unroll
-    for (int i = 0; i < N; ++i) out[i] = i < lim ? static_cast<Acc>(__ldg(p + i)) : Acc(0);
+    *reinterpret_cast<T*>(out.w) = __ldg(p);
   }
 }
 
-// Stores one half-vector of H output values with streaming stores (16-byte
-// FP32 or 8-byte uint16 vectors when `full`), else element by element.
-template <typename Tout, int H, typename Acc>
-__device__ __forceinline__ void store_half(Tout* op, const Acc (&val)[H], bool full, int lim) {
-  if constexpr (std::is_same<Tout, float>::value && H == 4) {
-    if (full) {
-      st_cs_v4(op, val[0], val[1], val[2], val[3]);
-      return;
-    }
-  }
-  if constexpr (std::is_same<Tout, uint16_t>::value && H == 4) {
-    if (full) {
-      const uint32_t lo = (uint32_t)to_u16_rn(val[0]) | ((uint32_t)to_u16_rn(val[1]) << 16);
-      const uint32_t hi = (uint32_t)to_u16_rn(val[2]) | ((uint32_t)to_u16_rn(val[3]) << 16);
-      asm volatile("st.global.cs.v2.b32 [%0], {%1, %2};" ::"l"(op), "r"(lo), "r"(hi) : "memory");
-      return;
-    }
-  }
-  if constexpr (std::is_same<Tout, float>::value && H == 2) {
-    if (full) {
-      asm volatile("st.global.cs.v2.f32 [%0], {%1, %2};" ::"l"(op), "f"(val[0]), "f"(val[1]) : "memory");
-      return;
-    }
-  }
+// Raw elements as accumulator values.  uint16: 2^23 + u in the float's bit
+// pattern by a byte permute, then 2^23 off again, exact and off the
+// conversion unit (cvt.f32.u16 issues once in 8 cycles).
+template <typename T, int H, typename Acc>
+__device__ __forceinline__ void widen(const RawVec<T, H>& r, Acc (&out)[H]) {
+  if constexpr (std::is_same<T, uint16_t>::value) {
 #pragma unroll
-  for (int i = 0; i < H; ++i) {
-    if (i >= lim) break;
-    if constexpr (std::is_same<Tout, uint16_t>::value)
-      op[i] = to_u16_rn(val[i]);
+    for (int i = 0; i < H; ++i)
+      out[i] = __uint_as_float(__byte_perm(r.w[i / 2], 0x4B000000u, i % 2 ? 0x7632 : 0x7610)) - 8388608.0f;
+  } else {
+    const T* e = reinterpret_cast<const T*>(r.w);
+#pragma unroll
+    for (int i = 0; i < H; ++i) out[i] = static_cast<Acc>(e[i]);
+  }
+}
+
+// Two values in [0, 65535] rounded half to even, packed: adding 2^23 leaves
+// the rounded integer in the low bits of the pattern.
+__device__ __forceinline__ uint32_t pack_rn(float lo, float hi) {
+  return __byte_perm(__float_as_uint(lo + 8388608.0f), __float_as_uint(hi + 8388608.0f), 0x5410);
+}
+
+// Stores one vector of H output values with streaming stores.  `INSIDE`: the
+// values are known to lie in [0, 65535] (interpolated uint16 counts).
+template <typename Tout, int H, bool INSIDE, typename Acc>
+__device__ __forceinline__ void store_vec(Tout* op, const Acc (&val)[H]) {
+  if constexpr (std::is_same<Tout, uint16_t>::value && H > 1) {
+    uint32_t q[H / 2];
+#pragma unroll
+    for (int i = 0; i < H / 2; ++i) {
+      if constexpr (INSIDE)
+        q[i] = pack_rn(val[2 * i], val[2 * i + 1]);
+      else  // clamp; NaN maps to 0
+        q[i] = pack_rn(fminf(fmaxf(val[2 * i], 0.0f), 65535.0f), fminf(fmaxf(val[2 * i + 1], 0.0f), 65535.0f));
+    }
+    if constexpr (H == 8)
+      st_cs_v4u(op, q[0], q[1], q[2], q[3]);
+    else if constexpr (H == 4)
+      asm volatile("st.global.cs.v2.b32 [%0], {%1, %2};" ::"l"(op), "r"(q[0]), "r"(q[1]) : "memory");
     else
-      op[i] = (Tout)val[i];
+      asm volatile("st.global.cs.b32 [%0], %1;" ::"l"(op), "r"(q[0]) : "memory");
+  } else if constexpr (std::is_same<Tout, uint16_t>::value) {
+    __stcs(op, to_u16_rn(val[0]));
+  } else if constexpr (std::is_same<Tout, float>::value && H == 4) {
+    st_cs_v4(op, val[0], val[1], val[2], val[3]);
+  } else if constexpr (std::is_same<Tout, float>::value && H == 2) {
+    asm volatile("st.global.cs.v2.f32 [%0], {%1, %2};" ::"l"(op), "f"(val[0]), "f"(val[1]) : "memory");
+  } else {
+    static_assert(H == 1, "vectors of 4 or 2 floats");
+    __stcs(op, (Tout)val[0]);
   }
 }
 
 // vol2 (uint16, may be NULL unless DUAL) receives the round-to-nearest-even
 // copy of the same values in the same pass.
-template <typename Tin, typename Tout, typename Acc, int VEC, bool DUAL>
+template <typename Tin, typename Tout, typename Acc, int H, int NH, bool DUAL>
 __global__ void __launch_bounds__(kThreadsX* kThreadsY)
-k_deskew(PlanView v, const Tin* __restrict__ raw, Tout* __restrict__ vol, uint16_t* __restrict__ vol2, int xtiles,
-         int in_vec_ok, int out_vec_ok, int out2_vec_ok) {
-  constexpr int H = VEC / 2;  // elements per half-vector
+k_deskew(PlanView v, const Tin* __restrict__ raw, Tout* __restrict__ vol, uint16_t* __restrict__ vol2,
+         int xtiles) {
+  constexpr bool kInside = std::is_same<Tin, uint16_t>::value;
   const int k = blockIdx.x / xtiles;
   const int xt = blockIdx.x - k * xtiles;
-  const int xh[2] = {xt * kThreadsX * VEC + (int)threadIdx.x * H,
-                     xt * kThreadsX * VEC + kThreadsX * H + (int)threadIdx.x * H};
-  if (xh[0] >= v.nx) return;
-  const int lim[2] = {v.nx - xh[0], v.nx - xh[1]};  // valid columns of each half
+  const int lane = threadIdx.x;
+  int xh[NH], lim[NH];  // first column and valid columns of each vector
+#pragma unroll
+  for (int h = 0; h < NH; ++h) {
+    xh[h] = xt * kThreadsX * H * NH + h * kThreadsX * H + lane * H;
+    lim[h] = v.nx - xh[h];
+  }
   const int jb = (blockIdx.y * kThreadsY + threadIdx.y) * kRunJ;
   if (jb >= v.ny) return;
-  const Split b = v.B[k];
+  const int nj = min(kRunJ, v.ny - jb);
   const size_t plane = (size_t)v.nrows * v.ncols;
   const Tin* rowp = raw + (size_t)k * v.ncols;
 
-  Acc a[2][H], bb[2][H], d[2][H];
-#pragma unroll
-  for (int h = 0; h < 2; ++h)
-#pragma unroll
-    for (int i = 0; i < H; ++i) a[h][i] = bb[h][i] = d[h][i] = Acc(0);
-  int ocur = -0x40000000;  // plane index held in a[] (none yet)
+  // lane l: lower plane and weight of column jb + l, and whether the walk
+  // changes planes there
+  int nl;
+  Acc wl;
+  plane_weight_t<Acc>(v.A[min(jb + lane, v.ny - 1)], v.B[k], v.linear, nl, wl);
+  const int nprev = __shfl_up_sync(0xffffffffu, nl, 1);
+  const unsigned change = __ballot_sync(0xffffffffu, lane == 0 || nl != nprev);
 
-  auto fetch = [&](int n, Acc(&out)[2][H]) {
+  auto fetch = [&](int n, RawVec<Tin, H>(&out)[NH]) {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < NH; ++h) {
       if (n >= 0 && n < v.nscan && lim[h] > 0) {
-        load_half<Tin, H, Acc>(rowp + (size_t)n * plane + xh[h], in_vec_ok && lim[h] >= H, lim[h], out[h]);
+        load_raw<Tin, H>(rowp + (size_t)n * plane + xh[h], out[h]);
       } else {
 #pragma unroll
-        for (int i = 0; i < H; ++i) out[h][i] = Acc(0);
+        for (int i = 0; i < (int)sizeof(out[h].w) / 4; ++i) out[h].w[i] = 0u;
       }
     }
   };
 
+  Acc a[NH][H], b[NH][H], d[NH][H];
+  RawVec<Tin, H> next[NH];  // plane ocur + 2
+  int ocur = -0x40000000;   // plane index held in a[] (none yet)
+#pragma unroll
+  for (int h = 0; h < NH; ++h)
+#pragma unroll
+    for (int i = 0; i < H; ++i) a[h][i] = b[h][i] = d[h][i] = Acc(0);
+  size_t orow = ((size_t)k * v.ny + jb) * v.nx;
+
 #pragma unroll 1
-  for (int jj = 0; jj < kRunJ; ++jj) {
-    const int j = jb + jj;
-    if (j >= v.ny) break;
-    int n0;
-    Acc w;
-    plane_weight_t<Acc>(v.A[j], b, v.linear, n0, w);
-    if (n0 != ocur) {
+  for (int jj = 0; jj < nj; ++jj, orow += v.nx) {
+    if ((change >> jj) & 1u) {
+      const int n0 = __shfl_sync(0xffffffffu, nl, jj);
       if (n0 == ocur + 1) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+        for (int h = 0; h < NH; ++h) {
 #pragma unroll
-          for (int i = 0; i < H; ++i) a[h][i] = bb[h][i];
+          for (int i = 0; i < H; ++i) a[h][i] = b[h][i];
+          widen<Tin, H, Acc>(next[h], b[h]);
+        }
       } else {
-        fetch(n0, a);
+        RawVec<Tin, H> r0[NH], r1[NH];
+        fetch(n0, r0);
+        fetch(n0 + 1, r1);
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+          widen<Tin, H, Acc>(r0[h], a[h]);
+          widen<Tin, H, Acc>(r1[h], b[h]);
+        }
       }
-      fetch(n0 + 1, bb);
+      fetch(n0 + 2, next);
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
+      for (int h = 0; h < NH; ++h)
 #pragma unroll
-        for (int i = 0; i < H; ++i) d[h][i] = bb[h][i] - a[h][i];
+        for (int i = 0; i < H; ++i) d[h][i] = b[h][i] - a[h][i];
       ocur = n0;
     }
-    const size_t orow = ((size_t)k * v.ny + j) * v.nx;
+    const Acc w = __shfl_sync(0xffffffffu, wl, jj);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < NH; ++h) {
       if (lim[h] <= 0) continue;
       Acc val[H];
 #pragma unroll
       for (int i = 0; i < H; ++i) val[i] = fma(w, d[h][i], a[h][i]);
-      store_half<Tout, H, Acc>(vol + orow + xh[h], val, out_vec_ok && lim[h] >= H, lim[h]);
-      if constexpr (DUAL) store_half<uint16_t, H, Acc>(vol2 + orow + xh[h], val, out2_vec_ok && lim[h] >= H, lim[h]);
+      store_vec<Tout, H, kInside>(vol + orow + xh[h], val);
+      if constexpr (DUAL)
+        store_vec<uint16_t, H, kInside>(vol2 + orow + xh[h], val);
     }
   }
 }
 
-template <typename Tin, typename Tout, typename Acc, int VEC, bool DUAL = false>
+// Whether every row of an array starts on a vector of H elements.
+template <typename T, int H>
+bool aligned(const void* q, int n) {
+  return n % H == 0 && (uintptr_t)q % (sizeof(T) * H) == 0;
+}
+
+template <typename Tin, typename Tout, typename Acc, int H, int NH, bool DUAL>
 opm_status run(const opm_plan* p, const void* raw, void* vol, void* vol2, cudaStream_t s) {
-  constexpr int H = VEC / 2;
   const PlanView& v = p->view;
-  const int xtiles = (v.nx + kThreadsX * VEC - 1) / (kThreadsX * VEC);
+  const int xtiles = (v.nx + kThreadsX * H * NH - 1) / (kThreadsX * H * NH);
   const long long gx = (long long)xtiles * v.nz;
   const int gy = (v.ny + kThreadsY * kRunJ - 1) / (kThreadsY * kRunJ);
   if (gx > 0x7fffffffLL || gy > 65535)
     return fail(OPM_ERR_UNSUPPORTED, "deskew grid exceeds launch limits");
-  const int in_vec_ok = (v.ncols % H == 0) && ((uintptr_t)raw % 8 == 0);
-  const int out_vec_ok = (v.nx % H == 0) && ((uintptr_t)vol % (sizeof(Tout) * H) == 0);
-  const int out2_vec_ok = (v.nx % H == 0) && ((uintptr_t)vol2 % (sizeof(uint16_t) * H) == 0);
   dim3 block(kThreadsX, kThreadsY);
   dim3 grid((unsigned)gx, (unsigned)gy);
-  k_deskew<Tin, Tout, Acc, VEC, DUAL><<<grid, block, 0, s>>>(v, static_cast<const Tin*>(raw), static_cast<Tout*>(vol),
-                                                             static_cast<uint16_t*>(vol2), xtiles, in_vec_ok,
-                                                             out_vec_ok, out2_vec_ok);
+  k_deskew<Tin, Tout, Acc, H, NH, DUAL><<<grid, block, 0, s>>>(v, static_cast<const Tin*>(raw), static_cast<Tout*>(vol),
+                                                               static_cast<uint16_t*>(vol2), xtiles);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? OPM_OK : cuda_fail(e, "launch k_deskew");
+}
+
+// Vectors of H elements when the rows of every array start on one; else one
+// element per lane and instruction, NH1 per lane: contiguous for the warp,
+// where element-wise vectors would leave strides of H between lanes.
+template <typename Tin, typename Tout, typename Acc, int H, int NH, bool DUAL = false>
+opm_status run_aligned(const opm_plan* p, const void* raw, void* vol, void* vol2, cudaStream_t s) {
+  constexpr int kNH1 = 4;
+  const int nx = p->view.nx;
+  if (aligned<Tin, H>(raw, nx) && aligned<Tout, H>(vol, nx) && (!DUAL || aligned<uint16_t, H>(vol2, nx)))
+    return run<Tin, Tout, Acc, H, NH, DUAL>(p, raw, vol, vol2, s);
+  return run<Tin, Tout, Acc, 1, kNH1, DUAL>(p, raw, vol, vol2, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -308,18 +370,23 @@ __global__ void k_zero2(float* a, long long na, float* b, long long nb) {
 
 opm_status launch_deskew(const opm_plan* p, const void* raw, opm_dtype in_t, void* vol,
                          opm_dtype out_t, cudaStream_t s) {
-  if (in_t == OPM_U16 && out_t == OPM_F32) return run<uint16_t, float, float, 8>(p, raw, vol, nullptr, s);
-  if (in_t == OPM_U16 && out_t == OPM_U16) return run<uint16_t, uint16_t, float, 8>(p, raw, vol, nullptr, s);
-  if (in_t == OPM_F32 && out_t == OPM_F32) return run<float, float, float, 4>(p, raw, vol, nullptr, s);
-  if (in_t == OPM_F32 && out_t == OPM_U16) return run<float, uint16_t, float, 4>(p, raw, vol, nullptr, s);
-  if (in_t == OPM_F64 && out_t == OPM_F64) return run<double, double, double, 2>(p, raw, vol, nullptr, s);
+  if (in_t == OPM_U16 && out_t == OPM_F32) return run_aligned<uint16_t, float, float, 4, 2>(p, raw, vol, nullptr, s);
+  if (in_t == OPM_U16 && out_t == OPM_U16) {
+    // 16-byte vectors where the rows allow them
+    if (aligned<uint16_t, 8>(raw, p->view.nx) && aligned<uint16_t, 8>(vol, p->view.nx))
+      return run<uint16_t, uint16_t, float, 8, 1, false>(p, raw, vol, nullptr, s);
+    return run_aligned<uint16_t, uint16_t, float, 4, 2>(p, raw, vol, nullptr, s);
+  }
+  if (in_t == OPM_F32 && out_t == OPM_F32) return run_aligned<float, float, float, 4, 1>(p, raw, vol, nullptr, s);
+  if (in_t == OPM_F32 && out_t == OPM_U16) return run_aligned<float, uint16_t, float, 4, 1>(p, raw, vol, nullptr, s);
+  if (in_t == OPM_F64 && out_t == OPM_F64) return run<double, double, double, 1, 2, false>(p, raw, vol, nullptr, s);
   return fail(OPM_ERR_UNSUPPORTED, "unsupported dtype pair");
 }
 
 opm_status launch_deskew_dual(const opm_plan* p, const void* raw, opm_dtype in_t, float* vol_f32, uint16_t* vol_u16,
                               cudaStream_t s) {
-  if (in_t == OPM_U16) return run<uint16_t, float, float, 8, true>(p, raw, vol_f32, vol_u16, s);
-  if (in_t == OPM_F32) return run<float, float, float, 4, true>(p, raw, vol_f32, vol_u16, s);
+  if (in_t == OPM_U16) return run_aligned<uint16_t, float, float, 4, 2, true>(p, raw, vol_f32, vol_u16, s);
+  if (in_t == OPM_F32) return run_aligned<float, float, float, 4, 1, true>(p, raw, vol_f32, vol_u16, s);
   return fail(OPM_ERR_UNSUPPORTED, "dual-output deskew takes uint16 or FP32 input");
 }
 
