@@ -42,7 +42,7 @@ UNIT = "GB/s"
 # Sources each timed kernel is compiled from: a change to any of them voids
 # the stored ncu traffic figure.
 KERNEL_SOURCES = {
-    "periodic": ["csrc/opm_project.cu", "csrc/opm_periodic.cuh", "csrc/opm_gen.cuh", "csrc/opm_tma.cuh",
+    "periodic": ["csrc/opm_project.cu", "csrc/opm_periodic.cuh", "csrc/opm_direct.cuh", "csrc/opm_tma.cuh",
                  "csrc/opm_common.cuh", "csrc/opm_internal.h", "csrc/opm_sched.h", "csrc/opm_plan.cu",
                  "../include/opm.h"],
     "liveview": ["csrc/opm_project.cu", "csrc/opm_tma.cuh", "csrc/opm_common.cuh", "csrc/opm_internal.h",

@@ -95,8 +95,8 @@ opm_status opm_plan_shape(const opm_plan* plan, int64_t* nz, int64_t* ny,
  *   *path = OPM_PATH_GENERAL: the general kernel (any plan; also every call
  *           with z-sum or arg-max output, or FP32 input).
  * Any output pointer may be NULL.  Errors: OPM_ERR_INVALID_ARG (plan NULL).
- * The raw stack's alignment is not known here; opm_project takes the plain
- * kernels when a row is not a multiple of 16 bytes or raw is misaligned.
+ * The raw stack's alignment is not known here; opm_project takes the general
+ * kernel when a row is not a multiple of 16 bytes or raw is misaligned.
  */
 typedef enum { OPM_PATH_GENERAL = 0, OPM_PATH_FAST = 1, OPM_PATH_PERIODIC = 2 } opm_path;
 opm_status opm_plan_path(const opm_plan* plan, int* path, int* fam_p, int* fam_q);
@@ -374,8 +374,8 @@ typedef enum {
   OPM_SHAPE_PER_J32X2 = 2, /* periodic kernel: 32 columns j per warp x 2 x per lane      */
   OPM_SHAPE_PER_J16X2 = 3, /* periodic kernel: 16 columns j per warp x 2 x per lane      */
                            /* (family 1/3; other families run as PER_J32X2)              */
-  OPM_SHAPE_GEN_J8X4 = 4   /* general kernel for every item: 8 j x 4 x, whole row band   */
-                           /* per unit, one row per stage                                 */
+  OPM_SHAPE_GEN_J8X4 = 4   /* general kernel for every item: 8 columns j per warp x 4     */
+                           /* columns x per lane, whole row band per unit                 */
 } opm_shape;
 
 /*

@@ -38,7 +38,7 @@
 #include <string>
 
 #include "opm_sched.h"
-#include "opm_gen.cuh"
+#include "opm_direct.cuh"
 #include "opm_periodic.cuh"
 
 namespace opm {
@@ -66,14 +66,19 @@ struct BatchItemDev {  // 64-byte aligned through its tensor map
   CUtensorMap tmap;      // raw stack of the item, box {128, 1, P}
   const FastRow* frow;   // fast-kernel tables, [ntile][nz] (fast items)
   const int* fnlo;       // [ntile][nz]
-  const Split* A;        // split tables (general items)
+  const Split* A;        // split tables and row bands (general items)
   const Split* B;
+  const Band* band;
+  const uint16_t* raw;   // sample (0, 0, 0) and pitches in elements (general items)
+  long long row_pitch, plane_pitch;
   float* zmip;
   float* ymip;
   float* zsum;
   int32_t* argz;
   int nz, ny, nx, P;
-  int linear;
+  int linear, nscan;
+  short wr, slots;       // row groups, staged planes and vector rows of the direct kernel (general items)
+  int vec;
 };
 static_assert(sizeof(BatchItemDev) == 256, "item");
 
@@ -224,70 +229,72 @@ k_batch_per(const unsigned char* __restrict__ wl, int Pl, unsigned* err) {
   if (warp == 0) per_drain(ring, g, ok, err);
 }
 
-// The general kernel's persistent loop (opm_gen.cuh) over the items the
-// fast kernels do not take: one unit per (x-tile, j-tile) and whole row
-// band, on one ring of slab depth Pg whose stage counter carries on across
-// units.
+// The general kernel: the direct kernel's jobs (opm_direct.cuh) over the
+// items the fast kernels do not take.  A unit is the whole row band of `pad`
+// columns from column `jt` at one x-tile: one CTA-wide piece of the item's row
+// groups, or the 32-column j-tile's pieces one after another where the work
+// list has no room for single ones.
 constexpr int kGenCtasPerSm = 2;
+// Planes per tile row that the general kernel's items may span.
+constexpr int kGenMaxPlanes = 221;
 
-__global__ void __launch_bounds__(kThreads, kGenCtasPerSm)
-k_batch_gen(const unsigned char* __restrict__ wl, int Pg, unsigned* err) {
+// Every form of the direct kernel's job is a function of its own, so that the
+// items with fewer outputs do not pay for the registers of the others.
+template <bool VEC, bool JUMP, bool SUM, bool ARG>
+__device__ __noinline__ void gen_tile(const direct::Job& jb, unsigned char* smem) {
+  direct::tile<uint16_t, VEC, SUM, ARG, JUMP>(jb, smem);
+}
+
+template <bool VEC, bool JUMP>
+__device__ __forceinline__ void gen_job(const direct::Job& jb, unsigned char* smem) {
+  if (jb.argz)
+    jb.zsum ? gen_tile<VEC, JUMP, true, true>(jb, smem) : gen_tile<VEC, JUMP, false, true>(jb, smem);
+  else
+    jb.zsum ? gen_tile<VEC, JUMP, true, false>(jb, smem) : gen_tile<VEC, JUMP, false, false>(jb, smem);
+}
+
+__global__ void __launch_bounds__(direct::kCtaThreads, kGenCtasPerSm)
+k_batch_gen(const unsigned char* __restrict__ wl) {
   extern __shared__ __align__(128) unsigned char smem[];
   const BatchHdr* hdr = reinterpret_cast<const BatchHdr*>(wl);
-  const GenRing<uint16_t> ring{smem, Pg};
-  gen_ring_init<uint16_t>(ring);
-  const int warp = threadIdx.x >> 5;
-  const int lane = threadIdx.x & 31;
-  int g = 0;
-  bool ok = true;
-  int l = (int)blockIdx.x - (int)gridDim.x;
-  int u = 0, uend = 0;
-#pragma unroll 1
-  while (ok) {
-    if (u >= uend) {
-      const int* lists = reinterpret_cast<const int*>(wl + hdr->off_glists);
-      do {
-        l += gridDim.x;
-        if (l >= hdr->n_glists) break;
-        u = lists[l];
-        uend = lists[l + 1];
-      } while (u >= uend);
-      if (u >= uend) break;
-    }
-    const WorkUnit un = reinterpret_cast<const WorkUnit*>(wl + hdr->off_gunits)[u++];
-    const BatchItemDev* it = reinterpret_cast<const BatchItemDev*>(wl + kOffItems) + un.item;
-    GenJob jb;
-    jb.tmap = &it->tmap;
-    jb.A = it->A;
-    jb.B = it->B;
-    jb.linear = it->linear;
-    jb.ny = it->ny;
-    jb.nz = it->nz;
-    jb.nx = it->nx;
-    jb.P = it->P;
-    jb.j0 = un.jt * kTileJ;
-    jb.xbase = un.xt * kX;
-    jb.ks = un.ks;
-    jb.ke = un.ke;
-    jb.zmip = it->zmip;
-    jb.zsum = it->zsum;
-    jb.ymip = it->ymip;
-    jb.argz = it->argz;
-    if (warp == 0) {
-      if (lane == 0)
-        asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(jb.tmap) : "memory");
-      __syncwarp();
-      ok = gen_produce<uint16_t>(jb, ring, g, err, lane);
-    } else {
-      ok = gen_consume<uint16_t>(jb, ring, g, err, warp - 1, lane);
+  const int* lists = reinterpret_cast<const int*>(wl + hdr->off_glists);
+  for (int l = blockIdx.x; l < hdr->n_glists; l += gridDim.x) {
+    for (int u = lists[l]; u < lists[l + 1]; ++u) {
+      const WorkUnit un = reinterpret_cast<const WorkUnit*>(wl + hdr->off_gunits)[u];
+      const BatchItemDev* it = reinterpret_cast<const BatchItemDev*>(wl + kOffItems) + un.item;
+      direct::Job jb;
+      jb.raw = it->raw;
+      jb.slots = it->slots;
+      jb.row_pitch = (size_t)it->row_pitch;
+      jb.plane_pitch = (size_t)it->plane_pitch;
+      jb.A = it->A;
+      jb.B = it->B;
+      jb.linear = it->linear;
+      jb.nscan = it->nscan;
+      jb.ny = it->ny;
+      jb.nz = it->nz;
+      jb.nx = it->nx;
+      jb.wr = it->wr;
+      jb.band = it->band[un.jt / kTileJ];
+      jb.xb = un.xt * kX;
+      jb.zmip = it->zmip;
+      jb.zsum = it->zsum;
+      jb.ymip = it->ymip;
+      jb.argz = it->argz;
+      for (jb.jc = un.jt; jb.jc < min(un.jt + un.pad, jb.ny); jb.jc += direct::cta_cols(jb.wr)) {
+        if (jb.slots == direct::kJumpSlots)
+          it->vec ? gen_job<true, true>(jb, smem) : gen_job<false, true>(jb, smem);
+        else
+          it->vec ? gen_job<true, false>(jb, smem) : gen_job<false, false>(jb, smem);
+        __syncthreads();  // shared memory is read before the next job writes it
+      }
     }
   }
-  if (warp == 0) gen_drain<uint16_t>(ring, g, ok, err, lane);
 }
 
 // Shared memory of a batch launch for slab depth Pl (family 0: k_batch_fast).
 size_t batch_smem(int Pl, int family) { return family ? per::total(kPerStages, Pl) : fast::total(Pl); }
-size_t batch_gen_smem(int Pg) { return gen::total<uint16_t>(Pg); }
+size_t batch_gen_smem() { return direct::smem_bytes<uint16_t>(direct::kJumpSlots); }
 
 PFN_cuTensorMapEncodeTiled_v12000 batch_encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -310,7 +317,7 @@ struct WorkList {
   int n_items, n_units, n_segs, n_lists, Pl;
   int family;   // kFamilies index + 1 of the periodic kernel, or 0 (fast kernel)
   int n_gunits; // units of the general kernel
-  int Pg;       // its slab depth (deepest general item)
+  int Pg;       // planes of its deepest item's tile rows
   int run;      // columns j per compute warp of the periodic kernel (32 or 16)
   int shape;    // opm_shape the list was built for (never AUTO)
 };
@@ -372,6 +379,7 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
   int* hglists = reinterpret_cast<int*>(stage + off_glists);
   WorkUnit* hunits = reinterpret_cast<WorkUnit*>(stage + off_units);
   int64_t nunits = 0;
+  bool fine = false;  // room for every general item's single pieces
   int Pl = 2, Pg = 2, nseg = 0, family = -1, nfast = 0;
   // first pass: fast items' units; second pass: general items' units after them
   for (int pass = 0; pass < 2; ++pass) {
@@ -408,6 +416,14 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
         d.fnlo = p->view.fnlo;
         d.A = p->view.A;
         d.B = p->view.B;
+        d.band = p->view.band;
+        d.raw = it.raw;
+        d.row_pitch = rp;
+        d.plane_pitch = pp;
+        d.nscan = (int)p->nscan;
+        d.wr = (short)direct::row_groups(p->ny, p->nx);
+        d.slots = (short)direct::row_slots(!p->unit_steps, p->rho);
+        d.vec = direct::vec_rows<uint16_t>(it.raw, p->nx, rp, pp) && !p->force_generic;
         d.linear = p->view.linear;
         d.zmip = it.zmip;
         d.ymip = it.ymip;
@@ -432,24 +448,44 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
       if (it.ymip) hsegs[nseg++] = BatchSeg{it.ymip, (long long)(p->nz * p->nx)};
       const int xtiles = (int)((p->nx + kX - 1) / kX);
       const int jtiles = (int)((p->ny + kTileJ - 1) / kTileJ);
+      const int piece = fine ? direct::cta_cols(hitems[i].wr) : kTileJ;
       for (int jt = 0; jt < jtiles; ++jt) {
         const Band bd = p->hBand[jt];
-        const int step = fast ? kchunk : std::max(1, bd.hi - bd.lo);
-        const int cstart = fast ? (bd.lo / kchunk) * kchunk : bd.lo;
+        const int step = kchunk, cstart = (bd.lo / kchunk) * kchunk;
         const bool empty_unit = !fast && zout && bd.lo >= bd.hi;
-        for (int c0 = cstart; c0 < bd.hi || (empty_unit && c0 == cstart); c0 += step) {
+        if (!fast) {
+          if (bd.lo >= bd.hi && !empty_unit) continue;
+          for (int jc = jt * kTileJ; jc < std::min<int64_t>((jt + 1) * kTileJ, p->ny); jc += piece) {
+            if (nunits + xtiles > max_units)
+              return fail(OPM_ERR_UNSUPPORTED, std::string("the items need more than the ") + limit_what +
+                                                   "'s limit of " + std::to_string(max_units) + " work units (split)");
+            for (int xt = 0; xt < xtiles; ++xt)
+              hunits[nunits++] = WorkUnit{i, xt, jc, bd.lo, std::max(bd.lo, bd.hi), 0, 0, piece};
+          }
+          continue;
+        }
+        for (int c0 = cstart; c0 < bd.hi; c0 += step) {
           const int ks = std::max(bd.lo, c0), ke = std::min(bd.hi, c0 + step);
-          if (ks >= ke && !empty_unit) continue;
+          if (ks >= ke) continue;
           if (nunits + xtiles > max_units)
             return fail(OPM_ERR_UNSUPPORTED, std::string("the items need more than the ") + limit_what +
                                                  "'s limit of " + std::to_string(max_units) +
                                                  " work units (raise kchunk or split)");
           for (int xt = 0; xt < xtiles; ++xt)
-            hunits[nunits++] = WorkUnit{i, xt, jt, ks, std::max(ks, ke), 0, 0, 0};
+            hunits[nunits++] = WorkUnit{i, xt, jt, ks, ke, 0, 0, 0};
         }
       }
     }
-    if (pass == 0) nfast = (int)nunits;
+    if (pass == 0) {
+      nfast = (int)nunits;
+      int64_t pieces = 0;
+      for (int i = 0; i < n_items; ++i) {
+        const opm_plan* p = items[i].plan;
+        const int cols = direct::cta_cols(hitems[i].wr);
+        pieces += (p->ny + cols - 1) / cols * ((p->nx + kX - 1) / kX);
+      }
+      fine = nunits + pieces <= max_units;
+    }
   }
   const int ngen = (int)nunits - nfast;
   // balanced lists of units, one per persistent CTA, for each kernel
@@ -531,7 +567,7 @@ cudaError_t launch_worklist(const unsigned char* dev_wl, const WorkList& wl, int
     if (e != cudaSuccess) return e;
   }
   if (ggrid > 0) {
-    k_batch_gen<<<ggrid, kThreads, batch_gen_smem(wl.Pg), s>>>(dev_wl, wl.Pg, err);
+    k_batch_gen<<<ggrid, direct::kCtaThreads, batch_gen_smem(), s>>>(dev_wl);
     e = cudaGetLastError();
   }
   return e;
@@ -551,8 +587,8 @@ void batch_grids(const WorkList& wl, int nsm, int ctas_per_sm, bool all, int* gr
 opm_status batch_check_smem(const WorkList& wl, int smem_optin) {
   if (wl.n_units > 0 && (int)batch_smem(wl.Pl, wl.family) > smem_optin)
     return fail(OPM_ERR_UNSUPPORTED, "batch slab depth needs too much shared memory");
-  if (wl.n_gunits > 0 && (int)batch_gen_smem(wl.Pg) > smem_optin)
-    return fail(OPM_ERR_UNSUPPORTED, "general items' slab depth needs too much shared memory");
+  if (wl.n_gunits > 0 && wl.Pg > kGenMaxPlanes)
+    return fail(OPM_ERR_UNSUPPORTED, "general items span too many planes per tile row");
   return OPM_OK;
 }
 
@@ -604,10 +640,10 @@ struct opm_batch {
   int attr_set;
   cudaStream_t capture;  // private stream the graphs are captured on
   // Captured launches (zero kernel + persistent kernels), one per launch
-  // shape: kernel shape, periodic family and run, slab depths and grids.
+  // shape: kernel shape, periodic family and run, slab depth and grids.
   struct Graph {
     cudaGraphExec_t exec;
-    int key[7];
+    int key[6];
     unsigned long long used;  // launch counter at the last use
   } graphs[kGraphCache];
   unsigned long long launches;
@@ -730,11 +766,11 @@ opm_status opm_batch_launch_graph(opm_batch* b, int ctas_per_sm, void* stream) {
   // full grids: every CTA reads the unit counts from the device header
   int grid = 0, ggrid = 0;
   batch_grids(b->wl, b->nsm, ctas_per_sm, true, &grid, &ggrid);
-  const int key[7] = {grid ? b->wl.shape : 0, grid ? b->wl.family : 0, grid ? b->wl.run : 0,
-                      grid ? b->wl.Pl : 0,    grid,                     ggrid ? b->wl.Pg : 0, ggrid};
+  const int key[6] = {grid ? b->wl.shape : 0, grid ? b->wl.family : 0, grid ? b->wl.run : 0,
+                      grid ? b->wl.Pl : 0,    grid,                     ggrid};
   opm_batch::Graph* hit = nullptr;
   for (auto& gr : b->graphs)
-    if (gr.exec && std::equal(key, key + 7, gr.key)) hit = &gr;
+    if (gr.exec && std::equal(key, key + 6, gr.key)) hit = &gr;
   b->launches += 1;
   if (!hit) {
     // an empty slot, else the least recently used one
@@ -758,7 +794,7 @@ opm_status opm_batch_launch_graph(opm_batch* b, int ctas_per_sm, void* stream) {
       hit->exec = nullptr;
       return cuda_fail(e, "capturing the batch launch");
     }
-    std::copy(key, key + 7, hit->key);
+    std::copy(key, key + 6, hit->key);
     b->graph_captures += 1;
   }
   hit->used = b->launches;
@@ -774,7 +810,7 @@ opm_status opm_batch_info(const opm_batch* b, int* n_items, int64_t* n_units, in
   if (n_units) *n_units = (int64_t)b->wl.n_units + b->wl.n_gunits;
   if (smem_bytes)
     *smem_bytes = (int)std::max(b->wl.n_units ? batch_smem(b->wl.Pl, b->wl.family) : 0,
-                                b->wl.n_gunits ? batch_gen_smem(b->wl.Pg) : 0);
+                                b->wl.n_gunits ? batch_gen_smem() : 0);
   if (graph_captures) *graph_captures = b->graph_captures;
   return OPM_OK;
 }

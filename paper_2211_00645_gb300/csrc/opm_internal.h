@@ -108,6 +108,7 @@ struct opm_plan {
   int force_generic;  // use the plain (non-TMA) kernels for every call
   int P;              // planes staged per row for a 32-column tile
   int fast_ok;        // full tiles never step more than one plane per column
+  int unit_steps = 0; // inside every 8-column group (from 0), a column lies on its left neighbour's plane or the next
   int family = 0;     // 1 + index into kFamilies when the periodic kernel applies, else 0
   int lists_per_sm = 4;  // persistent CTA lists per SM of the live-view schedule
   int chunk_rows = 0;    // rows per work unit of that schedule (0: no schedule)

@@ -177,6 +177,16 @@ opm_status opm_plan_create(int64_t nscan, int64_t nrows, int64_t ncols,
         }
       }
     }
+    // The direct kernel's like assumption over 8-column groups, the last tile
+    // unshifted: the full tiles have just been checked when fast_ok held.
+    p->unit_steps = p->rho <= 1.0;
+    const int64_t checked = p->fast_ok ? ny / kTileJ * kTileJ : 0;
+    for (int64_t k = 0; p->unit_steps && k < nrows; ++k)
+      for (int64_t j = checked + 1; j < ny; ++j) {
+        if (j % 8 == 0) continue;
+        const int up = host_n0(p->hA[j], p->hB[k]) - host_n0(p->hA[j - 1], p->hB[k]);
+        if (up != 0 && up != 1) p->unit_steps = 0;
+      }
     // The fast kernel's per-(tile, row) tables, from the same formula.
     if (p->fast_ok) {
       p->hFrow.resize((size_t)ntile * nrows);

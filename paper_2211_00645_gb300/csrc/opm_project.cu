@@ -37,10 +37,10 @@
 //                  stacks) whose z-maxima combine by atomic max, which
 //                  balances tiles of very different band length; a
 //                  persistent grid of 4 CTAs per SM walks the chunks.
-//  k_project_gen   every output (z-sum, first argmax), uint16 or FP32 input,
-//                  any tile (partial last tile, column steps of several
-//                  planes), one row per stage, whole band per CTA
-//                  (opm_gen.cuh, shared with the batched general kernel).
+//  k_project_direct  every other call: z-sum, first arg-max, FP32 input, rows
+//                  that are not a multiple of 16 bytes, any geometry
+//                  (opm_direct.cuh, shared with the batch).  It reads global
+//                  memory directly, without the ring described above.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -48,7 +48,7 @@
 #include <cstring>
 #include <mutex>
 
-#include "opm_gen.cuh"
+#include "opm_direct.cuh"
 #include "opm_periodic.cuh"
 
 namespace opm {
@@ -58,11 +58,8 @@ namespace {
 struct ProjArgs {
   PlanView v;
   float* zmip;
-  float* zsum;
   float* ymip;
-  int32_t* argz;
   int P;       // staged planes per row
-  int jt0;     // first j-tile of this launch
 };
 
 // Fast kernel, persistent: one CTA per list of the plan's balanced schedule
@@ -163,99 +160,33 @@ k_project_per(const __grid_constant__ CUtensorMap tmap, const ProjArgs args) {
   if (warp == 0) per_drain(ring, g, ok, v.err);
 }
 
-// =====================================================================
-// General kernel (opm_gen.cuh): every output, uint16 or FP32, any tile, one
-// row per stage, one job (a tile's whole row band) per CTA on a grid of
-// (x-tile, j-tile).
-template <typename T>
-__global__ void __launch_bounds__(kThreads, 1)
-k_project_gen(const __grid_constant__ CUtensorMap tmap, const ProjArgs args) {
-  const PlanView& v = args.v;
+// Direct kernel (opm_direct.cuh): one job per CTA, x-tiles fastest.
+template <typename T, bool VEC, bool SUM, bool ARG, bool JUMP>
+__global__ void __launch_bounds__(direct::kCtaThreads, ARG && SUM ? 1 : 2)
+k_project_direct(const PlanView v, const T* __restrict__ raw, int wr, int slots, int xtiles, float* zmip, float* zsum,
+                 float* ymip, int32_t* argz) {
   extern __shared__ __align__(128) unsigned char smem[];
-  const GenRing<T> ring{smem, args.P};
-  gen_ring_init<T>(ring);
-  const int jt = blockIdx.y + args.jt0;
-  const Band band = v.band[jt];
-  GenJob jb;
-  jb.tmap = &tmap;
+  direct::Job jb;
+  jb.raw = raw;
+  jb.slots = slots;
+  jb.row_pitch = v.ncols;
+  jb.plane_pitch = (size_t)v.nrows * v.ncols;
   jb.A = v.A;
   jb.B = v.B;
   jb.linear = v.linear;
+  jb.nscan = v.nscan;
   jb.ny = v.ny;
   jb.nz = v.nz;
   jb.nx = v.nx;
-  jb.P = args.P;
-  jb.j0 = jt * kTileJ;
-  jb.xbase = blockIdx.x * kX;
-  jb.ks = band.lo;
-  jb.ke = band.hi;
-  jb.zmip = args.zmip;
-  jb.zsum = args.zsum;
-  jb.ymip = args.ymip;
-  jb.argz = args.argz;
-  const int warp = threadIdx.x >> 5;
-  const int lane = threadIdx.x & 31;
-  int g = 0;
-  if (warp == 0) {
-    const bool ok = gen_produce<T>(jb, ring, g, v.err, lane);
-    gen_drain<T>(ring, g, ok, v.err, lane);
-  } else {
-    (void)gen_consume<T>(jb, ring, g, v.err, warp - 1, lane);
-  }
-}
-
-// =====================================================================
-// Plain kernels for shapes the TMA path does not take (unaligned rows,
-// very coarse scan steps).  One thread per output pixel, every row visited.
-template <typename T>
-__global__ void k_zproj_plain(PlanView v, const T* __restrict__ raw, float* zmip, float* zsum,
-                              int32_t* argz) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long long)v.ny * v.nx) return;
-  const int j = (int)(idx / v.nx);
-  const int x = (int)(idx - (long long)j * v.nx);
-  const Split a = v.A[j];
-  const size_t plane = (size_t)v.nrows * v.ncols;
-  float zm = -INFINITY, zs = 0.0f;
-  int az = 0;
-  for (int k = 0; k < v.nz; ++k) {
-    int n0;
-    float w;
-    plane_weight(a, v.B[k], v.linear, n0, w);
-    const T* rp = raw + (size_t)k * v.ncols + x;
-    const float lo = (n0 >= 0 && n0 < v.nscan) ? to_f32(rp[(size_t)n0 * plane]) : 0.0f;
-    const float hi = (n0 + 1 >= 0 && n0 + 1 < v.nscan) ? to_f32(rp[(size_t)(n0 + 1) * plane]) : 0.0f;
-    const float val = fmaf(w, hi - lo, lo);
-    if (val > zm) {
-      zm = val;
-      az = k;
-    }
-    zs += val;
-  }
-  if (zmip) zmip[idx] = zm;
-  if (zsum) zsum[idx] = zs;
-  if (argz) argz[idx] = az;
-}
-
-template <typename T>
-__global__ void k_yproj_plain(PlanView v, const T* __restrict__ raw, float* ymip) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long long)v.nz * v.nx) return;
-  const int k = (int)(idx / v.nx);
-  const int x = (int)(idx - (long long)k * v.nx);
-  const Split b = v.B[k];
-  const size_t plane = (size_t)v.nrows * v.ncols;
-  const T* rp = raw + (size_t)k * v.ncols + x;
-  float ym = -INFINITY;
-  for (int j = 0; j < v.ny; ++j) {
-    int n0;
-    float w;
-    plane_weight(v.A[j], b, v.linear, n0, w);
-    const float lo = (n0 >= 0 && n0 < v.nscan) ? to_f32(rp[(size_t)n0 * plane]) : 0.0f;
-    const float hi = (n0 + 1 >= 0 && n0 + 1 < v.nscan) ? to_f32(rp[(size_t)(n0 + 1) * plane]) : 0.0f;
-    ym = fmaxf(ym, fmaf(w, hi - lo, lo));
-  }
-  ymip[idx] = ym;
+  jb.wr = wr;
+  jb.jc = (int)(blockIdx.x / xtiles) * direct::cta_cols(wr);
+  jb.xb = (int)(blockIdx.x % xtiles) * direct::kXW;
+  jb.band = v.band[jb.jc / kTileJ];
+  jb.zmip = zmip;
+  jb.zsum = zsum;
+  jb.ymip = ymip;
+  jb.argz = argz;
+  direct::tile<T, VEC, SUM, ARG, JUMP>(jb, smem);
 }
 
 // Initial values of the atomically combined outputs: the fast kernel folds
@@ -300,16 +231,13 @@ int max_optin_smem(int dev) {
   return cache[dev];
 }
 
-template <typename T>
 opm_status encode_raw(const PlanView& v, const void* raw, int P, CUtensorMap* map) {
   std::memset(map, 0, sizeof(*map));
   const cuuint64_t dims[3] = {(cuuint64_t)v.ncols, (cuuint64_t)v.nrows, (cuuint64_t)v.nscan};
-  const cuuint64_t strides[2] = {(cuuint64_t)v.ncols * sizeof(T), (cuuint64_t)v.nrows * v.ncols * sizeof(T)};
+  const cuuint64_t strides[2] = {(cuuint64_t)v.ncols * 2, (cuuint64_t)v.nrows * v.ncols * 2};
   const cuuint32_t box[3] = {(cuuint32_t)kX, 1u, (cuuint32_t)P};
   const cuuint32_t estr[3] = {1u, 1u, 1u};
-  const CUtensorMapDataType dt =
-      std::is_same<T, uint16_t>::value ? CU_TENSOR_MAP_DATA_TYPE_UINT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
-  CUresult cr = encode_fn()(map, dt, 3, const_cast<void*>(raw), dims, strides, box, estr,
+  CUresult cr = encode_fn()(map, CU_TENSOR_MAP_DATA_TYPE_UINT16, 3, const_cast<void*>(raw), dims, strides, box, estr,
                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (cr != CUDA_SUCCESS)
@@ -358,8 +286,8 @@ opm_status launch_per(const opm_plan* p, const CUtensorMap& map, const ProjArgs&
   return launch_per_f<0>(p, map, args, s, grid_div);
 }
 
-opm_status launch_fast(const opm_plan* p, const CUtensorMap& map, const ProjArgs& args, int tiles,
-                       cudaStream_t s, int grid_div) {
+opm_status launch_fast(const opm_plan* p, const CUtensorMap& map, const ProjArgs& args, cudaStream_t s,
+                       int grid_div) {
   static int done[64] = {0};
   if (p->family) return launch_per(p, map, args, s, grid_div);
   opm_status st = prepare_kernel(k_project_fast, p->device, done);
@@ -374,19 +302,39 @@ opm_status launch_fast(const opm_plan* p, const CUtensorMap& map, const ProjArgs
   return e == cudaSuccess ? OPM_OK : cuda_fail(e, "launch k_project_fast");
 }
 
-template <typename T>
-opm_status launch_gen(const opm_plan* p, const CUtensorMap& map, const ProjArgs& args, int tiles,
-                      cudaStream_t s) {
-  static int done[64] = {0};
-  opm_status st = prepare_kernel(k_project_gen<T>, p->device, done);
-  if (st != OPM_OK) return st;
+template <typename T, bool VEC, bool SUM, bool ARG>
+opm_status launch_direct_as(const opm_plan* p, const void* raw, float* zmip, float* zsum, float* ymip, int32_t* argz,
+                            cudaStream_t s) {
   const PlanView& v = p->view;
-  const int xtiles = (v.nx + kX - 1) / kX;
-  if (tiles > 65535) return fail(OPM_ERR_UNSUPPORTED, "projection grid exceeds launch limits");
-  dim3 grid(xtiles, tiles, 1);
-  k_project_gen<T><<<grid, kThreads, gen::total<T>(args.P), s>>>(map, args);
+  const int wr = direct::row_groups(v.ny, v.nx), cols = direct::cta_cols(wr);
+  const long long xtiles = (v.nx + direct::kXW - 1) / direct::kXW;
+  const long long nb = xtiles * ((v.ny + cols - 1) / cols);
+  if (nb > 0x7fffffffLL) return fail(OPM_ERR_UNSUPPORTED, "grid too large");
+  const bool jump = !p->unit_steps;
+  static int done[2][64] = {{0}};
+  const auto kern = jump ? k_project_direct<T, VEC, SUM, ARG, true> : k_project_direct<T, VEC, SUM, ARG, false>;
+  opm_status st = prepare_kernel(kern, p->device, done[jump]);
+  if (st != OPM_OK) return st;
+  const int slots = direct::row_slots(jump, p->rho);
+  kern<<<(unsigned)nb, direct::kCtaThreads, direct::smem_bytes<T>(slots), s>>>(
+      v, static_cast<const T*>(raw), wr, slots, (int)xtiles, zmip, zsum, ymip, argz);
   cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? OPM_OK : cuda_fail(e, "launch k_project_gen");
+  return e == cudaSuccess ? OPM_OK : cuda_fail(e, "launch k_project_direct");
+}
+
+template <typename T>
+opm_status launch_direct(const opm_plan* p, const void* raw, float* zmip, float* zsum, float* ymip, int32_t* argz,
+                         cudaStream_t s) {
+  const PlanView& v = p->view;
+  const bool vec = direct::vec_rows<T>(raw, v.nx, v.ncols, (int64_t)v.nrows * v.ncols) && !p->force_generic;
+  const auto go = [&](auto vc, auto sm, auto ar) {
+    return launch_direct_as<T, decltype(vc)::value, decltype(sm)::value, decltype(ar)::value>(p, raw, zmip, zsum, ymip,
+                                                                                             argz, s);
+  };
+  const std::true_type yes;
+  const std::false_type no;
+  if (vec) return argz ? (zsum ? go(yes, yes, yes) : go(yes, no, yes)) : (zsum ? go(yes, yes, no) : go(yes, no, no));
+  return argz ? (zsum ? go(no, yes, yes) : go(no, no, yes)) : (zsum ? go(no, yes, no) : go(no, no, no));
 }
 
 }  // namespace
@@ -395,40 +343,12 @@ opm_status launch_project(const opm_plan* p, const void* raw, opm_dtype in_t, fl
                           float* ymip, int32_t* argz, cudaStream_t s, int grid_div) {
   const PlanView& v = p->view;
   const bool u16 = in_t == OPM_U16;
-  const size_t es = u16 ? 2 : 4;
   const int P = p->P;
   const int smax = max_optin_smem(p->device);
-  const bool tma_ok = !p->force_generic && encode_fn() != nullptr && ((uintptr_t)raw % 16 == 0) &&
-                      ((size_t)v.ncols * es) % 16 == 0 && P <= 256;
-  const bool gen_ok = tma_ok && (int)(u16 ? gen::total<uint16_t>(P) : gen::total<float>(P)) <= smax;
-  const bool fast = gen_ok && u16 && !zsum && !argz && p->fast_ok && v.frow &&
+  // the TMA kernels: uint16 rows on 16 bytes, z-MIP and / or y-MIP only
+  const bool fast = u16 && !zsum && !argz && p->fast_ok && v.frow && !p->force_generic && encode_fn() != nullptr &&
+                    (uintptr_t)raw % 16 == 0 && (size_t)v.ncols * 2 % 16 == 0 &&
                     (int)(p->family ? per::total(kPerStages, P) : fast::total(P)) <= smax;
-
-  if (!gen_ok) {
-    const long long nzx = (long long)v.ny * v.nx, nyx = (long long)v.nz * v.nx;
-    const int tb = 256;
-    if (zmip || zsum || argz) {
-      const long long nb = (nzx + tb - 1) / tb;
-      if (nb > 0x7fffffffLL) return fail(OPM_ERR_UNSUPPORTED, "grid too large");
-      if (u16)
-        k_zproj_plain<uint16_t><<<(unsigned)nb, tb, 0, s>>>(v, static_cast<const uint16_t*>(raw), zmip, zsum, argz);
-      else
-        k_zproj_plain<float><<<(unsigned)nb, tb, 0, s>>>(v, static_cast<const float*>(raw), zmip, zsum, argz);
-      cudaError_t e = cudaGetLastError();
-      if (e != cudaSuccess) return cuda_fail(e, "launch k_zproj_plain");
-    }
-    if (ymip) {
-      const long long nb = (nyx + tb - 1) / tb;
-      if (nb > 0x7fffffffLL) return fail(OPM_ERR_UNSUPPORTED, "grid too large");
-      if (u16)
-        k_yproj_plain<uint16_t><<<(unsigned)nb, tb, 0, s>>>(v, static_cast<const uint16_t*>(raw), ymip);
-      else
-        k_yproj_plain<float><<<(unsigned)nb, tb, 0, s>>>(v, static_cast<const float*>(raw), ymip);
-      cudaError_t e = cudaGetLastError();
-      if (e != cudaSuccess) return cuda_fail(e, "launch k_yproj_plain");
-    }
-    return OPM_OK;
-  }
 
   // initial values of the atomically combined outputs
   float* zinit = fast ? zmip : nullptr;
@@ -441,20 +361,18 @@ opm_status launch_project(const opm_plan* p, const void* raw, opm_dtype in_t, fl
     if (e != cudaSuccess) return cuda_fail(e, "launch k_init_outputs");
   }
 
+  if (!fast)
+    return u16 ? launch_direct<uint16_t>(p, raw, zmip, zsum, ymip, argz, s)
+               : launch_direct<float>(p, raw, zmip, zsum, ymip, argz, s);
+
   ProjArgs args;
   args.v = v;
   args.zmip = zmip;
-  args.zsum = zsum;
   args.ymip = ymip;
-  args.argz = argz;
   args.P = P;
-  args.jt0 = 0;
   CUtensorMap map;
-  opm_status st = u16 ? encode_raw<uint16_t>(v, raw, P, &map) : encode_raw<float>(v, raw, P, &map);
-  if (st != OPM_OK) return st;
-  const int jtiles = (v.ny + kTileJ - 1) / kTileJ;
-  if (fast) return launch_fast(p, map, args, jtiles, s, grid_div);
-  return u16 ? launch_gen<uint16_t>(p, map, args, jtiles, s) : launch_gen<float>(p, map, args, jtiles, s);
+  opm_status st = encode_raw(v, raw, P, &map);
+  return st == OPM_OK ? launch_fast(p, map, args, s, grid_div) : st;
 }
 
 }  // namespace opm

@@ -12,7 +12,8 @@
 namespace opm {
 
 // Rows [ks, ke) of j-tile jt at x-tile xt of item `item` (0 for a single
-// stack).  `list` and `seq` are scheduling scratch.
+// stack).  `list` and `seq` are scheduling scratch.  (The batch's general
+// units: `pad` columns from column jt.)
 struct __align__(16) WorkUnit {
   int item, xt, jt, ks, ke;
   int list, seq, pad;

@@ -18,7 +18,6 @@ constexpr int kThreads = 32 * (kNW + 1);
 constexpr int kVec = 4;              // columns x per lane
 constexpr int kX = 32 * kVec;        // columns x per CTA
 constexpr int kStagesFast = 6;       // TMA ring depth, fast kernel
-constexpr int kStagesGen = 4;        // TMA ring depth, general kernel
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s: a launch takes < 10 ms
 
 static_assert(kJT * kNW == kTileJ, "tile");
@@ -149,54 +148,6 @@ __device__ __forceinline__ void atomic_max_f(float* addr, float v) {
 __device__ __forceinline__ int yidx(int xl) {
   const int L = xl >> 2;
   return (L << 2) + ((xl & 3) ^ ((L >> 3) & 3));
-}
-
-// 4 raw values of one staged row (this lane's 4 columns) as two FP32 pairs.
-template <typename T>
-__device__ __forceinline__ void lds_row(const unsigned char* p, f2 (&out)[2]) {
-  if constexpr (std::is_same<T, uint16_t>::value) {
-    const uint2 u = *reinterpret_cast<const uint2*>(p);
-    out[0] = u16x2_to_f2(u.x);
-    out[1] = u16x2_to_f2(u.y);
-  } else {
-    const float4 f = *reinterpret_cast<const float4*>(p);
-    out[0] = pk(f.x, f.y);
-    out[1] = pk(f.z, f.w);
-  }
-}
-
-// One staged row's streaming state for a compute lane: the lower plane a
-// and the difference d = b - a at slab offset o.
-struct Stream {
-  f2 a[2];
-  f2 d[2];
-  int o;
-};
-
-template <typename T>
-__device__ __forceinline__ void stream_reset(Stream& st, const unsigned char* lane_slab, int pitch, int o) {
-  f2 b[2];
-  st.o = o;
-  lds_row<T>(lane_slab + o * pitch, st.a);
-  lds_row<T>(lane_slab + (o + 1) * pitch, b);
-  st.d[0] = sub2(b[0], st.a[0]);
-  st.d[1] = sub2(b[1], st.a[1]);
-}
-
-template <typename T>
-__device__ __forceinline__ void stream_step(Stream& st, const unsigned char* lane_slab, int pitch) {
-  f2 b[2];
-  st.o += 1;
-  lds_row<T>(lane_slab + (st.o + 1) * pitch, b);
-  if constexpr (std::is_same<T, uint16_t>::value) {
-    // integers below 2^24: a + (b - a) == b exactly
-    st.a[0] = add2(st.a[0], st.d[0]);
-    st.a[1] = add2(st.a[1], st.d[1]);
-  } else {
-    lds_row<T>(lane_slab + st.o * pitch, st.a);
-  }
-  st.d[0] = sub2(b[0], st.a[0]);
-  st.d[1] = sub2(b[1], st.a[1]);
 }
 
 // Streaming on 32-bit shared-memory offsets for the fast kernel (uint16
