@@ -249,8 +249,7 @@ opm_status opm_warp_rows(const float* in, int64_t in_rows, int64_t ncols, float*
  * order) the z-MIP and y-MIP equal opm_project's on the whole stack bit for
  * bit; the z-sum equals it up to FP32 summation order.  Calls that update
  * the same outputs must be ordered on one stream.  Asynchronous; allocates
- * nothing.  A column search that runs past its bound records an error bit
- * (see opm_plan_check).
+ * nothing.
  * Errors: OPM_ERR_INVALID_ARG (NULL plan, no output, n out of range, plane
  * pointers not matching n), OPM_ERR_UNSUPPORTED (more than 65535 rows),
  * OPM_ERR_CUDA.
@@ -284,9 +283,8 @@ opm_status opm_max_combine(float* out, const float* a, const float* b, int64_t n
  *   view  [P]         the published projections.
  * All three must be zero before the first push and are owned by the caller.
  * After the call, view equals opm_project of the stack buffer bit for bit
- * (z-MIP and y-MIP).  A call costs two opm_stream_pair passes, one zeroing
- * and two maxima over P; the call for m = nscan - 1 also builds the next
- * suffixes (nscan - 2 maxima).  Asynchronous; allocates nothing.
+ * (z-MIP and y-MIP).  A call is one kernel over P; the call for m = nscan - 1
+ * also builds the next suffixes (one pass over the slots).  Asynchronous; allocates nothing.
  * Errors: OPM_ERR_INVALID_ARG (NULL, m out of range), OPM_ERR_UNSUPPORTED
  * (more than 65535 rows), OPM_ERR_CUDA.
  */

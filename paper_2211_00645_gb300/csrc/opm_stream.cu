@@ -6,19 +6,39 @@
 // plane, so the calls for n = -1 .. nscan - 1 cover the volume once; the
 // per-voxel arithmetic (plane, weight, FMA on the plane difference) is the
 // fast projection's, so the z-MIP and y-MIP end bit-identical to it.
+//
+// Both projections are gathered.  The lower plane falls along k and grows
+// along j, so the rows of one column j that belong to pair n are one run
+// (1 / (rho cos theta) rows, 3.7 on the live-view geometry), and so are the
+// columns of one row k (1 / rho); each output value is written by one thread,
+// once, with no atomics and nothing zeroed beforehand.  A warp takes one
+// column j (or row k) x 128 columns x and finds its run with a 32-way search
+// of the split table; the 8 warps of a CTA take neighbours, whose runs share
+// camera rows.  Consecutive pairs' runs adjoin, so the sliding view folds its
+// complete pair and its mixed pair in one walk, together with the maxima it
+// combines them with.
+//
+// What bounds it: L2 traffic (a push reads the run and one slot and writes a
+// slot and the view, 45 MB at 200 planes) and the search's latency.  Device
+// time back to back, 512 x 2048 frames, 35 deg, step 0.3, pixel 0.1, before
+// (a scatter of shared and global atomic maxima; a push was two of them, one
+// zeroing and two elementwise maxima) -> now: one pair 9.8 -> 9.2 us, with a
+// z-sum 14.9 -> 10.2; a push on 200 planes 30.3 -> 17.7, the last one with the
+// next suffixes 1240 -> 773 (5 GB of slots read and written, 6.5 TB/s); 87 x
+// 1304 frames of 50 planes: pair 5.0 -> 3.4, push 16.9 -> 5.7, last 135 -> 33.
+// Four rows' loads ahead cost occupancy and were slower (18.9 a push).
 #include <algorithm>
 
-#include "opm_common.cuh"
+#include "opm_tma.cuh"
 
 namespace opm {
 
 namespace {
 
-constexpr int kSVec = 4;         // columns x per thread
-constexpr int kSLanesX = 32;     // threads along x (one warp): 128 columns per CTA
-constexpr int kSRowsCta = 8;     // camera rows per CTA, one warp each
-constexpr int kSTileJ = 32;      // columns j of the CTA's shared z-MIP tile
-constexpr int kSearchSteps = 64; // bound on the column search of one row
+constexpr int kSXL = 4;            // columns x per lane
+constexpr int kSXW = 32 * kSXL;    // columns x per warp
+constexpr int kSWarps = 8;         // neighbouring columns j (rows k) per CTA
+constexpr int kNoPair = -0x40000000;
 
 __global__ void k_stream_zero(float* zmip, float* zsum, long long nj, float* ymip, long long nk) {
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -30,124 +50,295 @@ __global__ void k_stream_zero(float* zmip, float* zsum, long long nj, float* ymi
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nk; i += stride) ymip[i] = 0.0f;
 }
 
-// Loads this thread's kSVec columns of camera row k of one plane (zeros for
-// a missing plane or columns past the edge).
-__device__ __forceinline__ void load_row(const uint16_t* __restrict__ plane, const PlanView& v, int k, int x0,
-                                         bool vec, float (&out)[kSVec]) {
+// Plane pair n (frames lo = n and hi = n + 1; a frame outside the stack is
+// NULL and reads as zero).
+struct Pair {
+  const uint16_t* lo;
+  const uint16_t* hi;
+  int n;  // kNoPair: none
+};
+
+// First index in [0, count) for which `reached` holds (it holds from there
+// on), count if none.  Whole warp.
+template <typename Pred>
+__device__ __forceinline__ int first_index(int count, int lane, const Pred& reached) {
+  int lo = 0, hi = count;  // the answer lies in [lo, hi]
+  while (lo < hi) {
+    const int st = (hi - lo + 31) >> 5;
+    const int i = lo + lane * st;
+    const unsigned b = __ballot_sync(0xffffffffu, i >= hi || reached(i));
+    if (b == 0) {
+      lo += 31 * st + 1;
+    } else {
+      const int f = __ffs(b) - 1;
+      if (f == 0) return lo;
+      hi = min(hi, lo + f * st);
+      lo += (f - 1) * st + 1;
+    }
+  }
+  return lo;
+}
+
+// This lane's kSXL counts of camera row k of one frame: neighbours (VEC) or
+// columns 32 apart; zeros for a missing frame.
+template <bool VEC>
+__device__ __forceinline__ void load_counts(const uint16_t* __restrict__ frame, size_t o, int lim, f2 (&out)[2]) {
+  uint32_t w0 = 0, w1 = 0;
+  if (frame) {
+    const uint16_t* p = frame + o;
+    if constexpr (VEC) {
+      const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+      w0 = u.x, w1 = u.y;
+    } else {
+      if (0 < lim) w0 = __ldg(p);
+      if (32 < lim) w0 |= (uint32_t)__ldg(p + 32) << 16;
+      if (64 < lim) w1 = __ldg(p + 64);
+      if (96 < lim) w1 |= (uint32_t)__ldg(p + 96) << 16;
+    }
+  }
+  out[0] = u16x2_to_f2(w0);
+  out[1] = u16x2_to_f2(w1);
+}
+
+// Maxima (and sums of A's voxels) over one column's or row's voxels in pairs A
+// and B.
+struct Fold {
+  float a[kSXL], b[kSXL], s[kSXL];
+  bool any;  // A or B has a voxel here
+};
+
+__device__ __forceinline__ void fold_voxel(float w, const f2 (&lo)[2], const f2 (&hi)[2], float (&m)[kSXL],
+                                           float (&v)[kSXL]) {
+  const f2 w2 = pk(w, w);
 #pragma unroll
-  for (int i = 0; i < kSVec; ++i) out[i] = 0.0f;
-  if (!plane) return;
-  const uint16_t* p = plane + (size_t)k * v.ncols + x0;
-  if (vec) {
-    const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
-    out[0] = (float)(u.x & 0xFFFFu);
-    out[1] = (float)(u.x >> 16);
-    out[2] = (float)(u.y & 0xFFFFu);
-    out[3] = (float)(u.y >> 16);
-  } else {
-#pragma unroll
-    for (int i = 0; i < kSVec; ++i)
-      if (x0 + i < v.nx) out[i] = (float)__ldg(p + i);
+  for (int h = 0; h < 2; ++h) {
+    upk(fma2(w2, sub2(hi[h], lo[h]), lo[h]), v[2 * h], v[2 * h + 1]);  // the difference is exact
+    m[2 * h] = fmaxf(m[2 * h], v[2 * h]);
+    m[2 * h + 1] = fmaxf(m[2 * h + 1], v[2 * h + 1]);
   }
 }
 
-// A CTA covers kSRowsCta consecutive camera rows (one warp each, blockIdx.y)
-// and kSLanesX x kSVec columns x (blockIdx.x).  The columns j of row k whose
-// lower plane is n form one run; it is found from an FP32 estimate and
-// corrected with the exact split-table arithmetic.  The runs move up in j
-// with k (n0 grows with j and falls with k), so the CTA's rows share a
-// narrow band of columns j: their z-MIP values meet in a shared tile of
-// kSTileJ columns from the first row's run start (shared atomic max), and
-// the tile goes to the global z-MIP once per (j, x) at the end.  Voxels past
-// the tile take the global atomic directly.  uint16 voxels are >= 0 and the
-// outputs start at 0, so a zero left in the tile is skipped: the maxima are
-// the same bits as one global atomic per voxel.
-__global__ void __launch_bounds__(kSLanesX * kSRowsCta)
-k_stream_pair(PlanView v, const uint16_t* __restrict__ lo, const uint16_t* __restrict__ hi, int n, float* zmip,
-              float* zsum, float* ymip, int vec_ok) {
-  __shared__ float zt[kSTileJ][kSLanesX * kSVec];
-  __shared__ int jbase_s;
-  const int lane = threadIdx.x & 31, wrow = threadIdx.x >> 5;
-  const int k = blockIdx.y * kSRowsCta + wrow;
-  const int xl = lane * kSVec;
-  const int x0 = blockIdx.x * (kSLanesX * kSVec) + xl;
-  for (int i = threadIdx.x; i < kSTileJ * kSLanesX * kSVec; i += blockDim.x) (&zt[0][0])[i] = 0.0f;
-  // first column with lower plane >= n: estimate, then walk (bounded)
-  int j = 0, n0 = 0, steps = 0;
-  float w = 0.0f;
-  const bool row_ok = k < v.nz;
-  Split b{0, 0.0f};
-  if (row_ok) {
-    b = v.B[k];
-    const float half = v.linear ? 0.0f : 0.5f;
-    const float est = (float)v.J0 + ((float)n - half + (float)b.i + b.f) * v.rinv;
-    j = (int)fminf(fmaxf(floorf(est), 0.0f), (float)(v.ny - 1));
-    while (j > 0 && steps < kSearchSteps) {
-      plane_weight(v.A[j - 1], b, v.linear, n0, w);
-      if (n0 < n) break;
-      --j;
-      ++steps;
-    }
-    while (j < v.ny && steps < kSearchSteps) {
-      plane_weight(v.A[j], b, v.linear, n0, w);
-      if (n0 >= n) break;
-      ++j;
-      ++steps;
+// Column j: its rows in pair B (nB = nA + 1, which come first) and pair A.
+template <bool VEC, bool SUM>
+__device__ __forceinline__ void fold_column(const PlanView& v, const Pair& A, const Pair& B, int j, int lane, int x0,
+                                            int lim, Fold& f) {
+  const Split aj = v.A[j];
+  const int top = B.n != kNoPair ? B.n : A.n, bottom = A.n != kNoPair ? A.n : B.n;
+  auto lower = [&](int k) {
+    const Split b = v.B[k];
+    return aj.i - b.i - (aj.f - b.f < 0.0f);
+  };
+  for (int k = first_index(v.nz, lane, [&](int i) { return lower(i) <= top; }); k < v.nz; ++k) {
+    int n0;
+    float w;
+    plane_weight(aj, v.B[k], v.linear, n0, w);
+    if (n0 < bottom) break;
+    f.any = true;
+    const bool isB = n0 == B.n;
+    const size_t o = (size_t)k * v.ncols + x0;
+    f2 lo[2], hi[2];
+    load_counts<VEC>(isB ? B.lo : A.lo, o, lim, lo);
+    load_counts<VEC>(isB ? B.hi : A.hi, o, lim, hi);
+    float val[kSXL];
+    if (isB) {
+      fold_voxel(w, lo, hi, f.b, val);
+    } else {
+      fold_voxel(w, lo, hi, f.a, val);
+      if constexpr (SUM)
+#pragma unroll
+        for (int c = 0; c < kSXL; ++c) f.s[c] += val[c];
     }
   }
-  const bool found = row_ok && steps < kSearchSteps;
-  if (row_ok && !found && lane == 0) atomicOr(v.err, kErrSearch);
-  if (wrow == 0) jbase_s = j;  // the first row's run start (row 0 of a CTA always exists)
-  __syncthreads();
-  const int jbase = jbase_s;
-  if (found && x0 < v.nx) {
-    float a[kSVec], d[kSVec];
-    const bool vec = vec_ok && x0 + kSVec <= v.nx;
-    load_row(lo, v, k, x0, vec, a);
-    load_row(hi, v, k, x0, vec, d);
-#pragma unroll
-    for (int i = 0; i < kSVec; ++i) d[i] = d[i] - a[i];  // exact: integers below 2^24
-    float ym[kSVec];
-#pragma unroll
-    for (int i = 0; i < kSVec; ++i) ym[i] = 0.0f;  // uint16 voxels are >= 0
-    bool any = false;
-#pragma unroll 1
-    for (; j < v.ny; ++j) {
-      plane_weight(v.A[j], b, v.linear, n0, w);
-      if (n0 != n) break;
-      any = true;
-      const int jt = j - jbase;  // >= 0: runs move up with k
-      const bool in_tile = jt >= 0 && jt < kSTileJ;
-      const size_t row = (size_t)j * v.nx + x0;
-#pragma unroll
-      for (int i = 0; i < kSVec; ++i) {
-        if (x0 + i >= v.nx) break;
-        const float val = fmaf(w, d[i], a[i]);
-        ym[i] = fmaxf(ym[i], val);
-        if (zmip) {
-          if (in_tile)
-            atomicMax(reinterpret_cast<int*>(&zt[jt][xl + i]), __float_as_int(val));
-          else
-            atomicMax(reinterpret_cast<int*>(zmip + row + i), __float_as_int(val));
-        }
-        if (zsum) atomicAdd(zsum + row + i, val);
-      }
+}
+
+// Row k: its columns in pair A (which come first) and pair B.
+template <bool VEC>
+__device__ __forceinline__ void fold_row(const PlanView& v, const Pair& A, const Pair& B, int k, int lane, int x0,
+                                         int lim, Fold& f) {
+  const Split b = v.B[k];
+  const int top = B.n != kNoPair ? B.n : A.n, bottom = A.n != kNoPair ? A.n : B.n;
+  auto lower = [&](int j) {
+    const Split a = v.A[j];
+    return a.i - b.i - (a.f - b.f < 0.0f);
+  };
+  const size_t o = (size_t)k * v.ncols + x0;
+  f2 lo[2], hi[2];
+  int held = kNoPair;
+  for (int j = first_index(v.ny, lane, [&](int i) { return lower(i) >= bottom; }); j < v.ny; ++j) {
+    int n0;
+    float w;
+    plane_weight(v.A[j], b, v.linear, n0, w);
+    if (n0 > top) break;
+    f.any = true;
+    const bool isB = n0 == B.n;
+    if (n0 != held) {
+      load_counts<VEC>(isB ? B.lo : A.lo, o, lim, lo);
+      load_counts<VEC>(isB ? B.hi : A.hi, o, lim, hi);
+      held = n0;
     }
-    if (ymip && any) {
-      float* yr = ymip + (size_t)k * v.nx + x0;
+    float val[kSXL];
+    if (isB)
+      fold_voxel(w, lo, hi, f.b, val);
+    else
+      fold_voxel(w, lo, hi, f.a, val);
+  }
+}
+
+template <bool VEC>
+__device__ __forceinline__ void get(const float* p, int lim, float (&out)[kSXL]) {
+  if constexpr (VEC) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    out[0] = q.x, out[1] = q.y, out[2] = q.z, out[3] = q.w;
+  } else {
 #pragma unroll
-      for (int i = 0; i < kSVec; ++i)
-        if (x0 + i < v.nx) yr[i] = fmaxf(yr[i], ym[i]);  // one thread per (k, x) in this launch
+    for (int c = 0; c < kSXL; ++c) out[c] = 32 * c < lim ? p[32 * c] : 0.0f;
+  }
+}
+template <bool VEC>
+__device__ __forceinline__ void put(float* p, int lim, const float (&v)[kSXL]) {
+  if constexpr (VEC) {
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  } else {
+#pragma unroll
+    for (int c = 0; c < kSXL; ++c)
+      if (32 * c < lim) p[32 * c] = v[c];
+  }
+}
+__device__ __forceinline__ void max_into(float (&a)[kSXL], const float (&b)[kSXL]) {
+#pragma unroll
+  for (int c = 0; c < kSXL; ++c) a[c] = fmaxf(a[c], b[c]);
+}
+
+// Which column j or row k a warp owns, and its columns x.  Blocks: x-tiles
+// fastest, the columns [j0, j1) in groups of kSWarps, then the rows.
+struct Place {
+  bool column, live;
+  int i;        // j or k
+  int x0, lim;  // first column x of the lane, columns from there to the edge
+};
+template <bool VEC>
+__device__ __forceinline__ Place place(const PlanView& v, int xtiles, int j0, int j1) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int jgroups = (j1 - j0 + kSWarps - 1) / kSWarps;
+  const int g = blockIdx.x / xtiles, xb = (blockIdx.x - g * xtiles) * kSXW;
+  Place p;
+  p.column = g < jgroups;
+  p.i = (p.column ? j0 + g * kSWarps : (g - jgroups) * kSWarps) + warp;
+  p.live = p.i < (p.column ? j1 : v.nz);
+  p.x0 = xb + (VEC ? lane * kSXL : lane);
+  p.lim = v.nx - p.x0;
+  if (VEC && p.lim <= 0) p.x0 = 0;  // reads something, writes nothing
+  return p;
+}
+
+// Pair A into the outputs (any of them NULL): columns [j0, j1) hold its voxels.
+template <bool VEC, bool SUM>
+__global__ void __launch_bounds__(32 * kSWarps)
+k_stream_pair(PlanView v, Pair A, int xtiles, int j0, int j1, float* zmip, float* zsum, float* ymip) {
+  const Place p = place<VEC>(v, xtiles, j0, j1);
+  if (!p.live) return;
+  const int lane = threadIdx.x & 31;
+  const Pair none{nullptr, nullptr, kNoPair};
+  Fold f{};
+  if (p.column)
+    fold_column<VEC, SUM>(v, A, none, p.i, lane, p.x0, p.lim, f);
+  else
+    fold_row<VEC>(v, A, none, p.i, lane, p.x0, p.lim, f);
+  float* out = p.column ? zmip : ymip;
+  if (!f.any || p.lim <= 0) return;
+  const size_t o = (size_t)p.i * v.nx + p.x0;
+  float old[kSXL];
+  if (out) {
+    get<VEC>(out + o, p.lim, old);
+    max_into(f.a, old);
+    put<VEC>(out + o, p.lim, f.a);
+  }
+  if constexpr (SUM) {
+    if (p.column) {
+      get<VEC>(zsum + o, p.lim, old);
+#pragma unroll
+      for (int c = 0; c < kSXL; ++c) old[c] += f.s[c];
+      put<VEC>(zsum + o, p.lim, old);
     }
   }
-  if (!zmip) return;
-  __syncthreads();
-  const int xb = blockIdx.x * (kSLanesX * kSVec);
-  for (int i = threadIdx.x; i < kSTileJ * kSLanesX * kSVec; i += blockDim.x) {
-    const int jt = i / (kSLanesX * kSVec), xx = i % (kSLanesX * kSVec);
-    const float val = (&zt[0][0])[i];
-    if (val != 0.0f && jbase + jt < v.ny && xb + xx < v.nx)
-      atomicMax(reinterpret_cast<int*>(zmip + (size_t)(jbase + jt) * v.nx + xb + xx), __float_as_int(val));
+}
+
+// One push of the sliding view (launch_sliding_push): pair A is complete, B is
+// the mixed pair, or the stack's last (`last`: complete as well).
+//   run  = max(run, A[, B])   (fresh: without the old run)
+//   slotA = A, slotB = B      (where given)
+//   view = max(run, next, B)
+struct Slide {
+  float* run;
+  float* slotA;
+  float* slotB;
+  const float* next;
+  float* view;
+  bool fresh, last;
+};
+
+template <bool VEC>
+__global__ void __launch_bounds__(32 * kSWarps)
+k_sliding_push(PlanView v, Pair A, Pair B, Slide s, int xtiles) {
+  const Place p = place<VEC>(v, xtiles, 0, v.ny);
+  if (!p.live) return;
+  const int lane = threadIdx.x & 31;
+  const size_t o = (p.column ? (size_t)0 : (size_t)v.ny * v.nx) + (size_t)p.i * v.nx + p.x0;
+  float run[kSXL] = {}, next[kSXL] = {};
+  if (p.lim > 0) {  // on their way while the run is searched
+    if (!s.fresh) get<VEC>(s.run + o, p.lim, run);
+    if (s.next) get<VEC>(s.next + o, p.lim, next);
+  }
+  Fold f{};
+  if (p.column)
+    fold_column<VEC, false>(v, A, B, p.i, lane, p.x0, p.lim, f);
+  else
+    fold_row<VEC>(v, A, B, p.i, lane, p.x0, p.lim, f);
+  if (p.lim <= 0) return;
+  if (s.slotA) put<VEC>(s.slotA + o, p.lim, f.a);
+  if (s.slotB) put<VEC>(s.slotB + o, p.lim, f.b);
+  max_into(run, f.a);
+  if (s.last) max_into(run, f.b);
+  if (f.any || s.fresh) put<VEC>(s.run + o, p.lim, run);
+  max_into(run, next);
+  max_into(run, f.b);
+  put<VEC>(s.view + o, p.lim, run);
+}
+
+// Suffix maxima of the slots: slot q = max(slot q, .., slot last), q = last - 1
+// down to 1, one element (four when vec) per thread.
+template <typename V>
+__global__ void __launch_bounds__(256)
+k_suffix_max(V* slots, size_t per, int last) {
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= per) return;
+  V* p = slots + (size_t)last * per + i;
+  V m = *p;
+  // a few slots' loads in flight at a time
+  constexpr int kAhead = 4;
+  int q = last - 1;
+  for (; q >= kAhead; q -= kAhead) {
+    V t[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) t[u] = __ldcs(p - (size_t)(u + 1) * per);
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      p -= per;
+      if constexpr (sizeof(V) == 16)
+        m = make_float4(fmaxf(m.x, t[u].x), fmaxf(m.y, t[u].y), fmaxf(m.z, t[u].z), fmaxf(m.w, t[u].w));
+      else
+        m = fmaxf(m, t[u]);
+      *p = m;
+    }
+  }
+  for (; q >= 1; --q) {
+    p -= per;
+    const V t = *p;
+    if constexpr (sizeof(V) == 16)
+      m = make_float4(fmaxf(m.x, t.x), fmaxf(m.y, t.y), fmaxf(m.z, t.z), fmaxf(m.w, t.w));
+    else
+      m = fmaxf(m, t);
+    *p = m;
   }
 }
 
@@ -180,14 +371,42 @@ opm_status launch_stream_begin(const opm_plan* p, float* zmip, float* zsum, floa
   return e == cudaSuccess ? OPM_OK : cuda_fail(e, "launch k_stream_zero");
 }
 
+// Vectors of kSXL when frames and outputs start every row on one.
+static bool stream_vec(const PlanView& v, const void* f0, const void* f1, const void* f2) {
+  return v.nx % kSXL == 0 && (uintptr_t)f0 % 8 == 0 && (uintptr_t)f1 % 8 == 0 && (uintptr_t)f2 % 8 == 0;
+}
+static bool vec_out(const void* p) { return (uintptr_t)p % 16 == 0; }
+
+// Blocks for columns [j0, j1) and all rows; 0 when there are too many.
+static unsigned stream_blocks(const PlanView& v, long long columns, bool rows) {
+  const long long xtiles = (v.nx + kSXW - 1) / kSXW;
+  const long long groups = (columns + kSWarps - 1) / kSWarps + (rows ? (v.nz + kSWarps - 1) / kSWarps : 0);
+  return xtiles * groups <= 0x7fffffffLL ? (unsigned)(xtiles * groups) : 0u;
+}
+
 opm_status launch_stream_pair(const opm_plan* p, const uint16_t* lo, const uint16_t* hi, int n, float* zmip,
                               float* zsum, float* ymip, cudaStream_t s) {
   const PlanView& v = p->view;
-  const int xblocks = (v.nx + kSLanesX * kSVec - 1) / (kSLanesX * kSVec);
   if (v.nz > 65535) return fail(OPM_ERR_UNSUPPORTED, "more than 65535 camera rows");
-  const int vec_ok = (v.ncols % kSVec == 0) && ((uintptr_t)lo % 8 == 0) && ((uintptr_t)hi % 8 == 0);
-  const int rblocks = (v.nz + kSRowsCta - 1) / kSRowsCta;
-  k_stream_pair<<<dim3(xblocks, rblocks), kSLanesX * kSRowsCta, 0, s>>>(v, lo, hi, n, zmip, zsum, ymip, vec_ok);
+  // columns with a voxel in the pair: n0 grows with j and falls with k
+  const Split b0 = p->hB.front(), b1 = p->hB.back();
+  const auto lower = [](const Split& a, const Split& b) { return a.i - b.i - (a.f - b.f < 0.0f ? 1 : 0); };
+  const auto first = [&](const Split& b, int least) {
+    return (int)(std::partition_point(p->hA.begin(), p->hA.end(), [&](const Split& a) { return lower(a, b) < least; }) -
+                 p->hA.begin());
+  };
+  int j0 = first(b0, n), j1 = first(b1, n + 1);
+  if ((!zmip && !zsum) || j1 < j0) j1 = j0;
+  const unsigned blocks = stream_blocks(v, j1 - j0, ymip != nullptr);
+  if (blocks == 0) {
+    if (j1 == j0 && !ymip) return OPM_OK;  // the pair has no voxel
+    return fail(OPM_ERR_UNSUPPORTED, "plane-pair grid exceeds launch limits");
+  }
+  const bool vec = stream_vec(v, lo, hi, nullptr) && vec_out(zmip) && vec_out(zsum) && vec_out(ymip);
+  const int xtiles = (v.nx + kSXW - 1) / kSXW;
+  const auto kern = zsum ? (vec ? k_stream_pair<true, true> : k_stream_pair<false, true>)
+                         : (vec ? k_stream_pair<true, false> : k_stream_pair<false, false>);
+  kern<<<blocks, 32 * kSWarps, 0, s>>>(v, Pair{lo, hi, n}, xtiles, j0, j1, zmip, zsum, ymip);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? OPM_OK : cuda_fail(e, "launch k_stream_pair");
 }
@@ -223,39 +442,43 @@ opm_status launch_max_combine(float* out, const float* a, const float* b, int64_
 opm_status launch_sliding_push(const opm_plan* p, const uint16_t* stack, int m, float* run, float* slots,
                                float* view, cudaStream_t s) {
   const PlanView& v = p->view;
+  if (v.nz > 65535) return fail(OPM_ERR_UNSUPPORTED, "more than 65535 camera rows");
   const int N = v.nscan;
-  const size_t zn = (size_t)v.ny * v.nx, per = zn + (size_t)v.nz * v.nx;
+  const size_t per = ((size_t)v.ny + v.nz) * v.nx;
   const size_t frame = (size_t)v.nrows * v.ncols;
-  auto F = [&](int n) { return stack + (size_t)n * frame; };
+  auto F = [&](int n) { return n >= 0 && n < N ? stack + (size_t)n * frame : nullptr; };
   auto slot = [&](int q) { return slots + (size_t)q * per; };
-  opm_status st = OPM_OK;
-  // pair q (frames q, q + 1 of the new stack) into slot q, then into run
-  auto pair_into_slot = [&](int q) {
-    float* b = slot(q);
-    opm_status r = launch_stream_begin(p, b, nullptr, b + zn, s);
-    if (r == OPM_OK) r = launch_stream_pair(p, F(q), q + 1 < N ? F(q + 1) : nullptr, q, b, nullptr, b + zn, s);
-    if (r == OPM_OK) r = launch_max_combine(run, run, b, (int64_t)per, s);
-    return r;
-  };
-  if (m == 0) {  // pair -1: the new stack's first frame alone
-    st = launch_stream_begin(p, run, nullptr, run + zn, s);
-    if (st == OPM_OK) st = launch_stream_pair(p, nullptr, F(0), -1, run, nullptr, run + zn, s);
-  } else if (m == 1) {  // pair 0 is never read from a slot: straight into run
-    st = launch_stream_pair(p, F(0), F(1), 0, run, nullptr, run + zn, s);
-  } else {
-    st = pair_into_slot(m - 1);
+  const bool last = m == N - 1;
+  // the pair that frame m completes, and the one it opens (with the previous
+  // stack's frame m + 1, or with nothing behind the last frame)
+  const Pair A{F(m - 1), F(m), m - 1}, B{F(m), F(m + 1), m};
+  Slide sl;
+  sl.run = run;
+  sl.slotA = m >= 2 ? slot(m - 1) : nullptr;  // pairs -1 and 0 are never read from a slot
+  sl.slotB = last ? slot(m) : nullptr;
+  sl.next = last ? nullptr : slot(m + 1);
+  sl.view = view;
+  sl.fresh = m == 0;
+  sl.last = last;
+  const unsigned blocks = stream_blocks(v, v.ny, true);
+  if (blocks == 0) return fail(OPM_ERR_UNSUPPORTED, "sliding-view grid exceeds launch limits");
+  const bool vec = stream_vec(v, A.lo, A.hi, B.hi) && per % kSXL == 0 && vec_out(run) && vec_out(slots) && vec_out(view);
+  const int xtiles = (v.nx + kSXW - 1) / kSXW;
+  (vec ? k_sliding_push<true> : k_sliding_push<false>)<<<blocks, 32 * kSWarps, 0, s>>>(v, A, B, sl, xtiles);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(e, "launch k_sliding_push");
+  if (last && N > 2) {  // the next stack's suffixes
+    const size_t n = vec ? per / 4 : per;
+    const size_t nb = (n + 255) / 256;
+    if (nb > 0x7fffffffULL) return fail(OPM_ERR_UNSUPPORTED, "sliding-view grid exceeds launch limits");
+    if (vec)
+      k_suffix_max<<<(unsigned)nb, 256, 0, s>>>(reinterpret_cast<float4*>(slots), n, N - 1);
+    else
+      k_suffix_max<<<(unsigned)nb, 256, 0, s>>>(slots, n, N - 1);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(e, "launch k_suffix_max");
   }
-  if (st != OPM_OK) return st;
-  if (m == N - 1) {  // the last frame closes the stack, then the next suffixes
-    st = pair_into_slot(N - 1);
-    if (st == OPM_OK) st = launch_max_combine(view, run, run, (int64_t)per, s);
-    for (int q = N - 2; q >= 1 && st == OPM_OK; --q) st = launch_max_combine(slot(q), slot(q), slot(q + 1), (int64_t)per, s);
-    return st;
-  }
-  // new pairs, the previous stack's pairs m + 1 .. N - 1, then the mixed pair m
-  st = launch_max_combine(view, run, slot(m + 1), (int64_t)per, s);
-  if (st == OPM_OK) st = launch_stream_pair(p, F(m), F(m + 1), m, view, nullptr, view + zn, s);
-  return st;
+  return OPM_OK;
 }
 
 }  // namespace opm
