@@ -204,46 +204,75 @@ def opm_plan_check(plan: Plan):
 
 
 # ------------------------------------------------------------------ tensors
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
+
+
+_dtypes: dict = {}
 
 
 def _dtype_code(t) -> int:
-    torch = _torch()
-    m = {torch.uint16: OPM_U16, torch.float32: OPM_F32, torch.float64: OPM_F64}
-    if t.dtype not in m:
+    if not _dtypes:
+        torch = _torch()
+        _dtypes.update({torch.uint16: OPM_U16, torch.float32: OPM_F32, torch.float64: OPM_F64})
+    code = _dtypes.get(t.dtype)
+    if code is None:
         raise TypeError(f"unsupported dtype {t.dtype} (uint16, float32 or float64)")
-    return m[t.dtype]
+    return code
 
 
-def _ptr(t, shape=None, name="tensor"):
+def _device() -> int:
+    """The current CUDA device, -1 while this process has not used one."""
+    cuda = _torch().cuda
+    return cuda.current_device() if cuda.is_initialized() else -1
+
+
+def _ptr(t, shape=None, name="tensor", dev=None):
+    """Device address of a checked tensor (None for None).  Called for every
+    array of every call: each test is one cheap query, and calls with several
+    arrays ask for the current device once (``dev``)."""
     if t is None:
         return None
-    if not t.is_cuda:
+    index = t.get_device()
+    if index < 0:
         raise ValueError(f"{name} must be a CUDA tensor")
-    dev = _torch().cuda.current_device()
-    if t.device.index != dev:
+    if dev is None:
+        dev = _device()
+    if index != dev:
         # the plan lives on the current device; a kernel there must not be
         # handed another GPU's memory
-        raise ValueError(f"{name} is on cuda:{t.device.index}, the current device is cuda:{dev}")
+        raise ValueError(f"{name} is on cuda:{index}, the current device is cuda:{dev}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape:
         raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream(stream):
-    torch = _torch()
+def _current_raw_stream(dev: int) -> int:
+    """cudaStream_t of the device's current torch stream."""
+    return _torch()._C._cuda_getCurrentRawStream(dev)
+
+
+def _stream(stream, dev=None):
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+        if dev is None:
+            dev = _device()
+        return _current_raw_stream(dev) if dev >= 0 else 0
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def opm_deskew(plan: Plan, raw, vol, stream=None):
-    _check(load().opm_deskew(plan.handle, _ptr(raw, plan.raw_shape, "raw"), _dtype_code(raw),
-                             _ptr(vol, plan.vol_shape, "vol"), _dtype_code(vol), _stream(stream)), "opm_deskew")
+    dev = _device()
+    _check(load().opm_deskew(plan.handle, _ptr(raw, plan.raw_shape, "raw", dev), _dtype_code(raw),
+                             _ptr(vol, plan.vol_shape, "vol", dev), _dtype_code(vol), _stream(stream, dev)), "opm_deskew")
 
 
 def opm_sheet_rows(nscan: int, nrows: int, shear: float) -> int:
@@ -284,9 +313,10 @@ def opm_sliding_push(plan: Plan, stack, m: int, run, slots, view, stream=None):
     """``opm_sliding_push`` on CUDA tensors: stack uint16 [nscan][nrows][ncols],
     run and view float32 [P], slots float32 [nscan][P], P = ny nx + nz nx."""
     P = plan.ny * plan.nx + plan.nz * plan.nx
-    _check(load().opm_sliding_push(plan.handle, _ptr(stack, plan.raw_shape, "stack"), int(m),
-                                   _ptr(run, (P,), "run"), _ptr(slots, (plan.nscan, P), "slots"),
-                                   _ptr(view, (P,), "view"), _stream(stream)), "opm_sliding_push")
+    dev = _device()
+    _check(load().opm_sliding_push(plan.handle, _ptr(stack, plan.raw_shape, "stack", dev), int(m),
+                                   _ptr(run, (P,), "run", dev), _ptr(slots, (plan.nscan, P), "slots", dev),
+                                   _ptr(view, (P,), "view", dev), _stream(stream, dev)), "opm_sliding_push")
 
 
 def opm_sheet_check():
@@ -314,34 +344,41 @@ def opm_deskew_mip(plan: Plan, raw, vol_f32=None, vol_u16=None, zmip=None, ymip=
     if vol_u16 is not None and vol_u16.dtype != torch.uint16:
         raise TypeError("vol_u16 must be uint16")
     pj = (plan.ny, plan.nx)
-    _check(load().opm_deskew_mip(plan.handle, _ptr(raw, plan.raw_shape, "raw"), _dtype_code(raw),
-                                 _ptr(vol_f32, plan.vol_shape, "vol_f32"), _ptr(vol_u16, plan.vol_shape, "vol_u16"),
-                                 _ptr(zmip, pj, "zmip"), _ptr(ymip, (plan.nz, plan.nx), "ymip"), _stream(stream)),
+    dev = _device()
+    _check(load().opm_deskew_mip(plan.handle, _ptr(raw, plan.raw_shape, "raw", dev), _dtype_code(raw),
+                                 _ptr(vol_f32, plan.vol_shape, "vol_f32", dev),
+                                 _ptr(vol_u16, plan.vol_shape, "vol_u16", dev), _ptr(zmip, pj, "zmip", dev),
+                                 _ptr(ymip, (plan.nz, plan.nx), "ymip", dev), _stream(stream, dev)),
            "opm_deskew_mip")
 
 
 def opm_stream_begin(plan: Plan, zmip=None, zsum=None, ymip=None, stream=None):
     pj = (plan.ny, plan.nx)
-    _check(load().opm_stream_begin(plan.handle, _ptr(zmip, pj, "zmip"), _ptr(zsum, pj, "zsum"),
-                                   _ptr(ymip, (plan.nz, plan.nx), "ymip"), _stream(stream)), "opm_stream_begin")
+    dev = _device()
+    _check(load().opm_stream_begin(plan.handle, _ptr(zmip, pj, "zmip", dev), _ptr(zsum, pj, "zsum", dev),
+                                   _ptr(ymip, (plan.nz, plan.nx), "ymip", dev), _stream(stream, dev)), "opm_stream_begin")
 
 
 def opm_stream_pair(plan: Plan, plane_lo, plane_hi, n: int, zmip=None, zsum=None, ymip=None, stream=None):
     """Frames are uint16 CUDA tensors [nrows][ncols] (None outside the stack)."""
     fr = (plan.nrows, plan.ncols)
     pj = (plan.ny, plan.nx)
-    _check(load().opm_stream_pair(plan.handle, _ptr(plane_lo, fr, "plane_lo"), _ptr(plane_hi, fr, "plane_hi"), int(n),
-                                  _ptr(zmip, pj, "zmip"), _ptr(zsum, pj, "zsum"), _ptr(ymip, (plan.nz, plan.nx), "ymip"),
-                                  _stream(stream)), "opm_stream_pair")
+    dev = _device()
+    _check(load().opm_stream_pair(plan.handle, _ptr(plane_lo, fr, "plane_lo", dev),
+                                  _ptr(plane_hi, fr, "plane_hi", dev), int(n), _ptr(zmip, pj, "zmip", dev),
+                                  _ptr(zsum, pj, "zsum", dev), _ptr(ymip, (plan.nz, plan.nx), "ymip", dev),
+                                  _stream(stream, dev)), "opm_stream_pair")
 
 
 def opm_deskew_dual(plan: Plan, raw, vol_f32, vol_u16, stream=None):
     torch = _torch()
     if vol_f32.dtype != torch.float32 or vol_u16.dtype != torch.uint16:
         raise TypeError("vol_f32 must be float32 and vol_u16 uint16")
-    _check(load().opm_deskew_dual(plan.handle, _ptr(raw, plan.raw_shape, "raw"), _dtype_code(raw),
-                                  _ptr(vol_f32, plan.vol_shape, "vol_f32"), _ptr(vol_u16, plan.vol_shape, "vol_u16"),
-                                  _stream(stream)), "opm_deskew_dual")
+    dev = _device()
+    _check(load().opm_deskew_dual(plan.handle, _ptr(raw, plan.raw_shape, "raw", dev), _dtype_code(raw),
+                                  _ptr(vol_f32, plan.vol_shape, "vol_f32", dev),
+                                  _ptr(vol_u16, plan.vol_shape, "vol_u16", dev),
+                                  _stream(stream, dev)), "opm_deskew_dual")
 
 
 def opm_project(plan: Plan, raw, zmip=None, zsum=None, ymip=None, argz=None, stream=None):
@@ -352,18 +389,20 @@ def opm_project(plan: Plan, raw, zmip=None, zsum=None, ymip=None, argz=None, str
     if argz is not None and argz.dtype != torch.int32:
         raise TypeError("argz must be int32")
     pj = (plan.ny, plan.nx)
-    _check(load().opm_project(plan.handle, _ptr(raw, plan.raw_shape, "raw"), _dtype_code(raw),
-                              _ptr(zmip, pj, "zmip"), _ptr(zsum, pj, "zsum"),
-                              _ptr(ymip, (plan.nz, plan.nx), "ymip"), _ptr(argz, pj, "argz"),
-                              _stream(stream)), "opm_project")
+    dev = _device()
+    _check(load().opm_project(plan.handle, _ptr(raw, plan.raw_shape, "raw", dev), _dtype_code(raw),
+                              _ptr(zmip, pj, "zmip", dev), _ptr(zsum, pj, "zsum", dev),
+                              _ptr(ymip, (plan.nz, plan.nx), "ymip", dev), _ptr(argz, pj, "argz", dev),
+                              _stream(stream, dev)), "opm_project")
 
 
 def opm_skew_adjoint(plan: Plan, vol, raw_out, stream=None):
     if vol.dtype != raw_out.dtype:
         raise TypeError("vol and raw_out must share a dtype")
-    _check(load().opm_skew_adjoint(plan.handle, _ptr(vol, plan.vol_shape, "vol"),
-                                   _ptr(raw_out, plan.raw_shape, "raw_out"), _dtype_code(vol),
-                                   _stream(stream)), "opm_skew_adjoint")
+    dev = _device()
+    _check(load().opm_skew_adjoint(plan.handle, _ptr(vol, plan.vol_shape, "vol", dev),
+                                   _ptr(raw_out, plan.raw_shape, "raw_out", dev), _dtype_code(vol),
+                                   _stream(stream, dev)), "opm_skew_adjoint")
 
 
 def opm_mip_backward(plan: Plan, g_zmip, argz, g_raw, stream=None):
@@ -371,8 +410,9 @@ def opm_mip_backward(plan: Plan, g_zmip, argz, g_raw, stream=None):
     if g_zmip.dtype != torch.float32 or g_raw.dtype != torch.float32 or argz.dtype != torch.int32:
         raise TypeError("g_zmip/g_raw must be float32 and argz int32")
     pj = (plan.ny, plan.nx)
-    _check(load().opm_mip_backward(plan.handle, _ptr(g_zmip, pj, "g_zmip"), _ptr(argz, pj, "argz"),
-                                   _ptr(g_raw, plan.raw_shape, "g_raw"), _stream(stream)), "opm_mip_backward")
+    dev = _device()
+    _check(load().opm_mip_backward(plan.handle, _ptr(g_zmip, pj, "g_zmip", dev), _ptr(argz, pj, "argz", dev),
+                                   _ptr(g_raw, plan.raw_shape, "g_raw", dev), _stream(stream, dev)), "opm_mip_backward")
 
 
 # ------------------------------------------------------- allocating helpers

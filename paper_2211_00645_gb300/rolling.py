@@ -33,7 +33,7 @@ from __future__ import annotations
 
 from typing import Optional
 
-from . import Plan, opm_sliding_push, opm_stream_begin, opm_stream_pair
+from . import Plan, _current_raw_stream, opm_sliding_push, opm_stream_begin, opm_stream_pair
 
 
 class RollingView:
@@ -73,19 +73,29 @@ class RollingView:
     def _outs(self):
         return self.zmip, self.zsum, self.ymip
 
+    def _copy_in(self, dst, frame):
+        """frame (int16 view) into dst on the view's stream; entering a stream
+        context costs more than the rest of the copy call, so it is entered
+        only when another stream is current."""
+        torch = self.torch
+        if _current_raw_stream(dst.get_device()) == self.stream.cuda_stream:
+            dst.copy_(frame, non_blocking=True)
+        else:
+            with torch.cuda.stream(self.stream):
+                dst.copy_(frame, non_blocking=True)
+
     def push(self, frame) -> Optional[dict]:
         """Adds the next frame (uint16 [nrows][ncols], host or device).
         Returns {"zmip", "ymip"[, "zsum"], "frames", "complete"} (device
         tensors, valid until the next push) when the mode publishes a view."""
         torch = self.torch
         p = self.plan
-        if tuple(frame.shape) != (p.nrows, p.ncols) or frame.dtype != torch.uint16:
+        if frame.shape != (p.nrows, p.ncols) or frame.dtype != torch.uint16:
             raise ValueError(f"frame must be uint16 {(p.nrows, p.ncols)}")
         if self.mode == "sliding":
             return self._push_sliding(frame)
         cur = self.frames[self.n % 2]
-        with torch.cuda.stream(self.stream):
-            cur.view(torch.int16).copy_(frame.view(torch.int16), non_blocking=True)
+        self._copy_in(cur.view(torch.int16), frame.view(torch.int16))
         zmip, zsum, ymip = self._outs()
         if self.n == 0:
             opm_stream_begin(p, zmip, zsum, ymip, self.stream)
@@ -109,8 +119,7 @@ class RollingView:
         torch = self.torch
         p = self.plan
         m = self.n
-        with torch.cuda.stream(self.stream):
-            self.stack[m].view(torch.int16).copy_(frame.view(torch.int16), non_blocking=True)
+        self._copy_in(self.stack[m].view(torch.int16), frame.view(torch.int16))
         if self.fast_sliding:
             opm_sliding_push(p, self.stack, m, self.run, self.slots, self.view, self.stream)
         else:
