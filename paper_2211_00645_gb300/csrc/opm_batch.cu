@@ -160,7 +160,7 @@ k_batch_fast(const unsigned char* __restrict__ wl, int Pl, unsigned* err) {
       __syncwarp();
       ok = fast_produce(jb, ring, g, err, lane);
     } else {
-      ok = fast_consume(jb, ring, g, err, warp - 1, lane);
+      ok = fast_consume<true>(jb, ring, g, err, warp - 1, lane);
     }
   }
   if (warp == 0) fast_drain(ring, g, ok, err);
@@ -223,7 +223,7 @@ k_batch_per(const unsigned char* __restrict__ wl, int Pl, unsigned* err) {
       __syncwarp();
       ok = per_produce(jb, ring, g, err, lane);
     } else {
-      ok = per_consume<RUN, Pp, Qq>(jb, ring, g, err, warp - 1, lane);
+      ok = per_consume<RUN, Pp, Qq, true>(jb, ring, g, err, warp - 1, lane);
     }
   }
   if (warp == 0) per_drain(ring, g, ok, err);

@@ -404,17 +404,24 @@ namespace {
 
 // The volume on the caller's stream s and the live view beside it on the
 // plan's high-priority side stream, forked from and joined back into s.
-// The live view's persistent kernel takes a quarter of its usual grid (one
-// CTA per SM), so each SM also holds volume CTAs: the issue-bound projection
-// then fills the issue slots the write-bound volume leaves idle.  Each
-// kernel computes exactly what it computes alone.
+// The live view's persistent kernel takes a part of its usual grid, so each SM
+// also holds volume CTAs: the issue-bound projection then fills the issue
+// slots the write-bound volume leaves idle.  Each kernel computes exactly what
+// it computes alone.
+// The two should end together: beside an FP32 volume (4 or 6 bytes a voxel) one
+// projection CTA per SM, beside a uint16 volume, which is written in half the
+// time, two.  us for the pair at 4 / 2 / 1 of them per SM and one after the
+// other (uint16 volume + z-MIP of 1000 x 1024 x 2048, 45 deg, 0.2, 0.115):
+// 3475 / 3297 / 3676 / 3746; uint16 + z + y of the 200 x 512 x 2048 live view:
+// 526 / 503 / 554 / 541; FP32 + z + y of it: 824 / 792 / 785 / 843.
 opm_status deskew_beside_project(const opm_plan* p, const void* raw, opm_dtype in_t, float* volf, uint16_t* volh,
                                  float* zmip, float* ymip, cudaStream_t s) {
   std::lock_guard<std::mutex> lock(p->side_mu);
   cudaError_t e = cudaEventRecord(p->fork_ev, s);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(p->side, p->fork_ev, 0);
   if (e != cudaSuccess) return cuda_fail(e, "forking the live view onto the side stream");
-  opm_status st = launch_project(p, raw, in_t, zmip, nullptr, ymip, nullptr, p->side, p->lists_per_sm);
+  opm_status st = launch_project(p, raw, in_t, zmip, nullptr, ymip, nullptr, p->side,
+                                 volf ? p->lists_per_sm : p->lists_per_sm / 2);
   opm_status sv = OPM_OK;
   if (volf && volh)
     sv = launch_deskew_dual(p, raw, in_t, volf, volh, s);

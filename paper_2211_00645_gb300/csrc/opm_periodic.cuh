@@ -170,7 +170,7 @@ __device__ __forceinline__ f2 lds_x2(const unsigned char* smem, uint32_t off) {
 // row 0 at phase PH0 and row 1 at phase PH1.  off0 / off1: shared-memory
 // offset of this lane's 2 columns x in the tile's first plane of each row;
 // wof0 / wof1: the tile's (w, w) weight pairs of each row.
-template <int RUN, int Pp, int Qq, int PH0, int PH1>
+template <int RUN, int Pp, int Qq, bool YMIP, int PH0, int PH1>
 __device__ __forceinline__ void per_pair(const unsigned char* __restrict__ smem, uint32_t off0, uint32_t off1,
                                          uint32_t wof0, uint32_t wof1, float (&zmax)[RUN][per::kXL],
                                          float (&ym0)[per::kXL], float (&ym1)[per::kXL]) {
@@ -204,7 +204,7 @@ __device__ __forceinline__ void per_pair(const unsigned char* __restrict__ smem,
     upk(fma2((t & 1) ? wq1.y : wq1.x, d1, a1), v1[0], v1[1]);
 #pragma unroll
     for (int c = 0; c < kXL; ++c) zmax[t][c] = max3(zmax[t][c], v0[c], v1[c]);
-    if (pcand(Pp, Qq, PH0, t, RUN)) {
+    if (YMIP && pcand(Pp, Qq, PH0, t, RUN)) {
       if (pcount(Pp, Qq, PH0, t, RUN) % 2 == 0) {
 #pragma unroll
         for (int c = 0; c < kXL; ++c) p0[c] = v0[c];
@@ -213,7 +213,7 @@ __device__ __forceinline__ void per_pair(const unsigned char* __restrict__ smem,
         for (int c = 0; c < kXL; ++c) ym0[c] = max3(ym0[c], p0[c], v0[c]);
       }
     }
-    if (pcand(Pp, Qq, PH1, t, RUN)) {
+    if (YMIP && pcand(Pp, Qq, PH1, t, RUN)) {
       if (pcount(Pp, Qq, PH1, t, RUN) % 2 == 0) {
 #pragma unroll
         for (int c = 0; c < kXL; ++c) p1[c] = v1[c];
@@ -223,29 +223,29 @@ __device__ __forceinline__ void per_pair(const unsigned char* __restrict__ smem,
       }
     }
   }
-  if (pcount(Pp, Qq, PH0, RUN, RUN) % 2 == 1) {
+  if (YMIP && pcount(Pp, Qq, PH0, RUN, RUN) % 2 == 1) {
 #pragma unroll
     for (int c = 0; c < kXL; ++c) ym0[c] = fmaxf(ym0[c], p0[c]);
   }
-  if (pcount(Pp, Qq, PH1, RUN, RUN) % 2 == 1) {
+  if (YMIP && pcount(Pp, Qq, PH1, RUN, RUN) % 2 == 1) {
 #pragma unroll
     for (int c = 0; c < kXL; ++c) ym1[c] = fmaxf(ym1[c], p1[c]);
   }
 }
 
 // Phase pair idx = PH0 * Qq + PH1 in [LO, HI), by a balanced branch tree.
-template <int RUN, int Pp, int Qq, int LO, int HI>
+template <int RUN, int Pp, int Qq, bool YMIP, int LO, int HI>
 __device__ __forceinline__ void per_tree(int idx, const unsigned char* __restrict__ smem, uint32_t off0,
                                          uint32_t off1, uint32_t wof0, uint32_t wof1, float (&zmax)[RUN][per::kXL],
                                          float (&ym0)[per::kXL], float (&ym1)[per::kXL]) {
   if constexpr (HI - LO == 1) {
-    per_pair<RUN, Pp, Qq, LO / Qq, LO % Qq>(smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
+    per_pair<RUN, Pp, Qq, YMIP, LO / Qq, LO % Qq>(smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
   } else {
     constexpr int MID = (LO + HI) / 2;
     if (idx < MID)
-      per_tree<RUN, Pp, Qq, LO, MID>(idx, smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
+      per_tree<RUN, Pp, Qq, YMIP, LO, MID>(idx, smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
     else
-      per_tree<RUN, Pp, Qq, MID, HI>(idx, smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
+      per_tree<RUN, Pp, Qq, YMIP, MID, HI>(idx, smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
   }
 }
 
@@ -259,7 +259,7 @@ constexpr int kPhaseShift = 16;
 // both rows of every stage.  z-maxima stay in registers and are folded into
 // zmip at the end of the job; each row's y-max over the run goes to ymip
 // right away.  Returns false when a bounded wait gave up.
-template <int RUN, int Pp, int Qq>
+template <int RUN, int Pp, int Qq, bool YMIP>
 __device__ __forceinline__ bool per_consume(const FastJob& jb, const PerRing& r, int& g, unsigned* err, int i,
                                             int lane) {
   using namespace per;
@@ -307,10 +307,11 @@ __device__ __forceinline__ bool per_consume(const FastJob& jb, const PerRing& r,
 #pragma unroll
     for (int c = 0; c < kXL; ++c) ym0[c] = ym1[c] = 0.0f;
     const uint32_t wof0 = tab0 + (uint32_t)(h * RUN * 8);
-    per_tree<RUN, Pp, Qq, 0, Qq * Qq>(c0 * Qq + c1, smem, row0 + rr0.y * pitch, row1 + rr1.y * pitch, wof0,
+    per_tree<RUN, Pp, Qq, YMIP, 0, Qq * Qq>(c0 * Qq + c1, smem, row0 + rr0.y * pitch, row1 + rr1.y * pitch, wof0,
                                       wof0 + (uint32_t)sizeof(FastRow), zmax, ym0, ym1);
     __syncwarp();
     if (lane == 0) mbar_arrive(&r.sfree()[s]);
+    if constexpr (!YMIP) continue;
     float* ymip = lds_volatile_ptr(&js->ymip);
     if (ymip) {
       const int nx = lds_volatile_s32(&js->nx);

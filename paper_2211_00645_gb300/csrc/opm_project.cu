@@ -66,6 +66,7 @@ struct ProjArgs {
 // (units of 256 rows of one j-tile at one x-tile).  The stage counter
 // carries on across a CTA's units, so the next unit's slabs stream in while
 // the current one drains.
+template <bool YMIP>
 __global__ void __launch_bounds__(kThreads, 4)
 k_project_fast(const __grid_constant__ CUtensorMap tmap, const ProjArgs args) {
   const PlanView& v = args.v;
@@ -106,7 +107,7 @@ k_project_fast(const __grid_constant__ CUtensorMap tmap, const ProjArgs args) {
     if (warp == 0)
       ok = fast_produce(jb, ring, g, v.err, lane);
     else
-      ok = fast_consume(jb, ring, g, v.err, warp - 1, lane);
+      ok = fast_consume<YMIP>(jb, ring, g, v.err, warp - 1, lane);
   }
   if (warp == 0) fast_drain(ring, g, ok, v.err);
 }
@@ -114,7 +115,7 @@ k_project_fast(const __grid_constant__ CUtensorMap tmap, const ProjArgs args) {
 // Periodic kernel (opm_periodic.cuh): the fast kernel's schedule, tables
 // and TMA ring for plans with pixel/step = Pp/Qq, with straight-line compute
 // warps per phase pair; MINB CTAs per SM, S ring stages.
-template <int Pp, int Qq, int RUN, int MINB, int S>
+template <int Pp, int Qq, int RUN, int MINB, int S, bool YMIP>
 __global__ void __launch_bounds__(per::Cfg<RUN>::kThreads, MINB)
 k_project_per(const __grid_constant__ CUtensorMap tmap, const ProjArgs args) {
   const PlanView& v = args.v;
@@ -155,7 +156,7 @@ k_project_per(const __grid_constant__ CUtensorMap tmap, const ProjArgs args) {
     if (warp == 0)
       ok = per_produce(jb, ring, g, v.err, lane);
     else
-      ok = per_consume<RUN, Pp, Qq>(jb, ring, g, v.err, warp - 1, lane);
+      ok = per_consume<RUN, Pp, Qq, YMIP>(jb, ring, g, v.err, warp - 1, lane);
   }
   if (warp == 0) per_drain(ring, g, ok, v.err);
 }
@@ -264,15 +265,16 @@ opm_status launch_per_f(const opm_plan* p, const CUtensorMap& map, const ProjArg
   if constexpr (F < kNumFamilies) {
     if (p->family - 1 != F) return launch_per_f<F + 1>(p, map, args, s, grid_div);
     constexpr int Pp = kFamilies[F].p, Qq = kFamilies[F].q;
-    static int done[64] = {0};
-    opm_status st = prepare_kernel(k_project_per<Pp, Qq, kPerRun, kPerCtasPerSm, kPerStages>, p->device, done);
+    static int done[2][64] = {{0}};
+    const auto kern = args.ymip ? k_project_per<Pp, Qq, kPerRun, kPerCtasPerSm, kPerStages, true>
+                                : k_project_per<Pp, Qq, kPerRun, kPerCtasPerSm, kPerStages, false>;
+    opm_status st = prepare_kernel(kern, p->device, done[args.ymip != nullptr]);
     if (st != OPM_OK) return st;
     const PlanView& v = p->view;
     const int full = std::min(v.nunits, v.nlists);
     if (full == 0) return OPM_OK;
     const int grid = std::max(1, full / std::max(1, grid_div));
-    k_project_per<Pp, Qq, kPerRun, kPerCtasPerSm, kPerStages>
-        <<<grid, per::Cfg<kPerRun>::kThreads, per::total(kPerStages, args.P), s>>>(map, args);
+    kern<<<grid, per::Cfg<kPerRun>::kThreads, per::total(kPerStages, args.P), s>>>(map, args);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? OPM_OK : cuda_fail(e, "launch k_project_per");
   } else {
@@ -288,16 +290,17 @@ opm_status launch_per(const opm_plan* p, const CUtensorMap& map, const ProjArgs&
 
 opm_status launch_fast(const opm_plan* p, const CUtensorMap& map, const ProjArgs& args, cudaStream_t s,
                        int grid_div) {
-  static int done[64] = {0};
+  static int done[2][64] = {{0}};
   if (p->family) return launch_per(p, map, args, s, grid_div);
-  opm_status st = prepare_kernel(k_project_fast, p->device, done);
+  const auto kern = args.ymip ? k_project_fast<true> : k_project_fast<false>;
+  opm_status st = prepare_kernel(kern, p->device, done[args.ymip != nullptr]);
   if (st != OPM_OK) return st;
   const PlanView& v = p->view;
   if (!v.units || !v.lists) return fail(OPM_ERR_INTERNAL, "plan has no fast-kernel schedule");
   const int full = std::min(v.nunits, v.nlists);
   if (full == 0) return OPM_OK;
   const int grid = std::max(1, full / std::max(1, grid_div));
-  k_project_fast<<<grid, kThreads, fast::total(args.P), s>>>(map, args);
+  kern<<<grid, kThreads, fast::total(args.P), s>>>(map, args);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? OPM_OK : cuda_fail(e, "launch k_project_fast");
 }

@@ -350,8 +350,10 @@ __device__ __forceinline__ float* lds_volatile_ptr(float* const* p) {
 
 // Compute warp cw (0..3): columns j0 + 8cw .. + 7 of the job, both rows of
 // every stage; z-maxima in registers, folded into zmip at the end of the job;
-// the y-max of each stage folded into ymip after the 4-warp rendezvous.
+// the y-max of each stage folded into ymip after the 4-warp rendezvous (YMIP;
+// without it a stage is free as soon as its four warps have read it).
 // Returns false when a bounded wait gave up.
+template <bool YMIP>
 __device__ __forceinline__ bool fast_consume(const FastJob& jb, const FastRing& r, int& g, unsigned* err,
                                              int cw, int lane) {
   using namespace fast;
@@ -416,6 +418,7 @@ __device__ __forceinline__ bool fast_consume(const FastJob& jb, const FastRing& 
       upk(fma2(w1, st1.d[1], st1.a[1]), v1[2], v1[3]);
 #pragma unroll
       for (int c = 0; c < kVec; ++c) zmax[j][c] = max3(zmax[j][c], v0[c], v1[c]);
+      if constexpr (!YMIP) continue;
       if (j & 1) {
 #pragma unroll
         for (int c = 0; c < kVec; ++c) {
@@ -429,6 +432,11 @@ __device__ __forceinline__ bool fast_consume(const FastJob& jb, const FastRing& 
           vp1[c] = v1[c];
         }
       }
+    }
+    if constexpr (!YMIP) {
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&r.ydone()[s]);
+      continue;
     }
     // y-max: combine the four warps in shared memory, then each warp folds
     // 32 columns of both rows into the global y-MIP
