@@ -111,11 +111,12 @@ __global__ void k_batch_zero(const unsigned char* __restrict__ wl) {
   }
 }
 
+template <int S>
 __global__ void __launch_bounds__(kThreads, 4)
 k_batch_fast(const unsigned char* __restrict__ wl, int Pl, unsigned* err) {
   extern __shared__ __align__(128) unsigned char smem[];
   const BatchHdr* hdr = reinterpret_cast<const BatchHdr*>(wl);
-  const FastRing ring = fast_ring(smem, Pl);
+  const FastRing<S> ring = fast_ring<S>(smem, Pl);
   fast_ring_init(ring);
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -293,7 +294,7 @@ k_batch_gen(const unsigned char* __restrict__ wl) {
 }
 
 // Shared memory of a batch launch for slab depth Pl (family 0: k_batch_fast).
-size_t batch_smem(int Pl, int family) { return family ? per::total(kPerStages, Pl) : fast::total(Pl); }
+size_t batch_smem(int Pl, int family) { return family ? per::total(kPerStages, Pl) : fast::total(fast_stages(Pl), Pl); }
 size_t batch_gen_smem() { return direct::smem_bytes<uint16_t>(direct::kJumpSlots); }
 
 PFN_cuTensorMapEncodeTiled_v12000 batch_encode_fn() {
@@ -550,6 +551,17 @@ void launch_batch_per(const unsigned char* dev_wl, const WorkList& wl, int grid,
   }
 }
 
+// The fast kernel with the ring depth of slab depth Pl.
+using BatchFast = void (*)(const unsigned char*, int, unsigned*);
+BatchFast batch_fast_kernel(int Pl) {
+  switch (fast_stages(Pl)) {
+    case 6: return k_batch_fast<6>;
+    case 5: return k_batch_fast<5>;
+    case 4: return k_batch_fast<4>;
+    default: return k_batch_fast<3>;
+  }
+}
+
 // Zero kernel, then the fast (or periodic) kernel's `grid` persistent CTAs
 // when the list has fast units, then the general kernel's `ggrid` CTAs when
 // it has general units, all on `s`.
@@ -562,7 +574,7 @@ cudaError_t launch_worklist(const unsigned char* dev_wl, const WorkList& wl, int
     if (wl.family)
       launch_batch_per<0>(dev_wl, wl, grid, err, s);
     else
-      k_batch_fast<<<grid, kThreads, fast::total(wl.Pl), s>>>(dev_wl, wl.Pl, err);
+      batch_fast_kernel(wl.Pl)<<<grid, kThreads, batch_smem(wl.Pl, 0), s>>>(dev_wl, wl.Pl, err);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -612,7 +624,10 @@ cudaError_t set_per_attrs(int smem_optin) {
 }
 
 cudaError_t set_fast_attrs(int smem_optin) {
-  cudaError_t e = set_kernel_smem(k_batch_fast, smem_optin);
+  cudaError_t e = set_kernel_smem(k_batch_fast<6>, smem_optin);
+  if (e == cudaSuccess) e = set_kernel_smem(k_batch_fast<5>, smem_optin);
+  if (e == cudaSuccess) e = set_kernel_smem(k_batch_fast<4>, smem_optin);
+  if (e == cudaSuccess) e = set_kernel_smem(k_batch_fast<3>, smem_optin);
   if (e == cudaSuccess) e = set_kernel_smem(k_batch_gen, smem_optin);
   return e == cudaSuccess ? set_per_attrs<0>(smem_optin) : e;
 }

@@ -65,6 +65,19 @@ struct Family {
 };
 constexpr Family kFamilies[] = {{1, 3}, {1, 2}};
 constexpr int kNumFamilies = (int)(sizeof(kFamilies) / sizeof(kFamilies[0]));
+// Ring depth of the fast kernel for slab depth P: the deepest of 6 .. 3 stages
+// (two rows each) that still lets four of its CTAs into an SM's 228 KB of shared
+// memory (1 KB of it per CTA is the system's).  A fifth CTA's worth of rows in
+// flight is worth less than the fourth CTA: 200 x 512 x 2048 at 45 deg, step
+// 0.2, pixel 0.115 (21 planes), z + y: 203 us with 6 stages (3 CTAs per SM, the
+// schedule's fourth list a second wave), 162 with 4; 1024 columns at pixel / step 0.7 100 -> 77, 0.92 83 -> 68.
+constexpr int kFastStages[] = {6, 5, 4, 3};
+constexpr int fast_ring_bytes(int S, int P) { return S * (2 * P * 256 + 2 * 288 + 2 * 512 + 24) + 192; }
+constexpr int fast_stages(int P) {
+  for (int S : kFastStages)
+    if (4 * (fast_ring_bytes(S, P) + 1024) <= 228 * 1024) return S;
+  return 3;
+}
 constexpr int kPerRun = 32;       // columns j per compute warp of the periodic kernel
 constexpr int kPerCtasPerSm = 4;  // its persistent CTAs per SM
 constexpr int kPerStages = 6;     // its TMA ring depth

@@ -66,12 +66,12 @@ struct ProjArgs {
 // (units of 256 rows of one j-tile at one x-tile).  The stage counter
 // carries on across a CTA's units, so the next unit's slabs stream in while
 // the current one drains.
-template <bool YMIP>
+template <bool YMIP, int S>
 __global__ void __launch_bounds__(kThreads, 4)
 k_project_fast(const __grid_constant__ CUtensorMap tmap, const ProjArgs args) {
   const PlanView& v = args.v;
   extern __shared__ __align__(128) unsigned char smem[];
-  const FastRing ring = fast_ring(smem, args.P);
+  const FastRing<S> ring = fast_ring<S>(smem, args.P);
   fast_ring_init(ring);
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -288,21 +288,33 @@ opm_status launch_per(const opm_plan* p, const CUtensorMap& map, const ProjArgs&
   return launch_per_f<0>(p, map, args, s, grid_div);
 }
 
-opm_status launch_fast(const opm_plan* p, const CUtensorMap& map, const ProjArgs& args, cudaStream_t s,
-                       int grid_div) {
+template <int S>
+opm_status launch_fast_s(const opm_plan* p, const CUtensorMap& map, const ProjArgs& args, cudaStream_t s,
+                         int grid_div) {
+  static_assert(fast_ring_bytes(S, 14) == (int)fast::total(S, 14), "the plan's arithmetic of the ring");
   static int done[2][64] = {{0}};
-  if (p->family) return launch_per(p, map, args, s, grid_div);
-  const auto kern = args.ymip ? k_project_fast<true> : k_project_fast<false>;
+  const auto kern = args.ymip ? k_project_fast<true, S> : k_project_fast<false, S>;
   opm_status st = prepare_kernel(kern, p->device, done[args.ymip != nullptr]);
   if (st != OPM_OK) return st;
   const PlanView& v = p->view;
-  if (!v.units || !v.lists) return fail(OPM_ERR_INTERNAL, "plan has no fast-kernel schedule");
   const int full = std::min(v.nunits, v.nlists);
   if (full == 0) return OPM_OK;
   const int grid = std::max(1, full / std::max(1, grid_div));
-  kern<<<grid, kThreads, fast::total(args.P), s>>>(map, args);
+  kern<<<grid, kThreads, fast::total(S, args.P), s>>>(map, args);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? OPM_OK : cuda_fail(e, "launch k_project_fast");
+}
+
+opm_status launch_fast(const opm_plan* p, const CUtensorMap& map, const ProjArgs& args, cudaStream_t s,
+                       int grid_div) {
+  if (p->family) return launch_per(p, map, args, s, grid_div);
+  if (!p->view.units || !p->view.lists) return fail(OPM_ERR_INTERNAL, "plan has no fast-kernel schedule");
+  switch (fast_stages(args.P)) {
+    case 6: return launch_fast_s<6>(p, map, args, s, grid_div);
+    case 5: return launch_fast_s<5>(p, map, args, s, grid_div);
+    case 4: return launch_fast_s<4>(p, map, args, s, grid_div);
+    default: return launch_fast_s<3>(p, map, args, s, grid_div);
+  }
 }
 
 template <typename T, bool VEC, bool SUM, bool ARG>
@@ -351,7 +363,7 @@ opm_status launch_project(const opm_plan* p, const void* raw, opm_dtype in_t, fl
   // the TMA kernels: uint16 rows on 16 bytes, z-MIP and / or y-MIP only
   const bool fast = u16 && !zsum && !argz && p->fast_ok && v.frow && !p->force_generic && encode_fn() != nullptr &&
                     (uintptr_t)raw % 16 == 0 && (size_t)v.ncols * 2 % 16 == 0 &&
-                    (int)(p->family ? per::total(kPerStages, P) : fast::total(P)) <= smax;
+                    (int)(p->family ? per::total(kPerStages, P) : fast::total(fast_stages(P), P)) <= smax;
 
   // initial values of the atomically combined outputs
   float* zinit = fast ? zmip : nullptr;

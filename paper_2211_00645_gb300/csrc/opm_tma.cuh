@@ -17,7 +17,6 @@ constexpr int kJT = kTileJ / kNW;    // columns j per compute warp (8)
 constexpr int kThreads = 32 * (kNW + 1);
 constexpr int kVec = 4;              // columns x per lane
 constexpr int kX = 32 * kVec;        // columns x per CTA
-constexpr int kStagesFast = 6;       // TMA ring depth, fast kernel
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s: a launch takes < 10 ms
 
 static_assert(kJT * kNW == kTileJ, "tile");
@@ -204,15 +203,14 @@ __device__ __forceinline__ void stream_step_u16(StreamPF& st, const unsigned cha
 // themselves, 32 columns per warp, after an mbarrier rendezvous.
 namespace fast {
 
-constexpr int S = kStagesFast;
-
-__host__ __device__ inline size_t slab_row_bytes(int P) { return (size_t)P * kX * 2; }
-__host__ __device__ inline size_t stage_slab_bytes(int P) { return 2 * slab_row_bytes(P); }
-__host__ __device__ inline size_t off_tab(int P) { return S * stage_slab_bytes(P); }        // FastRow [S][2]
-__host__ __device__ inline size_t off_ybuf(int P) { return off_tab(P) + S * 2 * sizeof(FastRow); }  // float [S][2][kX]
-__host__ __device__ inline size_t off_bar(int P) { return off_ybuf(P) + S * 2 * kX * 4; }
-__host__ __device__ inline size_t off_jobs(int P) { return off_bar(P) + 3 * S * 8; }  // JobS [kNW]
-__host__ __device__ inline size_t total(int P) { return off_jobs(P) + kNW * 48; }
+// Shared memory of a ring of S stages for slab depth P.
+__host__ __device__ constexpr size_t slab_row_bytes(int P) { return (size_t)P * kX * 2; }
+__host__ __device__ constexpr size_t stage_slab_bytes(int P) { return 2 * slab_row_bytes(P); }
+__host__ __device__ constexpr size_t off_tab(int S, int P) { return S * stage_slab_bytes(P); }                  // FastRow [S][2]
+__host__ __device__ constexpr size_t off_ybuf(int S, int P) { return off_tab(S, P) + S * 2 * sizeof(FastRow); }  // float [S][2][kX]
+__host__ __device__ constexpr size_t off_bar(int S, int P) { return off_ybuf(S, P) + S * 2 * kX * 4; }
+__host__ __device__ constexpr size_t off_jobs(int S, int P) { return off_bar(S, P) + 3 * S * 8; }  // JobS [kNW]
+__host__ __device__ constexpr size_t total(int S, int P) { return off_jobs(S, P) + kNW * 48; }
 
 }  // namespace fast
 
@@ -251,30 +249,33 @@ static_assert(sizeof(JobS) == 48, "JobS layout");
 // The ring in shared memory, laid out for slab depth Pl (>= every job's P).
 // Region addresses are recomputed from the base on use rather than held in
 // registers.
+template <int S>
 struct FastRing {
   unsigned char* base;
   int Pl;
-  __device__ __forceinline__ FastRow* tab() const { return reinterpret_cast<FastRow*>(base + fast::off_tab(Pl)); }
-  __device__ __forceinline__ float* ybuf() const { return reinterpret_cast<float*>(base + fast::off_ybuf(Pl)); }
+  __device__ __forceinline__ FastRow* tab() const { return reinterpret_cast<FastRow*>(base + fast::off_tab(S, Pl)); }
+  __device__ __forceinline__ float* ybuf() const { return reinterpret_cast<float*>(base + fast::off_ybuf(S, Pl)); }
   // producer -> consumers: slabs and tables landed
-  __device__ __forceinline__ uint64_t* full() const { return reinterpret_cast<uint64_t*>(base + fast::off_bar(Pl)); }
+  __device__ __forceinline__ uint64_t* full() const { return reinterpret_cast<uint64_t*>(base + fast::off_bar(S, Pl)); }
   // consumers -> producer: slot free
-  __device__ __forceinline__ uint64_t* ydone() const { return full() + fast::S; }
+  __device__ __forceinline__ uint64_t* ydone() const { return full() + S; }
   // consumers -> consumers: y-max of the stage combined
-  __device__ __forceinline__ uint64_t* cdone() const { return full() + 2 * fast::S; }
+  __device__ __forceinline__ uint64_t* cdone() const { return full() + 2 * S; }
   // one per compute warp
-  __device__ __forceinline__ JobS* jobs() const { return reinterpret_cast<JobS*>(base + fast::off_jobs(Pl)); }
+  __device__ __forceinline__ JobS* jobs() const { return reinterpret_cast<JobS*>(base + fast::off_jobs(S, Pl)); }
 };
 
-__device__ __forceinline__ FastRing fast_ring(unsigned char* smem, int Pl) {
-  FastRing r;
+template <int S>
+__device__ __forceinline__ FastRing<S> fast_ring(unsigned char* smem, int Pl) {
+  FastRing<S> r;
   r.base = smem;
   r.Pl = Pl;
   return r;
 }
 
 // Whole CTA: barrier init and y-max buffer reset, then a CTA barrier.
-__device__ __forceinline__ void fast_ring_init(const FastRing& r) {
+template <int S>
+__device__ __forceinline__ void fast_ring_init(const FastRing<S>& r) {
   using namespace fast;
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
@@ -290,7 +291,8 @@ __device__ __forceinline__ void fast_ring_init(const FastRing& r) {
 
 // Producer warp: stage the job's rows.  `g` is the CTA's running stage
 // count (ring slot and phase), advanced by the job's stage count.
-__device__ __forceinline__ bool fast_produce(const FastJob& jb, const FastRing& r, int& g, unsigned* err,
+template <int S>
+__device__ __forceinline__ bool fast_produce(const FastJob& jb, const FastRing<S>& r, int& g, unsigned* err,
                                              int lane) {
   using namespace fast;
   const uint32_t pitch = kX * 2;
@@ -330,7 +332,8 @@ __device__ __forceinline__ bool fast_produce(const FastJob& jb, const FastRing& 
 
 // Producer warp, after its last job: the CTA's shared memory must outlive
 // every copy it issued (bounded wait on the last S stages).
-__device__ __forceinline__ void fast_drain(const FastRing& r, int g, bool ok, unsigned* err) {
+template <int S>
+__device__ __forceinline__ void fast_drain(const FastRing<S>& r, int g, bool ok, unsigned* err) {
   using namespace fast;
   for (int q = max(0, g - S); q < g; ++q)
     if (!mbar_wait(&r.full()[q % S], (q / S) & 1, err, ok ? kWaitLimitNs : 50000000ull)) break;
@@ -353,8 +356,8 @@ __device__ __forceinline__ float* lds_volatile_ptr(float* const* p) {
 // the y-max of each stage folded into ymip after the 4-warp rendezvous (YMIP;
 // without it a stage is free as soon as its four warps have read it).
 // Returns false when a bounded wait gave up.
-template <bool YMIP>
-__device__ __forceinline__ bool fast_consume(const FastJob& jb, const FastRing& r, int& g, unsigned* err,
+template <bool YMIP, int S>
+__device__ __forceinline__ bool fast_consume(const FastJob& jb, const FastRing<S>& r, int& g, unsigned* err,
                                              int cw, int lane) {
   using namespace fast;
   const uint32_t pitch = kX * 2;
@@ -396,7 +399,7 @@ __device__ __forceinline__ bool fast_consume(const FastJob& jb, const FastRing& 
     StreamPF st0, st1;
     stream_reset_u16(st0, smem, lane0, pitch, r0.ofirst);
     stream_reset_u16(st1, smem, lane1, pitch, r1.ofirst);
-    const uint32_t w0off = (uint32_t)(off_tab(r.Pl) + (s * 2 + 0) * sizeof(FastRow)) + cw * kJT * 8;
+    const uint32_t w0off = (uint32_t)(off_tab(S, r.Pl) + (s * 2 + 0) * sizeof(FastRow)) + cw * kJT * 8;
     const uint32_t w1off = w0off + (uint32_t)sizeof(FastRow);
 
     float ym0[kVec], ym1[kVec], vp0[kVec], vp1[kVec];
