@@ -65,8 +65,14 @@ constexpr size_t kOffItems = 256;
 struct BatchItemDev {  // 64-byte aligned through its tensor map
   CUtensorMap tmap;      // raw stack of the item, box {128, 1, P}
   const FastRow* frow;   // fast-kernel tables, [ntile][nz] (fast items)
-  const int* fnlo;       // [ntile][nz]
-  const Split* A;        // split tables and row bands (general items)
+  union {
+    const int* fnlo;        // [ntile][nz] (fast kernel)
+    const RowPair* pairs;   // row pairs, tile after tile (periodic kernel)
+  };
+  union {
+    const Split* A;         // split tables and row bands (general items)
+    const int* pair0;       // [ntile + 1] (periodic kernel)
+  };
   const Split* B;
   const Band* band;
   const uint16_t* raw;   // sample (0, 0, 0) and pitches in elements (general items)
@@ -209,7 +215,7 @@ k_batch_per(const unsigned char* __restrict__ wl, int Pl, unsigned* err) {
     jb.nz = it->nz;
     jb.nx = it->nx;
     jb.rows = it->frow + (size_t)un.jt * jb.nz;
-    jb.nlos = it->fnlo + (size_t)un.jt * jb.nz;
+    jb.pairs = it->pairs + it->pair0[un.jt];
     jb.zmip = it->zmip;
     jb.ymip = it->ymip;
     jb.j0 = tile_j0(un.jt, it->ny);
@@ -349,19 +355,33 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
   if (!items && n_items > 0) return fail(OPM_ERR_INVALID_ARG, "items is NULL");
   if (kchunk < 0) return fail(OPM_ERR_INVALID_ARG, "kchunk must be >= 0");
   if (!batch_encode_fn()) return fail(OPM_ERR_UNSUPPORTED, "cuTensorMapEncodeTiled is unavailable");
+  // The fast items' kernel: the periodic one (32 or 16 columns j per warp)
+  // needs one family shared by all of them, else the fast kernel runs them.
+  // Items are validated by the pass below.
+  auto is_fast = [&](const opm_batch_item& it) {
+    return it.plan && !gen_all && plan_fast_ok(it.plan) && !it.zsum && !it.argz && (it.zmip || it.ymip);
+  };
+  int family = -1;
+  for (int i = 0; i < n_items; ++i)
+    if (is_fast(items[i])) family = (family < 0 || family == items[i].plan->family) ? items[i].plan->family : 0;
+  if (family < 0 || shape == OPM_SHAPE_FAST_J8X4) family = 0;
+  if (!gen_all) {
+    if (shape == OPM_SHAPE_AUTO) shape = family ? OPM_SHAPE_PER_J32X2 : OPM_SHAPE_FAST_J8X4;
+    if (!family) shape = OPM_SHAPE_FAST_J8X4;
+    // 16-column runs exist for the first family only; the others run 32
+    if (shape == OPM_SHAPE_PER_J16X2 && family != 1) shape = OPM_SHAPE_PER_J32X2;
+  }
   if (kchunk == 0) {
     // The single-stack rule: the largest of kChunkRows .. kMinChunkRows rows
     // that gives the CTA lists at least kUnitsPerList fast units each, without
-    // going past the unit capacity.  Items are validated by the pass below.
+    // going past the unit capacity.
     auto nfast_units = [&](int rows) {
       int64_t n = 0;
       for (int i = 0; i < n_items; ++i) {
-        const opm_batch_item& it = items[i];
-        const opm_plan* p = it.plan;
-        if (!p || gen_all || !plan_fast_ok(p) || it.zsum || it.argz || (!it.zmip && !it.ymip)) continue;
+        if (!is_fast(items[i])) continue;
+        const opm_plan* p = items[i].plan;
         const int64_t xtiles = (p->nx + kX - 1) / kX;
-        for (const Band& bd : p->hBand)
-          if (bd.lo < bd.hi) n += xtiles * ((bd.hi - 1) / rows - bd.lo / rows + 1);
+        for (const Band& bd : p->hBand) n += xtiles * band_units(bd, rows);
       }
       return n;
     };
@@ -380,8 +400,17 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
   int* hglists = reinterpret_cast<int*>(stage + off_glists);
   WorkUnit* hunits = reinterpret_cast<WorkUnit*>(stage + off_units);
   int64_t nunits = 0;
+  bool pairs_fit = family > 0;  // room for every unit of the row pairs
+  if (family) {
+    int64_t n = 0;
+    for (int i = 0; i < n_items; ++i)
+      if (is_fast(items[i]))
+        for (int jt = 0; jt < (int)items[i].plan->hBand.size(); ++jt)
+          n += (items[i].plan->nx + kX - 1) / kX * pair_units(items[i].plan, jt, kchunk);
+    pairs_fit = n <= max_units;
+  }
   bool fine = false;  // room for every general item's single pieces
-  int Pl = 2, Pg = 2, nseg = 0, family = -1, nfast = 0;
+  int Pl = 2, Pg = 2, nseg = 0, nfast = 0;
   // first pass: fast items' units; second pass: general items' units after them
   for (int pass = 0; pass < 2; ++pass) {
     for (int i = 0; i < n_items; ++i) {
@@ -414,8 +443,13 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
           return fail(OPM_ERR_CUDA, "item " + std::to_string(i) + ": cuTensorMapEncodeTiled failed (" +
                                         std::to_string((int)cr) + ")");
         d.frow = p->view.frow;
-        d.fnlo = p->view.fnlo;
-        d.A = p->view.A;
+        if (family && is_fast(it)) {
+          d.pairs = p->view.pairs;
+          d.pair0 = p->view.pair0;
+        } else {
+          d.fnlo = p->view.fnlo;
+          d.A = p->view.A;
+        }
         d.B = p->view.B;
         d.band = p->view.band;
         d.raw = it.raw;
@@ -441,7 +475,6 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
       if (!zout && !it.ymip) continue;
       if (fast) {
         Pl = std::max(Pl, p->P);
-        family = (family < 0 || family == p->family) ? p->family : 0;
         if (it.zmip) hsegs[nseg++] = BatchSeg{it.zmip, (long long)(p->ny * p->nx)};
       } else {
         Pg = std::max(Pg, p->P);
@@ -452,7 +485,6 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
       const int piece = fine ? direct::cta_cols(hitems[i].wr) : kTileJ;
       for (int jt = 0; jt < jtiles; ++jt) {
         const Band bd = p->hBand[jt];
-        const int step = kchunk, cstart = (bd.lo / kchunk) * kchunk;
         const bool empty_unit = !fast && zout && bd.lo >= bd.hi;
         if (!fast) {
           if (bd.lo >= bd.hi && !empty_unit) continue;
@@ -465,15 +497,16 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
           }
           continue;
         }
-        for (int c0 = cstart; c0 < bd.hi; c0 += step) {
-          const int ks = std::max(bd.lo, c0), ke = std::min(bd.hi, c0 + step);
-          if (ks >= ke) continue;
+        const int64_t n = pairs_fit ? pair_units(p, jt, kchunk) : band_units(bd, kchunk);
+        for (int64_t u = 0; u < n; ++u) {
+          const Band r = unit_range(p, jt, kchunk, family, u, n);
+          if (r.lo >= r.hi) continue;
           if (nunits + xtiles > max_units)
             return fail(OPM_ERR_UNSUPPORTED, std::string("the items need more than the ") + limit_what +
                                                  "'s limit of " + std::to_string(max_units) +
                                                  " work units (raise kchunk or split)");
           for (int xt = 0; xt < xtiles; ++xt)
-            hunits[nunits++] = WorkUnit{i, xt, jt, ks, ke, 0, 0, 0};
+            hunits[nunits++] = WorkUnit{i, xt, jt, r.lo, r.hi, 0, 0, 0};
         }
       }
     }
@@ -510,22 +543,9 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
   out->n_segs = nseg;
   out->n_lists = nlists;
   out->Pl = Pl;
-  // the fast items' kernel: the periodic one (32 or 16 columns j per warp)
-  // needs one family shared by all of them, else the fast kernel runs them
-  if (family < 0) family = 0;
-  if (gen_all) {
-    family = 0;
-  } else if (shape == OPM_SHAPE_AUTO) {
-    shape = family ? OPM_SHAPE_PER_J32X2 : OPM_SHAPE_FAST_J8X4;
-  } else if (shape == OPM_SHAPE_FAST_J8X4 || family == 0) {
-    shape = OPM_SHAPE_FAST_J8X4;
-    family = 0;
-  }
   out->family = family;
   out->n_gunits = ngen;
   out->Pg = Pg;
-  // 16-column runs exist for the first family only; the others run 32
-  if (shape == OPM_SHAPE_PER_J16X2 && family != 1) shape = OPM_SHAPE_PER_J32X2;
   out->run = shape == OPM_SHAPE_PER_J16X2 ? 16 : kPerRun;
   out->shape = shape;
   return OPM_OK;

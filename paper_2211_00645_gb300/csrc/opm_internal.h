@@ -54,6 +54,12 @@ struct __align__(16) FastRow {
 };
 static_assert(sizeof(FastRow) == 288, "FastRow is copied as 288 bytes");
 
+// Two camera rows of one j-tile that step through their planes alike (the same
+// phase of a periodic plan), and the first plane of each.
+struct __align__(16) RowPair {
+  int k0, k1, n0, n1;
+};
+
 // Plans whose lower plane advances by p/q planes per output column j
 // (pixel/step = p/q) take the periodic live-view kernel (opm_periodic.cuh):
 // along a camera row, the 32 columns of a tile sit on planes
@@ -103,6 +109,8 @@ struct PlanView {
   unsigned* err;      // error word
   const FastRow* frow;  // [ntile][nz] fast-kernel tables (NULL unless fast_ok)
   const int* fnlo;      // [ntile][nz] first staged plane of each (tile, row)
+  const RowPair* pairs;   // row pairs of every tile of a periodic plan, tile after tile
+  const int* pair0;       // [ntile + 1] first pair of each tile
   const WorkUnit* units;  // fast-kernel work units, list by list (NULL unless fast_ok)
   const int* lists;       // [nlists + 1] first unit of each persistent CTA's list
   int nunits, nlists;
@@ -129,6 +137,8 @@ struct opm_plan {
   std::vector<float> hYinit;
   std::vector<opm::FastRow> hFrow;  // fast-kernel tables (when fast_ok)
   std::vector<int> hFnlo;
+  std::vector<opm::RowPair> hPairs;  // periodic plans: the band's rows of every tile, paired by phase
+  std::vector<int> hPair0;           // [ntile + 1]
   std::vector<opm::WorkUnit> hUnits;  // fast-kernel schedule (when fast_ok and a device exists)
   std::vector<int> hLists;
   int device;        // -1: created without a device
@@ -193,4 +203,30 @@ __device__ __forceinline__ void plane_weight(Split a, Split b, int linear,
 namespace opm {
 // Fast-projection eligibility and slab depth of a plan (host side).
 inline bool plan_fast_ok(const opm_plan* p) { return p && p->fast_ok && p->view.frow != nullptr; }
+
+// Units of a j-tile's row band for `rows` rows per unit (cut at multiples of
+// `rows`).
+inline int64_t band_units(const Band& bd, int rows) {
+  return bd.lo < bd.hi ? (bd.hi - 1) / rows - bd.lo / rows + 1 : 0;
+}
+// As many units as j-tile jt takes in a periodic schedule: the pairing may add
+// a few rows to the band's.
+inline int64_t pair_units(const opm_plan* p, int jt, int rows) {
+  const int64_t all = 2 * (int64_t)(p->hPair0[jt + 1] - p->hPair0[jt]), c = rows + (rows & 1);
+  return (all + c - 1) / c;
+}
+// Row range [ks, ke) of unit u of n, n = band_units of j-tile jt for the fast
+// kernel; for a periodic one (family > 0) two rows for each of the tile's
+// row pairs, `rows` at a time and what is left to the last (units of even
+// length are balanced worse: live view 143 against 136 us).  An empty range is
+// no unit.
+inline Band unit_range(const opm_plan* p, int jt, int rows, int family, int64_t u, int64_t n) {
+  if (family) {
+    const int64_t all = 2 * (int64_t)(p->hPair0[jt + 1] - p->hPair0[jt]), c = rows + (rows & 1);
+    return Band{(int32_t)std::min(all, u * c), (int32_t)(u == n - 1 ? all : std::min(all, (u + 1) * c))};
+  }
+  const Band bd = p->hBand[jt];
+  const int32_t c0 = (bd.lo / rows + (int32_t)u) * rows;
+  return Band{std::max(bd.lo, c0), std::min(bd.hi, c0 + rows)};
+}
 }  // namespace opm

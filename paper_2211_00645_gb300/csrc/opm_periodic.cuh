@@ -13,9 +13,24 @@
 // first and last column of each plane interval (along a row the voxels of
 // one interval are a + w (b - a) with w increasing in j, and a correctly
 // rounded FMA is monotone in w; the plan checks that the weights increase
-// inside every interval).  The arithmetic is that of every other kernel of
-// the library (the plan's weights, FMA on the exact plane difference), so
-// the outputs are the same bit for bit.
+// inside every interval).  Every q-th column has the same weight, bit for bit
+// (the plan builds its column table from the exact ratio and checks it), so a
+// row's q weights stay in registers.  The arithmetic is that of every other
+// kernel of the library (the plan's weights, FMA on the exact plane
+// difference), so the outputs are the same bit for bit.
+//
+// The two rows of a stage have the same phase: the plan pairs every tile's
+// rows by phase (RowPair), and a unit is a run of such pairs.  That leaves q
+// bodies of code instead of q^2, 18 KB for q = 3.  Straight-line code starves
+// the schedulers once the bodies in use outgrow the instruction caches (a
+// probe of independent maxima: three bodies of 4 KB run at full rate, six at a
+// quarter to two thirds of it), and with rows paired in order six of nine 6 KB
+// bodies were in use.  What bounds it now is dispatch: packed FMAs, adds and
+// 3-input maxima take two to three cycles each, and more warps do not help (5
+// CTAs per SM: 145 us below).  us, rows in order with a weight pair per column
+// -> this: 200 x 512 x 2048 (35 deg, step 0.3, pixel 0.1) 149 -> 136, 1024 of
+// its columns 86 -> 79, 256 columns 40 -> 35; six two-channel stacks of the
+// serving mix 863 -> 754; 1/2 (step 0.2) 155.5 -> 155.
 //
 // CTA: one producer warp (TMA ring of two camera rows per stage, as in
 // opm_tma.cuh) and two compute warps.  Each compute warp owns all 32 columns
@@ -49,15 +64,15 @@ struct Cfg {
 __host__ __device__ inline size_t off_tab(int S, int P) { return S * fast::stage_slab_bytes(P); }  // FastRow [S][2]
 __host__ __device__ inline size_t off_bar(int S, int P) { return off_tab(S, P) + S * 2 * sizeof(FastRow); }
 __host__ __device__ inline size_t off_jobs(int S, int P) { return off_bar(S, P) + 2 * S * 8; }  // JobP [kMaxCW]
-__host__ __device__ inline size_t total(int S, int P) { return off_jobs(S, P) + kMaxCW * 48; }
+__host__ __device__ inline size_t off_rows(int S, int P) { return off_jobs(S, P) + kMaxCW * 48; }  // int2 [S]: camera rows
+__host__ __device__ inline size_t total(int S, int P) { return off_rows(S, P) + S * 8; }
 
 struct JobP {  // a compute warp's job fields, parked in shared memory
   float* zmip;
   float* ymip;
-  int nx, nz, j0, xbase;
-  int k0g;   // camera row of stage g is k0g + 2 g
+  int nx, j0, xbase;
   int gend;  // stage count at the end of the job
-  int pad[2];
+  int pad[4];
 };
 static_assert(sizeof(JobP) == 48, "JobP layout");
 
@@ -93,6 +108,8 @@ struct PerRing {
   __device__ __forceinline__ per::JobP* jobs() const {
     return reinterpret_cast<per::JobP*>(base + per::off_jobs(S, Pl));
   }
+  // camera rows of each stage
+  __device__ __forceinline__ int2* rows() const { return reinterpret_cast<int2*>(base + per::off_rows(S, Pl)); }
 };
 
 __device__ __forceinline__ PerRing per_ring(unsigned char* smem, int S, int Pl) {
@@ -115,39 +132,33 @@ __device__ __forceinline__ void per_ring_init(const PerRing& r, int ncw) {
   __syncthreads();
 }
 
-// Producer warp: stage the job's rows (two per stage) once the slot is free.
-// `g` is the CTA's running stage count, advanced by the job's stage count.
+// Producer warp: stage the job's row pairs once the slot is free.  `g` is the
+// CTA's running stage count, advanced by the job's stage count.
 __device__ __forceinline__ bool per_produce(const FastJob& jb, const PerRing& r, int& g, unsigned* err, int lane) {
   const uint32_t pitch = kX * 2;
   const int S = r.S;
-  const int nst = (jb.ke - jb.ks + 1) / 2;
-  int kbase = jb.ks;  // first staged planes of 32 rows per load, one group ahead
-  int ncur = jb.nlos[min(kbase + lane, jb.nz - 1)];
-  int nnext = jb.nlos[min(kbase + 32 + lane, jb.nz - 1)];
+  const RowPair* pairs = jb.pairs + jb.ks / 2;
+  const int nst = (jb.ke - jb.ks) / 2;
+  RowPair cur = pairs[min(lane, nst - 1)];  // 32 pairs per load, one group ahead
+  RowPair next = pairs[min(32 + lane, nst - 1)];
 #pragma unroll 1
   for (int it = 0; it < nst; ++it, ++g) {
     const int s = g % S;
     if (g >= S && !mbar_wait(&r.sfree()[s], ((g - S) / S) & 1, err)) return false;
-    int nlo[2];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int k = jb.ks + 2 * it + q;
-      if (k - kbase >= 32) {  // warp-uniform: rows advance in order
-        kbase += 32;
-        ncur = nnext;
-        nnext = jb.nlos[min(kbase + 32 + lane, jb.nz - 1)];
-      }
-      nlo[q] = __shfl_sync(0xffffffffu, ncur, k - kbase);
+    if (it > 0 && it % 32 == 0) {
+      cur = next;
+      next = pairs[min(it + 32 + lane, nst - 1)];
     }
+    const int k0 = __shfl_sync(0xffffffffu, cur.k0, it % 32), k1 = __shfl_sync(0xffffffffu, cur.k1, it % 32);
+    const int n0 = __shfl_sync(0xffffffffu, cur.n0, it % 32), n1 = __shfl_sync(0xffffffffu, cur.n1, it % 32);
     if (lane == 0) {
-      const int k0 = jb.ks + 2 * it;
-      const int k1 = k0 + 1;  // k1 == nz: a padding row, staged as TMA zero fill
       unsigned char* slab = r.base + s * fast::stage_slab_bytes(r.Pl);
+      r.rows()[s] = make_int2(k0, k1);
       mbar_arrive_tx(&r.full()[s], (unsigned)(2 * jb.P * pitch + 2 * sizeof(FastRow)));
-      tma_load_3d(slab, jb.tmap, &r.full()[s], jb.xbase, k0, nlo[0]);
-      tma_load_3d(slab + fast::slab_row_bytes(r.Pl), jb.tmap, &r.full()[s], jb.xbase, k1, k1 < jb.nz ? nlo[1] : 0);
+      tma_load_3d(slab, jb.tmap, &r.full()[s], jb.xbase, k0, n0);
+      tma_load_3d(slab + fast::slab_row_bytes(r.Pl), jb.tmap, &r.full()[s], jb.xbase, k1, n1);
       bulk_load(&r.tab()[s * 2 + 0], jb.rows + k0, sizeof(FastRow), &r.full()[s]);
-      bulk_load(&r.tab()[s * 2 + 1], jb.rows + min(k1, jb.nz - 1), sizeof(FastRow), &r.full()[s]);
+      bulk_load(&r.tab()[s * 2 + 1], jb.rows + k1, sizeof(FastRow), &r.full()[s]);
     }
     __syncwarp();
   }
@@ -166,11 +177,11 @@ __device__ __forceinline__ f2 lds_x2(const unsigned char* smem, uint32_t off) {
   return u16x2_to_f2(*reinterpret_cast<const uint32_t*>(smem + off));
 }
 
-// Both camera rows of a stage for one compute warp: a run of RUN columns,
-// row 0 at phase PH0 and row 1 at phase PH1.  off0 / off1: shared-memory
-// offset of this lane's 2 columns x in the tile's first plane of each row;
-// wof0 / wof1: the tile's (w, w) weight pairs of each row.
-template <int RUN, int Pp, int Qq, bool YMIP, int PH0, int PH1>
+// Both camera rows of a stage for one compute warp: a run of RUN columns, both
+// rows at phase PH.  off0 / off1: shared-memory offset of this lane's 2
+// columns x in the tile's first plane of each row; wof0 / wof1: the run's (w,
+// w) weight pairs of each row, of which the first Qq repeat.
+template <int RUN, int Pp, int Qq, bool YMIP, int PH>
 __device__ __forceinline__ void per_pair(const unsigned char* __restrict__ smem, uint32_t off0, uint32_t off1,
                                          uint32_t wof0, uint32_t wof1, float (&zmax)[RUN][per::kXL],
                                          float (&ym0)[per::kXL], float (&ym1)[per::kXL]) {
@@ -180,72 +191,64 @@ __device__ __forceinline__ void per_pair(const unsigned char* __restrict__ smem,
   f2 a1 = lds_x2(smem, off1), b1 = lds_x2(smem, off1 + pitch);
   f2 d0 = sub2(b0, a0), d1 = sub2(b1, a1);
   float p0[kXL], p1[kXL];
-  ulonglong2 wq0, wq1;
+  f2 w0[Qq], w1[Qq];
+#pragma unroll
+  for (int t = 0; t < Qq; ++t) {
+    w0[t] = *reinterpret_cast<const f2*>(smem + wof0 + 8 * t);
+    w1[t] = *reinterpret_cast<const f2*>(smem + wof1 + 8 * t);
+  }
 #pragma unroll
   for (int t = 0; t < RUN; ++t) {
-    // next plane of a row: integers below 2^24, so the new lower plane is
+    // next plane of the rows: integers below 2^24, so the new lower plane is
     // exactly the old upper one
-    if (t > 0 && pofs(Pp, Qq, PH0, t) != pofs(Pp, Qq, PH0, t - 1)) {
+    if (t > 0 && pofs(Pp, Qq, PH, t) != pofs(Pp, Qq, PH, t - 1)) {
       a0 = b0;
-      b0 = lds_x2(smem, off0 + (uint32_t)(pofs(Pp, Qq, PH0, t) + 1) * pitch);
-      d0 = sub2(b0, a0);
-    }
-    if (t > 0 && pofs(Pp, Qq, PH1, t) != pofs(Pp, Qq, PH1, t - 1)) {
       a1 = b1;
-      b1 = lds_x2(smem, off1 + (uint32_t)(pofs(Pp, Qq, PH1, t) + 1) * pitch);
+      b0 = lds_x2(smem, off0 + (uint32_t)(pofs(Pp, Qq, PH, t) + 1) * pitch);
+      b1 = lds_x2(smem, off1 + (uint32_t)(pofs(Pp, Qq, PH, t) + 1) * pitch);
+      d0 = sub2(b0, a0);
       d1 = sub2(b1, a1);
     }
-    if ((t & 1) == 0) {  // weights of columns t and t + 1 of both rows
-      wq0 = *reinterpret_cast<const ulonglong2*>(smem + wof0 + 8 * t);
-      wq1 = *reinterpret_cast<const ulonglong2*>(smem + wof1 + 8 * t);
-    }
     float v0[kXL], v1[kXL];
-    upk(fma2((t & 1) ? wq0.y : wq0.x, d0, a0), v0[0], v0[1]);
-    upk(fma2((t & 1) ? wq1.y : wq1.x, d1, a1), v1[0], v1[1]);
+    upk(fma2(w0[t % Qq], d0, a0), v0[0], v0[1]);
+    upk(fma2(w1[t % Qq], d1, a1), v1[0], v1[1]);
 #pragma unroll
     for (int c = 0; c < kXL; ++c) zmax[t][c] = max3(zmax[t][c], v0[c], v1[c]);
-    if (YMIP && pcand(Pp, Qq, PH0, t, RUN)) {
-      if (pcount(Pp, Qq, PH0, t, RUN) % 2 == 0) {
+    if (YMIP && pcand(Pp, Qq, PH, t, RUN)) {
+      if (pcount(Pp, Qq, PH, t, RUN) % 2 == 0) {
 #pragma unroll
-        for (int c = 0; c < kXL; ++c) p0[c] = v0[c];
+        for (int c = 0; c < kXL; ++c) p0[c] = v0[c], p1[c] = v1[c];
       } else {
 #pragma unroll
-        for (int c = 0; c < kXL; ++c) ym0[c] = max3(ym0[c], p0[c], v0[c]);
-      }
-    }
-    if (YMIP && pcand(Pp, Qq, PH1, t, RUN)) {
-      if (pcount(Pp, Qq, PH1, t, RUN) % 2 == 0) {
-#pragma unroll
-        for (int c = 0; c < kXL; ++c) p1[c] = v1[c];
-      } else {
-#pragma unroll
-        for (int c = 0; c < kXL; ++c) ym1[c] = max3(ym1[c], p1[c], v1[c]);
+        for (int c = 0; c < kXL; ++c) {
+          ym0[c] = max3(ym0[c], p0[c], v0[c]);
+          ym1[c] = max3(ym1[c], p1[c], v1[c]);
+        }
       }
     }
   }
-  if (YMIP && pcount(Pp, Qq, PH0, RUN, RUN) % 2 == 1) {
+  if (YMIP && pcount(Pp, Qq, PH, RUN, RUN) % 2 == 1) {
 #pragma unroll
-    for (int c = 0; c < kXL; ++c) ym0[c] = fmaxf(ym0[c], p0[c]);
-  }
-  if (YMIP && pcount(Pp, Qq, PH1, RUN, RUN) % 2 == 1) {
-#pragma unroll
-    for (int c = 0; c < kXL; ++c) ym1[c] = fmaxf(ym1[c], p1[c]);
+    for (int c = 0; c < kXL; ++c) {
+      ym0[c] = fmaxf(ym0[c], p0[c]);
+      ym1[c] = fmaxf(ym1[c], p1[c]);
+    }
   }
 }
 
-// Phase pair idx = PH0 * Qq + PH1 in [LO, HI), by a balanced branch tree.
+// Phase ph in [LO, HI), by a balanced branch tree.
 template <int RUN, int Pp, int Qq, bool YMIP, int LO, int HI>
-__device__ __forceinline__ void per_tree(int idx, const unsigned char* __restrict__ smem, uint32_t off0,
-                                         uint32_t off1, uint32_t wof0, uint32_t wof1, float (&zmax)[RUN][per::kXL],
+__device__ __forceinline__ void per_tree(int ph, const unsigned char* __restrict__ smem, uint32_t off0, uint32_t off1,
+                                         uint32_t wof0, uint32_t wof1, float (&zmax)[RUN][per::kXL],
                                          float (&ym0)[per::kXL], float (&ym1)[per::kXL]) {
   if constexpr (HI - LO == 1) {
-    per_pair<RUN, Pp, Qq, YMIP, LO / Qq, LO % Qq>(smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
+    per_pair<RUN, Pp, Qq, YMIP, LO>(smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
   } else {
     constexpr int MID = (LO + HI) / 2;
-    if (idx < MID)
-      per_tree<RUN, Pp, Qq, YMIP, LO, MID>(idx, smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
+    if (ph < MID)
+      per_tree<RUN, Pp, Qq, YMIP, LO, MID>(ph, smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
     else
-      per_tree<RUN, Pp, Qq, YMIP, MID, HI>(idx, smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
+      per_tree<RUN, Pp, Qq, YMIP, MID, HI>(ph, smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
   }
 }
 
@@ -273,11 +276,9 @@ __device__ __forceinline__ bool per_consume(const FastJob& jb, const PerRing& r,
     js->zmip = jb.zmip;
     js->ymip = jb.ymip;
     js->nx = jb.nx;
-    js->nz = jb.nz;
     js->j0 = jb.j0;
     js->xbase = jb.xbase;
-    js->k0g = jb.ks - 2 * g;
-    js->gend = g + (jb.ke - jb.ks + 1) / 2;
+    js->gend = g + (jb.ke - jb.ks) / 2;
   }
   __syncwarp();
   float zmax[RUN][kXL];
@@ -299,30 +300,27 @@ __device__ __forceinline__ bool per_consume(const FastJob& jb, const PerRing& r,
     const uint32_t rec = (uint32_t)(offsetof(FastRow, rec) + (h * RUN / 8) * sizeof(FastRec));
     const uint2 rr0 = *reinterpret_cast<const uint2*>(smem + tab0 + rec);
     const uint2 rr1 = *reinterpret_cast<const uint2*>(smem + tab0 + (uint32_t)sizeof(FastRow) + rec);
-    const int c0 = (int)((rr0.x >> kPhaseShift) & 255u);
-    const int c1 = (int)((rr1.x >> kPhaseShift) & 255u);
+    const int2 rows = r.rows()[s];
     const uint32_t row0 = (uint32_t)(s * fast::stage_slab_bytes(r.Pl)) + xoff;
     const uint32_t row1 = row0 + (uint32_t)fast::slab_row_bytes(r.Pl);
     float ym0[kXL], ym1[kXL];
 #pragma unroll
     for (int c = 0; c < kXL; ++c) ym0[c] = ym1[c] = 0.0f;
     const uint32_t wof0 = tab0 + (uint32_t)(h * RUN * 8);
-    per_tree<RUN, Pp, Qq, YMIP, 0, Qq * Qq>(c0 * Qq + c1, smem, row0 + rr0.y * pitch, row1 + rr1.y * pitch, wof0,
-                                      wof0 + (uint32_t)sizeof(FastRow), zmax, ym0, ym1);
+    per_tree<RUN, Pp, Qq, YMIP, 0, Qq>((int)((rr0.x >> kPhaseShift) & 255u), smem, row0 + rr0.y * pitch,
+                                       row1 + rr1.y * pitch, wof0, wof0 + (uint32_t)sizeof(FastRow), zmax, ym0, ym1);
     __syncwarp();
     if (lane == 0) mbar_arrive(&r.sfree()[s]);
     if constexpr (!YMIP) continue;
     float* ymip = lds_volatile_ptr(&js->ymip);
     if (ymip) {
       const int nx = lds_volatile_s32(&js->nx);
-      const int k0 = lds_volatile_s32(&js->k0g) + 2 * g;
       const int x = lds_volatile_s32(&js->xbase) + xh * kXW + lane * kXL;
-      const bool second = k0 + 1 < lds_volatile_s32(&js->nz);
 #pragma unroll
       for (int c = 0; c < kXL; ++c) {
         if (x + c < nx) {
-          atomicMax(reinterpret_cast<int*>(ymip + (size_t)k0 * nx + x + c), __float_as_int(ym0[c]));
-          if (second) atomicMax(reinterpret_cast<int*>(ymip + (size_t)(k0 + 1) * nx + x + c), __float_as_int(ym1[c]));
+          atomicMax(reinterpret_cast<int*>(ymip + (size_t)rows.x * nx + x + c), __float_as_int(ym0[c]));
+          atomicMax(reinterpret_cast<int*>(ymip + (size_t)rows.y * nx + x + c), __float_as_int(ym1[c]));
         }
       }
     }

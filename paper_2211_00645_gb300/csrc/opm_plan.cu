@@ -134,6 +134,18 @@ opm_status opm_plan_create(int64_t nscan, int64_t nrows, int64_t ncols,
     const double half = (interp == OPM_INTERP_NEAREST) ? 0.5 : 0.0;
     p->hA.resize(ny);
     for (int64_t j = 0; j < ny; ++j) p->hA[j] = split((double)(j - p->J0) * p->rho + half);
+    // pixel/step of a compiled family up to the last bits: the exact ratio, so
+    // that the fractions of every q-th column are the same FP32 number
+    for (const Family& f : kFamilies) {
+      if (std::fabs(p->rho * f.q - f.p) > 1e-14 * f.p) continue;
+      const int64_t den = 2 * (int64_t)f.q;
+      for (int64_t j = 0; j < ny; ++j) {
+        const int64_t num = 2 * f.p * (j - p->J0) + (interp == OPM_INTERP_NEAREST ? f.q : 0);
+        const int64_t fl = num >= 0 ? num / den : -((-num + den - 1) / den);
+        p->hA[j] = Split{(int32_t)fl, (float)((double)(num - fl * den) / (double)den)};
+      }
+      break;
+    }
     p->hB.resize(nrows);
     for (int64_t k = 0; k < nrows; ++k) p->hB[k] = split((double)k * c * p->rho);
 
@@ -249,8 +261,13 @@ opm_status opm_plan_create(int64_t nscan, int64_t nrows, int64_t ncols,
       };
       for (int f = 0; f < kNumFamilies && !p->family; ++f) {
         bool all = true;
-        for (size_t i = 0; all && i < p->hFrow.size(); ++i)
-          all = phase(p->hFrow[i], kFamilies[f].p, kFamilies[f].q) >= 0;
+        for (size_t i = 0; all && i < p->hFrow.size(); ++i) {
+          const FastRow& fr = p->hFrow[i];
+          all = phase(fr, kFamilies[f].p, kFamilies[f].q) >= 0;
+          // the kernel keeps the weights of q columns for the whole row
+          for (int t = kFamilies[f].q; all && t < kTileJ; ++t)
+            all = std::memcmp(&fr.w[t][0], &fr.w[t - kFamilies[f].q][0], sizeof(float)) == 0;
+        }
         if (all) p->family = f + 1;
       }
       if (p->family) {
@@ -260,6 +277,32 @@ opm_status opm_plan_create(int64_t nscan, int64_t nrows, int64_t ncols,
           for (int g = 0; g < 4; ++g) fr.rec[g].adv |= (unsigned)((8 * g * fp + ph) % fq) << 16;
         }
         p->lists_per_sm = kPerCtasPerSm;
+        // The rows of every tile's band by phase, two at a time (an odd one
+        // out is paired with itself: maxima do not mind).  Rows of one phase
+        // in one tile share one in every other; all tiles take these classes
+        // of rows in the same order, so that neighbouring tiles, whose slabs
+        // overlap by two planes, read the same rows at about the same time.
+        p->hPair0.assign(ntile + 1, 0);
+        for (int64_t t = 0; t < ntile; ++t) {
+          p->hPair0[t] = (int)p->hPairs.size();
+          const int64_t turn = ((int64_t)tile_j0((int)t, (int)ny) - p->J0) * fp % fq + fq;
+          for (int cls = 0; cls < fq; ++cls) {
+            const int ph = (int)((cls + turn) % fq);
+            int64_t odd = -1;
+            for (int64_t k = p->hBand[t].lo; k < p->hBand[t].hi; ++k) {
+              if ((int)((p->hFrow[t * nrows + k].rec[0].adv >> 16) & 255u) != ph) continue;
+              if (odd < 0) {
+                odd = k;
+                continue;
+              }
+              p->hPairs.push_back(RowPair{(int)odd, (int)k, p->hFnlo[t * nrows + odd], p->hFnlo[t * nrows + k]});
+              odd = -1;
+            }
+            if (odd >= 0)
+              p->hPairs.push_back(RowPair{(int)odd, (int)odd, p->hFnlo[t * nrows + odd], p->hFnlo[t * nrows + odd]});
+          }
+        }
+        p->hPair0[ntile] = (int)p->hPairs.size();
       }
     }
 
@@ -312,19 +355,18 @@ opm_status opm_plan_create(int64_t nscan, int64_t nrows, int64_t ncols,
       const int nlists = std::min(std::max(nsm, 1) * p->lists_per_sm, kMaxLists);
       auto nchunks = [&](int rows) {
         int64_t n = 0;
-        for (const Band& bd : p->hBand)
-          if (bd.lo < bd.hi) n += (bd.hi - 1) / rows - bd.lo / rows + 1;
+        for (const Band& bd : p->hBand) n += band_units(bd, rows);
         return n * xtiles;
       };
       int rows = kChunkRows;
       while (rows > kMinChunkRows && (double)nchunks(rows) < kUnitsPerList * nlists) rows /= 2;
       p->chunk_rows = rows;
       for (int jt = 0; jt < (int)p->hBand.size(); ++jt) {
-        const Band bd = p->hBand[jt];
-        for (int c0 = (bd.lo / rows) * rows; c0 < bd.hi; c0 += rows) {
-          const int ks = std::max(bd.lo, c0), ke = std::min(bd.hi, c0 + rows);
-          if (ks >= ke) continue;
-          for (int xt = 0; xt < xtiles; ++xt) p->hUnits.push_back(WorkUnit{0, xt, jt, ks, ke, 0, 0, 0});
+        const int64_t n = p->family ? pair_units(p, jt, rows) : band_units(p->hBand[jt], rows);
+        for (int64_t u = 0; u < n; ++u) {
+          const Band r = unit_range(p, jt, rows, p->family, u, n);
+          if (r.lo >= r.hi) continue;
+          for (int xt = 0; xt < xtiles; ++xt) p->hUnits.push_back(WorkUnit{0, xt, jt, r.lo, r.hi, 0, 0, 0});
         }
       }
       if (p->hUnits.size() > (size_t)INT32_MAX) p->fast_ok = 0;
@@ -341,9 +383,11 @@ opm_status opm_plan_create(int64_t nscan, int64_t nrows, int64_t ncols,
   const size_t szY = align256(sizeof(float) * p->hYinit.size());
   const size_t szF = align256(sizeof(FastRow) * p->hFrow.size());
   const size_t szN = align256(sizeof(int) * p->hFnlo.size());
+  const size_t szP = align256(sizeof(RowPair) * p->hPairs.size());
+  const size_t szQ = align256(sizeof(int) * p->hPair0.size());
   const size_t szU = align256(sizeof(WorkUnit) * p->hUnits.size());
   const size_t szL = align256(sizeof(int) * p->hLists.size());
-  const size_t total = szA + szB + szT + szY + szF + szN + szU + szL + 256;
+  const size_t total = szA + szB + szT + szY + szF + szN + szP + szQ + szU + szL + 256;
   e = cudaMalloc(&p->dmem, total);
   if (e != cudaSuccess) {
     delete p;
@@ -356,9 +400,12 @@ opm_status opm_plan_create(int64_t nscan, int64_t nrows, int64_t ncols,
   float* dY = reinterpret_cast<float*>(base + szA + szB + szT);
   FastRow* dF = reinterpret_cast<FastRow*>(base + szA + szB + szT + szY);
   int* dN = reinterpret_cast<int*>(base + szA + szB + szT + szY + szF);
-  WorkUnit* dU = reinterpret_cast<WorkUnit*>(base + szA + szB + szT + szY + szF + szN);
-  int* dL = reinterpret_cast<int*>(base + szA + szB + szT + szY + szF + szN + szU);
-  unsigned* dE = reinterpret_cast<unsigned*>(base + szA + szB + szT + szY + szF + szN + szU + szL);
+  char* after = base + szA + szB + szT + szY + szF + szN;
+  RowPair* dP = reinterpret_cast<RowPair*>(after);
+  int* dQ = reinterpret_cast<int*>(after + szP);
+  WorkUnit* dU = reinterpret_cast<WorkUnit*>(after + szP + szQ);
+  int* dL = reinterpret_cast<int*>(after + szP + szQ + szU);
+  unsigned* dE = reinterpret_cast<unsigned*>(after + szP + szQ + szU + szL);
   if ((e = cudaMemcpy(dA, p->hA.data(), sizeof(Split) * p->hA.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemcpy(dB, p->hB.data(), sizeof(Split) * p->hB.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemcpy(dT, p->hBand.data(), sizeof(Band) * p->hBand.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
@@ -367,6 +414,11 @@ opm_status opm_plan_create(int64_t nscan, int64_t nrows, int64_t ncols,
        (e = cudaMemcpy(dF, p->hFrow.data(), sizeof(FastRow) * p->hFrow.size(), cudaMemcpyHostToDevice)) != cudaSuccess) ||
       (!p->hFnlo.empty() &&
        (e = cudaMemcpy(dN, p->hFnlo.data(), sizeof(int) * p->hFnlo.size(), cudaMemcpyHostToDevice)) != cudaSuccess) ||
+      (!p->hPairs.empty() && (e = cudaMemcpy(dP, p->hPairs.data(), sizeof(RowPair) * p->hPairs.size(),
+                                             cudaMemcpyHostToDevice)) != cudaSuccess) ||
+      (!p->hPair0.empty() &&
+       (e = cudaMemcpy(dQ, p->hPair0.data(), sizeof(int) * p->hPair0.size(), cudaMemcpyHostToDevice)) !=
+           cudaSuccess) ||
       (!p->hUnits.empty() &&
        (e = cudaMemcpy(dU, p->hUnits.data(), sizeof(WorkUnit) * p->hUnits.size(), cudaMemcpyHostToDevice)) !=
            cudaSuccess) ||
@@ -398,6 +450,8 @@ opm_status opm_plan_create(int64_t nscan, int64_t nrows, int64_t ncols,
   v.err = dE;
   v.frow = p->hFrow.empty() ? nullptr : dF;
   v.fnlo = p->hFnlo.empty() ? nullptr : dN;
+  v.pairs = p->hPairs.empty() ? nullptr : dP;
+  v.pair0 = p->hPair0.empty() ? nullptr : dQ;
   v.units = p->hUnits.empty() ? nullptr : dU;
   v.lists = p->hLists.empty() ? nullptr : dL;
   v.nunits = (int)p->hUnits.size();

@@ -114,7 +114,7 @@ k_project_fast(const __grid_constant__ CUtensorMap tmap, const ProjArgs args) {
 
 // Periodic kernel (opm_periodic.cuh): the fast kernel's schedule, tables
 // and TMA ring for plans with pixel/step = Pp/Qq, with straight-line compute
-// warps per phase pair; MINB CTAs per SM, S ring stages.
+// warps per phase; MINB CTAs per SM, S ring stages.
 template <int Pp, int Qq, int RUN, int MINB, int S, bool YMIP>
 __global__ void __launch_bounds__(per::Cfg<RUN>::kThreads, MINB)
 k_project_per(const __grid_constant__ CUtensorMap tmap, const ProjArgs args) {
@@ -145,7 +145,7 @@ k_project_per(const __grid_constant__ CUtensorMap tmap, const ProjArgs args) {
     jb.ke = un.ke;
     jb.tmap = &tmap;
     jb.rows = v.frow + (size_t)un.jt * v.nz;
-    jb.nlos = v.fnlo + (size_t)un.jt * v.nz;
+    jb.pairs = v.pairs + v.pair0[un.jt];
     jb.zmip = args.zmip;
     jb.ymip = args.ymip;
     jb.nz = v.nz;

@@ -228,6 +228,7 @@ struct FastJob {
   const CUtensorMap* tmap;  // the stack's raw tensor map (box {128, 1, P})
   const FastRow* rows;      // plane tables of this j-tile, indexed by camera row
   const int* nlos;          // first staged plane of this j-tile, per camera row
+  const RowPair* pairs;     // this j-tile's row pairs (periodic kernel: ks, ke count their rows)
   float* zmip;              // [ny][nx] or NULL
   float* ymip;              // [nz][nx] or NULL
   int nz, nx, j0, xbase, ks, ke, P;
