@@ -53,15 +53,12 @@ KERNEL_SOURCES = {
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per full-size
 # launch from ncu captures, keyed by the hash of the kernel's sources at
-# capture time (reported as null once a source has changed).  periodic:
-# captured at full size (448.58 MB read, 9.17 MB written, 76.8 M warp
-# instructions).  volume_f32:
-# captured with 100 scan planes (213.11 MB read, 2963.51 MB written) and
-# scaled to 200 planes, reads by the raw bytes (x2.0) and writes by the
-# volume bytes (x1.4161).
+# capture time (reported as null once a source has changed).  Both captured at
+# full size.  periodic: 448.36 MB read, 7.33 MB written, 70.2 M warp
+# instructions; volume_f32: 450.21 MB read, 4221.39 MB written.
 NCU_TRAFFIC = {
-    "periodic": {"src_sha": "0916abe0e7ee", "bytes_per_launch": 457752064, "warp_insts_per_launch": 76816242},
-    "volume_f32": {"src_sha": "4eff36766d3d", "bytes_per_launch": 4622836946},
+    "periodic": {"src_sha": "ded4b65b407e", "bytes_per_launch": 455692288, "warp_insts_per_launch": 70173217},
+    "volume_f32": {"src_sha": "10e9902e7130", "bytes_per_launch": 4671601408},
 }
 
 L2_BYTES = 129 * 10**6  # L2 of the GB300 (bytes)

@@ -125,7 +125,7 @@ struct opm_plan {
   int64_t nscan, nrows, ncols, nz, ny, nx, J0;
   double theta, step, pixel, c, rho;
   int interp;
-  int force_generic;  // use the plain (non-TMA) kernels for every call
+  int force_generic;  // use the direct kernel's element-wise form for every projection
   int P;              // planes staged per row for a 32-column tile
   int fast_ok;        // full tiles never step more than one plane per column
   int unit_steps = 0; // inside every 8-column group (from 0), a column lies on its left neighbour's plane or the next
