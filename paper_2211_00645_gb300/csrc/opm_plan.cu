@@ -134,20 +134,29 @@ opm_status opm_plan_create(int64_t nscan, int64_t nrows, int64_t ncols,
     const double half = (interp == OPM_INTERP_NEAREST) ? 0.5 : 0.0;
     p->hA.resize(ny);
     for (int64_t j = 0; j < ny; ++j) p->hA[j] = split((double)(j - p->J0) * p->rho + half);
-    // pixel/step of a compiled family up to the last bits: the exact ratio, so
-    // that the fractions of every q-th column are the same FP32 number
-    for (const Family& f : kFamilies) {
-      if (std::fabs(p->rho * f.q - f.p) > 1e-14 * f.p) continue;
-      const int64_t den = 2 * (int64_t)f.q;
-      for (int64_t j = 0; j < ny; ++j) {
-        const int64_t num = 2 * f.p * (j - p->J0) + (interp == OPM_INTERP_NEAREST ? f.q : 0);
-        const int64_t fl = num >= 0 ? num / den : -((-num + den - 1) / den);
-        p->hA[j] = Split{(int32_t)fl, (float)((double)(num - fl * den) / (double)den)};
-      }
-      break;
-    }
     p->hB.resize(nrows);
     for (int64_t k = 0; k < nrows; ++k) p->hB[k] = split((double)k * c * p->rho);
+    // LINEAR with pixel/step a compiled family up to the last bits: the exact
+    // ratio, so that the fractions of every q-th column are the same FP32
+    // number.  Where cos(theta) is a short binary fraction (60 and 90 degrees)
+    // rows and columns share plane coordinates, and the rows take the exact
+    // ratio as well: a coordinate that is a whole number then has a weight of
+    // exactly 0 (rounded on one side only it would lie a hair below, weight 1
+    // on the plane under it).  NEAREST has no weights to repeat, and at a tie
+    // the exact ratio could pick the other plane: it keeps the rounded one.
+    for (const Family& f : kFamilies) {
+      if (interp != OPM_INTERP_LINEAR || std::fabs(p->rho * f.q - f.p) > 1e-14 * f.p) continue;
+      const auto exact = [](int64_t num, int64_t den) {
+        const int64_t fl = num >= 0 ? num / den : -((-num + den - 1) / den);
+        return Split{(int32_t)fl, (float)((double)(num - fl * den) / (double)den)};
+      };
+      for (int64_t j = 0; j < ny; ++j) p->hA[j] = exact(f.p * (j - p->J0), f.q);
+      constexpr int kBits = 20;  // k < 2^29, so that k c 2^20 p stays below 2^52
+      const double cs = std::ldexp(c, kBits);
+      if (cs == std::floor(cs))
+        for (int64_t k = 0; k < nrows; ++k) p->hB[k] = exact(k * (int64_t)cs * f.p, (int64_t)f.q << kBits);
+      break;
+    }
 
     // Row band of every 32-wide j-tile, from the kernels' own plane formula
     // with a margin of one plane on each side.  n0 is non-increasing in k.
