@@ -410,9 +410,28 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
   int* hglists = reinterpret_cast<int*>(stage + off_glists);
   WorkUnit* hunits = reinterpret_cast<WorkUnit*>(stage + off_units);
   int64_t nunits = 0;
-  bool pairs_fit = family > 0;  // room for every unit of the row pairs
-  if (family) {
+  // Units of the general items: `fine`, a CTA's single pieces, else whole
+  // 32-column tiles.
+  auto general_units = [&](bool fine) {
     int64_t n = 0;
+    for (int i = 0; i < n_items; ++i) {
+      const opm_batch_item& it = items[i];
+      const opm_plan* p = it.plan;
+      const bool zout = it.zmip || it.zsum || it.argz;
+      if (!p || is_fast(it) || (!zout && !it.ymip)) continue;
+      const int cols = fine ? direct::cta_cols(direct::row_groups(p->ny, p->nx)) : kTileJ;
+      for (int64_t jt = 0; jt < (int64_t)p->hBand.size(); ++jt)
+        if (zout || p->hBand[jt].lo < p->hBand[jt].hi)
+          n += (p->nx + kX - 1) / kX * ((std::min<int64_t>(kTileJ, p->ny - jt * kTileJ) + cols - 1) / cols);
+    }
+    return n;
+  };
+  // Room for every unit of the row pairs beside the general items'?  Else the
+  // pairs are cut into as many units as the rows take in order, so that what
+  // fits the list does not depend on the pairing.
+  bool pairs_fit = family > 0;
+  if (family) {
+    int64_t n = general_units(false);
     for (int i = 0; i < n_items; ++i)
       if (is_fast(items[i]))
         for (int jt = 0; jt < (int)items[i].plan->hBand.size(); ++jt)
@@ -522,13 +541,7 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
     }
     if (pass == 0) {
       nfast = (int)nunits;
-      int64_t pieces = 0;
-      for (int i = 0; i < n_items; ++i) {
-        const opm_plan* p = items[i].plan;
-        const int cols = direct::cta_cols(hitems[i].wr);
-        pieces += (p->ny + cols - 1) / cols * ((p->nx + kX - 1) / kX);
-      }
-      fine = nunits + pieces <= max_units;
+      fine = nunits + general_units(true) <= max_units;
     }
   }
   const int ngen = (int)nunits - nfast;
