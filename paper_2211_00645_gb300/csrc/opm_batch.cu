@@ -182,7 +182,7 @@ k_batch_fast(const unsigned char* __restrict__ wl, int Pl, unsigned* err) {
 template <int RUN>
 constexpr int per_minb() { return RUN == 16 ? 3 : kPerCtasPerSm; }
 
-template <int Pp, int Qq, int RUN>
+template <int Pp, int Qq, int RUN, bool REP>
 __global__ void __launch_bounds__(per::Cfg<RUN>::kThreads, per_minb<RUN>())
 k_batch_per(const unsigned char* __restrict__ wl, int Pl, unsigned* err) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -230,7 +230,7 @@ k_batch_per(const unsigned char* __restrict__ wl, int Pl, unsigned* err) {
       __syncwarp();
       ok = per_produce(jb, ring, g, err, lane);
     } else {
-      ok = per_consume<RUN, Pp, Qq, true>(jb, ring, g, err, warp - 1, lane);
+      ok = per_consume<RUN, Pp, Qq, true, REP>(jb, ring, g, err, warp - 1, lane);
     }
   }
   if (warp == 0) per_drain(ring, g, ok, err);
@@ -333,13 +333,14 @@ struct WorkList {
   size_t used;  // bytes of the image to copy
   int n_items, n_units, n_segs, n_lists, Pl;
   int family;   // kFamilies index + 1 of the periodic kernel, or 0 (fast kernel)
+  int rep;      // 1: every periodic item's weights repeat
   int n_gunits; // units of the general kernel
   int Pg;       // planes of its deepest item's tile rows
   int run;      // columns j per compute warp of the periodic kernel (32 or 16)
   int shape;    // opm_shape the list was built for (never AUTO)
 };
 
-constexpr WorkList kEmptyWorkList = {kOffItems, 0, 0, 0, 0, 2, 0, 0, 2, kPerRun, OPM_SHAPE_PER_J32X2};
+constexpr WorkList kEmptyWorkList = {kOffItems, 0, 0, 0, 0, 2, 0, 1, 0, 2, kPerRun, OPM_SHAPE_PER_J32X2};
 
 // Builds the work-list image of `items` into `stage` (room for max_items
 // items and max_units units; 64-byte aligned).  Allocates nothing on
@@ -371,9 +372,12 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
   auto is_fast = [&](const opm_batch_item& it) {
     return it.plan && !gen_all && plan_fast_ok(it.plan) && !it.zsum && !it.argz && (it.zmip || it.ymip);
   };
-  int family = -1;
-  for (int i = 0; i < n_items; ++i)
-    if (is_fast(items[i])) family = (family < 0 || family == items[i].plan->family) ? items[i].plan->family : 0;
+  int family = -1, rep = 1;
+  for (int i = 0; i < n_items; ++i) {
+    if (!is_fast(items[i])) continue;
+    family = (family < 0 || family == items[i].plan->family) ? items[i].plan->family : 0;
+    rep &= items[i].plan->weights_repeat;
+  }
   if (family < 0 || shape == OPM_SHAPE_FAST_J8X4) family = 0;
   if (!gen_all) {
     if (shape == OPM_SHAPE_AUTO) shape = family ? OPM_SHAPE_PER_J32X2 : OPM_SHAPE_FAST_J8X4;
@@ -567,6 +571,7 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
   out->n_lists = nlists;
   out->Pl = Pl;
   out->family = family;
+  out->rep = rep;
   out->n_gunits = ngen;
   out->Pg = Pg;
   out->run = shape == OPM_SHAPE_PER_J16X2 ? 16 : kPerRun;
@@ -578,19 +583,19 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
 // header lists, so one grid shape serves every content.
 constexpr int kZeroRows = 32;
 
-template <int F>
+template <int F, bool REP>
 void launch_batch_per(const unsigned char* dev_wl, const WorkList& wl, int grid, unsigned* err, cudaStream_t s) {
   if constexpr (F < kNumFamilies) {
-    if (wl.family - 1 != F) return launch_batch_per<F + 1>(dev_wl, wl, grid, err, s);
+    if (wl.family - 1 != F) return launch_batch_per<F + 1, REP>(dev_wl, wl, grid, err, s);
     constexpr int Pp = kFamilies[F].p, Qq = kFamilies[F].q;
     const size_t smem = batch_smem(wl.Pl, wl.family);
     if constexpr (F == 0) {  // 16-column runs are compiled for the first family only
       if (wl.run == 16) {
-        k_batch_per<Pp, Qq, 16><<<grid, per::Cfg<16>::kThreads, smem, s>>>(dev_wl, wl.Pl, err);
+        k_batch_per<Pp, Qq, 16, REP><<<grid, per::Cfg<16>::kThreads, smem, s>>>(dev_wl, wl.Pl, err);
         return;
       }
     }
-    k_batch_per<Pp, Qq, kPerRun><<<grid, per::Cfg<kPerRun>::kThreads, smem, s>>>(dev_wl, wl.Pl, err);
+    k_batch_per<Pp, Qq, kPerRun, REP><<<grid, per::Cfg<kPerRun>::kThreads, smem, s>>>(dev_wl, wl.Pl, err);
   }
 }
 
@@ -615,7 +620,7 @@ cudaError_t launch_worklist(const unsigned char* dev_wl, const WorkList& wl, int
   if (e != cudaSuccess) return e;
   if (grid > 0) {
     if (wl.family)
-      launch_batch_per<0>(dev_wl, wl, grid, err, s);
+      wl.rep ? launch_batch_per<0, true>(dev_wl, wl, grid, err, s) : launch_batch_per<0, false>(dev_wl, wl, grid, err, s);
     else
       batch_fast_kernel(wl.Pl)<<<grid, kThreads, batch_smem(wl.Pl, 0), s>>>(dev_wl, wl.Pl, err);
     e = cudaGetLastError();
@@ -655,13 +660,13 @@ cudaError_t set_kernel_smem(K kern, int smem_optin) {
   return e;
 }
 
-template <int F>
+template <int F, bool REP>
 cudaError_t set_per_attrs(int smem_optin) {
   if constexpr (F < kNumFamilies) {
-    cudaError_t e = set_kernel_smem(k_batch_per<kFamilies[F].p, kFamilies[F].q, kPerRun>, smem_optin);
+    cudaError_t e = set_kernel_smem(k_batch_per<kFamilies[F].p, kFamilies[F].q, kPerRun, REP>, smem_optin);
     if constexpr (F == 0)
-      if (e == cudaSuccess) e = set_kernel_smem(k_batch_per<kFamilies[F].p, kFamilies[F].q, 16>, smem_optin);
-    return e == cudaSuccess ? set_per_attrs<F + 1>(smem_optin) : e;
+      if (e == cudaSuccess) e = set_kernel_smem(k_batch_per<kFamilies[F].p, kFamilies[F].q, 16, REP>, smem_optin);
+    return e == cudaSuccess ? set_per_attrs<F + 1, REP>(smem_optin) : e;
   }
   return cudaSuccess;
 }
@@ -672,7 +677,8 @@ cudaError_t set_fast_attrs(int smem_optin) {
   if (e == cudaSuccess) e = set_kernel_smem(k_batch_fast<4>, smem_optin);
   if (e == cudaSuccess) e = set_kernel_smem(k_batch_fast<3>, smem_optin);
   if (e == cudaSuccess) e = set_kernel_smem(k_batch_gen, smem_optin);
-  return e == cudaSuccess ? set_per_attrs<0>(smem_optin) : e;
+  if (e == cudaSuccess) e = set_per_attrs<0, true>(smem_optin);
+  return e == cudaSuccess ? set_per_attrs<0, false>(smem_optin) : e;
 }
 
 }  // namespace
@@ -698,10 +704,10 @@ struct opm_batch {
   int attr_set;
   cudaStream_t capture;  // private stream the graphs are captured on
   // Captured launches (zero kernel + persistent kernels), one per launch
-  // shape: kernel shape, periodic family and run, slab depth and grids.
+  // shape: kernel shape, periodic family, run and weights, slab depth and grids.
   struct Graph {
     cudaGraphExec_t exec;
-    int key[6];
+    int key[7];
     unsigned long long used;  // launch counter at the last use
   } graphs[kGraphCache];
   unsigned long long launches;
@@ -824,11 +830,11 @@ opm_status opm_batch_launch_graph(opm_batch* b, int ctas_per_sm, void* stream) {
   // full grids: every CTA reads the unit counts from the device header
   int grid = 0, ggrid = 0;
   batch_grids(b->wl, b->nsm, ctas_per_sm, true, &grid, &ggrid);
-  const int key[6] = {grid ? b->wl.shape : 0, grid ? b->wl.family : 0, grid ? b->wl.run : 0,
+  const int key[7] = {grid ? b->wl.shape : 0, grid ? b->wl.family : 0, grid ? b->wl.run : 0, grid ? b->wl.rep : 0,
                       grid ? b->wl.Pl : 0,    grid,                     ggrid};
   opm_batch::Graph* hit = nullptr;
   for (auto& gr : b->graphs)
-    if (gr.exec && std::equal(key, key + 6, gr.key)) hit = &gr;
+    if (gr.exec && std::equal(key, key + 7, gr.key)) hit = &gr;
   b->launches += 1;
   if (!hit) {
     // an empty slot, else the least recently used one
@@ -852,7 +858,7 @@ opm_status opm_batch_launch_graph(opm_batch* b, int ctas_per_sm, void* stream) {
       hit->exec = nullptr;
       return cuda_fail(e, "capturing the batch launch");
     }
-    std::copy(key, key + 6, hit->key);
+    std::copy(key, key + 7, hit->key);
     b->graph_captures += 1;
   }
   hit->used = b->launches;

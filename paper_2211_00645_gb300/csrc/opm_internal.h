@@ -130,6 +130,7 @@ struct opm_plan {
   int fast_ok;        // full tiles never step more than one plane per column
   int unit_steps = 0; // inside every 8-column group (from 0), a column lies on its left neighbour's plane or the next
   int family = 0;     // 1 + index into kFamilies when the periodic kernel applies, else 0
+  bool weights_repeat = false;  // periodic plans: every q-th column of a row has the same weight, bit for bit
   int lists_per_sm = 4;  // persistent CTA lists per SM of the live-view schedule
   int chunk_rows = 0;    // rows per work unit of that schedule (0: no schedule)
   std::vector<opm::Split> hA, hB;

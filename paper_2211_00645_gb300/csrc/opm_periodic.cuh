@@ -180,8 +180,8 @@ __device__ __forceinline__ f2 lds_x2(const unsigned char* smem, uint32_t off) {
 // Both camera rows of a stage for one compute warp: a run of RUN columns, both
 // rows at phase PH.  off0 / off1: shared-memory offset of this lane's 2
 // columns x in the tile's first plane of each row; wof0 / wof1: the run's (w,
-// w) weight pairs of each row, of which the first Qq repeat.
-template <int RUN, int Pp, int Qq, bool YMIP, int PH>
+// w) weight pairs of each row, of which the first Qq repeat (REP) or not.
+template <int RUN, int Pp, int Qq, bool YMIP, bool REP, int PH>
 __device__ __forceinline__ void per_pair(const unsigned char* __restrict__ smem, uint32_t off0, uint32_t off1,
                                          uint32_t wof0, uint32_t wof1, float (&zmax)[RUN][per::kXL],
                                          float (&ym0)[per::kXL], float (&ym1)[per::kXL]) {
@@ -191,11 +191,14 @@ __device__ __forceinline__ void per_pair(const unsigned char* __restrict__ smem,
   f2 a1 = lds_x2(smem, off1), b1 = lds_x2(smem, off1 + pitch);
   f2 d0 = sub2(b0, a0), d1 = sub2(b1, a1);
   float p0[kXL], p1[kXL];
-  f2 w0[Qq], w1[Qq];
+  constexpr int kW = REP ? Qq : 2;  // weights held per row: the run's, or two columns'
+  f2 w0[kW], w1[kW];
+  if constexpr (REP) {
 #pragma unroll
-  for (int t = 0; t < Qq; ++t) {
-    w0[t] = *reinterpret_cast<const f2*>(smem + wof0 + 8 * t);
-    w1[t] = *reinterpret_cast<const f2*>(smem + wof1 + 8 * t);
+    for (int t = 0; t < Qq; ++t) {
+      w0[t] = *reinterpret_cast<const f2*>(smem + wof0 + 8 * t);
+      w1[t] = *reinterpret_cast<const f2*>(smem + wof1 + 8 * t);
+    }
   }
 #pragma unroll
   for (int t = 0; t < RUN; ++t) {
@@ -209,9 +212,14 @@ __device__ __forceinline__ void per_pair(const unsigned char* __restrict__ smem,
       d0 = sub2(b0, a0);
       d1 = sub2(b1, a1);
     }
+    if (!REP && t % 2 == 0) {
+      const ulonglong2 q0 = *reinterpret_cast<const ulonglong2*>(smem + wof0 + 8 * t);
+      const ulonglong2 q1 = *reinterpret_cast<const ulonglong2*>(smem + wof1 + 8 * t);
+      w0[0] = q0.x, w0[1] = q0.y, w1[0] = q1.x, w1[1] = q1.y;
+    }
     float v0[kXL], v1[kXL];
-    upk(fma2(w0[t % Qq], d0, a0), v0[0], v0[1]);
-    upk(fma2(w1[t % Qq], d1, a1), v1[0], v1[1]);
+    upk(fma2(w0[t % kW], d0, a0), v0[0], v0[1]);
+    upk(fma2(w1[t % kW], d1, a1), v1[0], v1[1]);
 #pragma unroll
     for (int c = 0; c < kXL; ++c) zmax[t][c] = max3(zmax[t][c], v0[c], v1[c]);
     if (YMIP && pcand(Pp, Qq, PH, t, RUN)) {
@@ -237,18 +245,18 @@ __device__ __forceinline__ void per_pair(const unsigned char* __restrict__ smem,
 }
 
 // Phase ph in [LO, HI), by a balanced branch tree.
-template <int RUN, int Pp, int Qq, bool YMIP, int LO, int HI>
+template <int RUN, int Pp, int Qq, bool YMIP, bool REP, int LO, int HI>
 __device__ __forceinline__ void per_tree(int ph, const unsigned char* __restrict__ smem, uint32_t off0, uint32_t off1,
                                          uint32_t wof0, uint32_t wof1, float (&zmax)[RUN][per::kXL],
                                          float (&ym0)[per::kXL], float (&ym1)[per::kXL]) {
   if constexpr (HI - LO == 1) {
-    per_pair<RUN, Pp, Qq, YMIP, LO>(smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
+    per_pair<RUN, Pp, Qq, YMIP, REP, LO>(smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
   } else {
     constexpr int MID = (LO + HI) / 2;
     if (ph < MID)
-      per_tree<RUN, Pp, Qq, YMIP, LO, MID>(ph, smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
+      per_tree<RUN, Pp, Qq, YMIP, REP, LO, MID>(ph, smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
     else
-      per_tree<RUN, Pp, Qq, YMIP, MID, HI>(ph, smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
+      per_tree<RUN, Pp, Qq, YMIP, REP, MID, HI>(ph, smem, off0, off1, wof0, wof1, zmax, ym0, ym1);
   }
 }
 
@@ -262,7 +270,7 @@ constexpr int kPhaseShift = 16;
 // both rows of every stage.  z-maxima stay in registers and are folded into
 // zmip at the end of the job; each row's y-max over the run goes to ymip
 // right away.  Returns false when a bounded wait gave up.
-template <int RUN, int Pp, int Qq, bool YMIP>
+template <int RUN, int Pp, int Qq, bool YMIP, bool REP>
 __device__ __forceinline__ bool per_consume(const FastJob& jb, const PerRing& r, int& g, unsigned* err, int i,
                                             int lane) {
   using namespace per;
@@ -307,8 +315,9 @@ __device__ __forceinline__ bool per_consume(const FastJob& jb, const PerRing& r,
 #pragma unroll
     for (int c = 0; c < kXL; ++c) ym0[c] = ym1[c] = 0.0f;
     const uint32_t wof0 = tab0 + (uint32_t)(h * RUN * 8);
-    per_tree<RUN, Pp, Qq, YMIP, 0, Qq>((int)((rr0.x >> kPhaseShift) & 255u), smem, row0 + rr0.y * pitch,
-                                       row1 + rr1.y * pitch, wof0, wof0 + (uint32_t)sizeof(FastRow), zmax, ym0, ym1);
+    per_tree<RUN, Pp, Qq, YMIP, REP, 0, Qq>((int)((rr0.x >> kPhaseShift) & 255u), smem, row0 + rr0.y * pitch,
+                                            row1 + rr1.y * pitch, wof0, wof0 + (uint32_t)sizeof(FastRow), zmax, ym0,
+                                            ym1);
     __syncwarp();
     if (lane == 0) mbar_arrive(&r.sfree()[s]);
     if constexpr (!YMIP) continue;

@@ -53,6 +53,9 @@ static int host_n0(Split a, Split b) {
   return a.i - b.i - (d < 0.0f ? 1 : 0);
 }
 
+// pixel/step is p/q up to rounding.
+static bool near_ratio(double rho, const Family& f) { return std::fabs(rho * f.q - f.p) <= 1e-14 * f.p; }
+
 static size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
 static opm_status check_plan(const opm_plan* p) {
@@ -145,7 +148,7 @@ opm_status opm_plan_create(int64_t nscan, int64_t nrows, int64_t ncols,
     // on the plane under it).  NEAREST has no weights to repeat, and at a tie
     // the exact ratio could pick the other plane: it keeps the rounded one.
     for (const Family& f : kFamilies) {
-      if (interp != OPM_INTERP_LINEAR || std::fabs(p->rho * f.q - f.p) > 1e-14 * f.p) continue;
+      if (interp != OPM_INTERP_LINEAR || !near_ratio(p->rho, f)) continue;
       const auto exact = [](int64_t num, int64_t den) {
         const int64_t fl = num >= 0 ? num / den : -((-num + den - 1) / den);
         return Split{(int32_t)fl, (float)((double)(num - fl * den) / (double)den)};
@@ -271,23 +274,16 @@ opm_status opm_plan_create(int64_t nscan, int64_t nrows, int64_t ncols,
       std::vector<int> phases(p->hFrow.size());  // of every tile's rows, for the family found
       for (int f = 0; f < kNumFamilies && !p->family; ++f) {
         bool all = true;
-        // The kernel keeps the weights of q columns for the whole row.  Columns
-        // whose fractions repeat have weights that do; only where they do not
-        // are the rows compared one by one.  With that and the phases worked
-        // out once per row, the plan of a 200 x 512 x 2048 stack takes 4.4 ms
-        // on the host against 6.4.
-        bool repeat = true;
-        for (int64_t j = kFamilies[f].q; repeat && j < ny; ++j)
-          repeat = std::memcmp(&p->hA[j].f, &p->hA[j - kFamilies[f].q].f, sizeof(float)) == 0;
         for (size_t i = 0; all && i < p->hFrow.size(); ++i) {
-          const FastRow& fr = p->hFrow[i];
-          const int ph = phase(fr, kFamilies[f].p, kFamilies[f].q);
-          all = ph >= 0;
-          phases[i] = ph;
-          for (int t = kFamilies[f].q; all && !repeat && t < kTileJ; ++t)
-            all = std::memcmp(&fr.w[t][0], &fr.w[t - kFamilies[f].q][0], sizeof(float)) == 0;
+          phases[i] = phase(p->hFrow[i], kFamilies[f].p, kFamilies[f].q);
+          all = phases[i] >= 0;
         }
-        if (all) p->family = f + 1;
+        if (!all) continue;
+        p->family = f + 1;
+        // Columns with the exact ratio's fractions have weights that repeat
+        // (NEAREST has none).  Left to pixel and step alone, so that plans of
+        // one geometry take the same kernel whatever their size.
+        p->weights_repeat = near_ratio(p->rho, kFamilies[f]);
       }
       if (p->family) {
         const int fp = kFamilies[p->family - 1].p, fq = kFamilies[p->family - 1].q;

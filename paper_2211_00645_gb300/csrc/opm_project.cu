@@ -115,7 +115,7 @@ k_project_fast(const __grid_constant__ CUtensorMap tmap, const ProjArgs args) {
 // Periodic kernel (opm_periodic.cuh): the fast kernel's schedule, tables
 // and TMA ring for plans with pixel/step = Pp/Qq, with straight-line compute
 // warps per phase; MINB CTAs per SM, S ring stages.
-template <int Pp, int Qq, int RUN, int MINB, int S, bool YMIP>
+template <int Pp, int Qq, int RUN, int MINB, int S, bool YMIP, bool REP>
 __global__ void __launch_bounds__(per::Cfg<RUN>::kThreads, MINB)
 k_project_per(const __grid_constant__ CUtensorMap tmap, const ProjArgs args) {
   const PlanView& v = args.v;
@@ -156,7 +156,7 @@ k_project_per(const __grid_constant__ CUtensorMap tmap, const ProjArgs args) {
     if (warp == 0)
       ok = per_produce(jb, ring, g, v.err, lane);
     else
-      ok = per_consume<RUN, Pp, Qq, YMIP>(jb, ring, g, v.err, warp - 1, lane);
+      ok = per_consume<RUN, Pp, Qq, YMIP, REP>(jb, ring, g, v.err, warp - 1, lane);
   }
   if (warp == 0) per_drain(ring, g, ok, v.err);
 }
@@ -265,10 +265,12 @@ opm_status launch_per_f(const opm_plan* p, const CUtensorMap& map, const ProjArg
   if constexpr (F < kNumFamilies) {
     if (p->family - 1 != F) return launch_per_f<F + 1>(p, map, args, s, grid_div);
     constexpr int Pp = kFamilies[F].p, Qq = kFamilies[F].q;
-    static int done[2][64] = {{0}};
-    const auto kern = args.ymip ? k_project_per<Pp, Qq, kPerRun, kPerCtasPerSm, kPerStages, true>
-                                : k_project_per<Pp, Qq, kPerRun, kPerCtasPerSm, kPerStages, false>;
-    opm_status st = prepare_kernel(kern, p->device, done[args.ymip != nullptr]);
+    static int done[4][64] = {{0}};
+    const bool ym = args.ymip != nullptr, rep = p->weights_repeat;
+    constexpr int R = kPerRun, C = kPerCtasPerSm, S = kPerStages;
+    const auto kern = ym ? (rep ? k_project_per<Pp, Qq, R, C, S, true, true> : k_project_per<Pp, Qq, R, C, S, true, false>)
+                         : (rep ? k_project_per<Pp, Qq, R, C, S, false, true> : k_project_per<Pp, Qq, R, C, S, false, false>);
+    opm_status st = prepare_kernel(kern, p->device, done[2 * ym + rep]);
     if (st != OPM_OK) return st;
     const PlanView& v = p->view;
     const int full = std::min(v.nunits, v.nlists);
