@@ -9,24 +9,25 @@
 //
 // Both projections are gathered.  The lower plane falls along k and grows
 // along j, so the rows of one column j that belong to pair n are one run
-// (1 / (rho cos theta) rows, 3.7 on the live-view geometry), and so are the
-// columns of one row k (1 / rho); each output value is written by one thread,
-// once, with no atomics and nothing zeroed beforehand.  A warp takes one
-// column j (or row k) x 128 columns x and finds its run with a 32-way search
-// of the split table; the 8 warps of a CTA take neighbours, whose runs share
-// camera rows.  Consecutive pairs' runs adjoin, so the sliding view folds its
-// complete pair and its mixed pair in one walk, together with the maxima it
-// combines them with.
+// (1 / (rho cos theta) rows, 3.7 on the live-view geometry, all of them at 90
+// degrees), and so are the columns of one row k (1 / rho); each output value is
+// written by one thread, once, with no atomics and nothing zeroed beforehand.
+// A warp takes one column j (or row k) x 128 columns x and finds its run by 32
+// candidates around the place the geometry gives; the 8 warps of a CTA take
+// neighbours, whose runs share camera rows.  Where runs are long and columns few
+// several warps share a column (column_share).  Consecutive pairs' runs adjoin,
+// so the sliding view folds its complete pair and its mixed pair in one walk,
+// together with the maxima it combines them with; columns outside both runs are
+// passed through unsearched.
 //
 // What bounds it: L2 traffic (a push reads the run and one slot and writes a
-// slot and the view, 45 MB at 200 planes) and the search's latency.  Device
-// time back to back, 512 x 2048 frames, 35 deg, step 0.3, pixel 0.1, before
-// (a scatter of shared and global atomic maxima; a push was two of them, one
-// zeroing and two elementwise maxima) -> now: one pair 9.8 -> 9.2 us, with a
-// z-sum 14.9 -> 10.2; a push on 200 planes 30.3 -> 17.7, the last one with the
-// next suffixes 1240 -> 773 (5 GB of slots read and written, 6.5 TB/s); 87 x
-// 1304 frames of 50 planes: pair 5.0 -> 3.4, push 16.9 -> 5.7, last 135 -> 33.
-// Four rows' loads ahead cost occupancy and were slower (18.9 a push).
+// slot and the view, 45 MB at 200 planes) and the latency of search and walk.
+// Device time back to back, 512 x 2048 frames, 35 deg, step 0.3, pixel 0.1: a
+// pair 7.1 us, with a z-sum 7.6; a push on 24 planes 12.5; 87 x 1304 frames of
+// 24 planes: pair 3.2, push 4.7.  (A scatter of shared and global atomic maxima
+// took 9.8 and 15; a push made of two of them, one zeroing and two elementwise
+// maxima 28, and 15 on the small frames.)
+// Four rows' loads ahead in a short run cost occupancy and were slower.
 #include <algorithm>
 
 #include "opm_tma.cuh"
@@ -37,7 +38,8 @@ namespace {
 
 constexpr int kSXL = 4;            // columns x per lane
 constexpr int kSXW = 32 * kSXL;    // columns x per warp
-constexpr int kSWarps = 8;         // neighbouring columns j (rows k) per CTA
+constexpr int kSWarps = 8;         // warps per CTA: neighbouring columns j (or rows k), S warps to a column
+__host__ __device__ constexpr int cta_warps(int S) { return S > kSWarps ? S : kSWarps; }
 constexpr int kNoPair = -0x40000000;
 
 __global__ void k_stream_zero(float* zmip, float* zsum, long long nj, float* ymip, long long nk) {
@@ -59,10 +61,20 @@ struct Pair {
 };
 
 // First index in [0, count) for which `reached` holds (it holds from there
-// on), count if none.  Whole warp.
+// on), count if none.  Whole warp: 32 candidates around `guess` first, then
+// 32 evenly spaced ones at a time.
 template <typename Pred>
-__device__ __forceinline__ int first_index(int count, int lane, const Pred& reached) {
+__device__ __forceinline__ int first_index(int count, int lane, float guess, const Pred& reached) {
   int lo = 0, hi = count;  // the answer lies in [lo, hi]
+  const int i0 = max(0, (int)fminf(guess, (float)count) - 15);
+  const unsigned b0 = __ballot_sync(0xffffffffu, i0 + lane >= count || reached(i0 + lane));
+  const int f0 = b0 ? __ffs(b0) - 1 : 32;
+  if (f0 == 32)
+    lo = i0 + 32;
+  else if (f0 > 0 || i0 == 0)
+    return min(i0 + f0, count);
+  else
+    hi = min(i0, count);
   while (lo < hi) {
     const int st = (hi - lo + 31) >> 5;
     const int i = lo + lane * st;
@@ -79,25 +91,38 @@ __device__ __forceinline__ int first_index(int count, int lane, const Pred& reac
   return lo;
 }
 
-// This lane's kSXL counts of camera row k of one frame: neighbours (VEC) or
-// columns 32 apart; zeros for a missing frame.
+// First row k of column j whose lower plane is at most n, nz if none (it
+// falls along k); rows = 1 / (rho cos theta).
+__device__ __forceinline__ int first_row(const PlanView& v, float rows, const Split& aj, int n, int lane) {
+  return first_index(v.nz, lane, ((float)(aj.i - n - 1) + aj.f) * rows, [&](int k) {
+    const Split b = v.B[k];
+    return aj.i - b.i - (aj.f - b.f < 0.0f) <= n;
+  });
+}
+
+// This lane's kSXL counts of a camera row, two to a word: neighbours (VEC) or
+// columns XS apart (zeros past the edge).
+template <bool VEC, int XS = 32>
+__device__ __forceinline__ uint2 load_words(const uint16_t* __restrict__ p, int lim) {
+  if constexpr (VEC) {
+    return __ldg(reinterpret_cast<const uint2*>(p));
+  } else {
+    uint2 w = make_uint2(0, 0);
+    if (0 < lim) w.x = __ldg(p);
+    if (XS < lim) w.x |= (uint32_t)__ldg(p + XS) << 16;
+    if (2 * XS < lim) w.y = __ldg(p + 2 * XS);
+    if (3 * XS < lim) w.y |= (uint32_t)__ldg(p + 3 * XS) << 16;
+    return w;
+  }
+}
+
+// The same as FP32 values, of element o of one frame; zeros for a missing frame.
 template <bool VEC>
 __device__ __forceinline__ void load_counts(const uint16_t* __restrict__ frame, size_t o, int lim, f2 (&out)[2]) {
-  uint32_t w0 = 0, w1 = 0;
-  if (frame) {
-    const uint16_t* p = frame + o;
-    if constexpr (VEC) {
-      const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
-      w0 = u.x, w1 = u.y;
-    } else {
-      if (0 < lim) w0 = __ldg(p);
-      if (32 < lim) w0 |= (uint32_t)__ldg(p + 32) << 16;
-      if (64 < lim) w1 = __ldg(p + 64);
-      if (96 < lim) w1 |= (uint32_t)__ldg(p + 96) << 16;
-    }
-  }
-  out[0] = u16x2_to_f2(w0);
-  out[1] = u16x2_to_f2(w1);
+  uint2 w = make_uint2(0, 0);
+  if (frame) w = load_words<VEC>(frame + o, lim);
+  out[0] = u16x2_to_f2(w.x);
+  out[1] = u16x2_to_f2(w.y);
 }
 
 // Maxima (and sums of A's voxels) over one column's or row's voxels in pairs A
@@ -120,19 +145,15 @@ __device__ __forceinline__ void fold_voxel(float w, const f2 (&lo)[2], const f2 
 
 // Column j: its rows in pair B (nB = nA + 1, which come first) and pair A.
 template <bool VEC, bool SUM>
-__device__ __forceinline__ void fold_column(const PlanView& v, const Pair& A, const Pair& B, int j, int lane, int x0,
-                                            int lim, Fold& f) {
+__device__ __forceinline__ void fold_column(const PlanView& v, float rows, const Pair& A, const Pair& B, int j, int lane,
+                                            int x0, int lim, Fold& f) {
   const Split aj = v.A[j];
-  const int top = B.n != kNoPair ? B.n : A.n, bottom = A.n != kNoPair ? A.n : B.n;
-  auto lower = [&](int k) {
-    const Split b = v.B[k];
-    return aj.i - b.i - (aj.f - b.f < 0.0f);
-  };
-  for (int k = first_index(v.nz, lane, [&](int i) { return lower(i) <= top; }); k < v.nz; ++k) {
+  const int top = B.n != kNoPair ? B.n : A.n;
+  for (int k = first_row(v, rows, aj, top, lane); k < v.nz; ++k) {
     int n0;
     float w;
     plane_weight(aj, v.B[k], v.linear, n0, w);
-    if (n0 < bottom) break;
+    if (n0 < A.n) break;
     f.any = true;
     const bool isB = n0 == B.n;
     const size_t o = (size_t)k * v.ncols + x0;
@@ -151,57 +172,151 @@ __device__ __forceinline__ void fold_column(const PlanView& v, const Pair& A, co
   }
 }
 
+// The same for a run of many rows, shared by S warps of G row groups each (32 /
+// G lanes to a row): row group g = G s + lane / (32 / G) takes rows g, g + S G,
+// ... of the run, kAhead at a time.  Their loads overlap: which pair a row
+// belongs to is searched for, not read with the row, and a missing frame is a
+// mask, not a branch.  BOTH: pair B is given.  Afterwards the first 32 / G lanes
+// of warp s = 0 hold the column's results, joined in the order of the groups.
+// Every warp of the CTA takes part (live: it has a column).
+template <bool VEC, bool SUM, bool BOTH, int S, int G>
+__device__ __forceinline__ void fold_long_column(const PlanView& v, float per_plane, const Pair& A, const Pair& B,
+                                                 int j, bool live, int x0, int lim, Fold& f) {
+  constexpr int kAhead = 4, XS = 32 / G;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, s = warp % S;
+  if (live) {
+    const Split aj = v.A[j];
+    const int k0 = first_row(v, per_plane, aj, BOTH ? B.n : A.n, lane);
+    const int rows = first_row(v, per_plane, aj, A.n - 1, lane) - k0;
+    const int rowsB = BOTH ? first_row(v, per_plane, aj, A.n, lane) - k0 : 0;
+    f.any = rows > 0;
+    const uint16_t* const alo = A.lo ? A.lo : A.hi;
+    const uint16_t* const ahi = A.hi ? A.hi : A.lo;
+    const uint32_t malo = A.lo ? ~0u : 0u, mahi = A.hi ? ~0u : 0u;
+    const uint16_t* const blo = BOTH ? (B.lo ? B.lo : B.hi) : nullptr;
+    const uint16_t* const bhi = BOTH ? (B.hi ? B.hi : B.lo) : nullptr;
+    const uint32_t mblo = BOTH && B.lo ? ~0u : 0u, mbhi = BOTH && B.hi ? ~0u : 0u;
+#pragma unroll 1
+    for (int r = s * G; r < rows; r += kAhead * S * G) {
+      uint2 lo[kAhead], hi[kAhead];
+      Split bk[kAhead];
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u) {
+        const int i = min(r + u * S * G + lane / XS, rows - 1);  // the last row again: maxima do not mind
+        const bool isB = BOTH && i < rowsB;
+        const size_t o = (size_t)(k0 + i) * v.ncols + x0;
+        bk[u] = v.B[k0 + i];
+        lo[u] = load_words<VEC, XS>((isB ? blo : alo) + o, lim);
+        hi[u] = load_words<VEC, XS>((isB ? bhi : ahi) + o, lim);
+      }
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u) {
+        const int i = r + u * S * G + lane / XS;
+        const bool isB = BOTH && min(i, rows - 1) < rowsB;
+        const uint32_t ml = isB ? mblo : malo, mh = isB ? mbhi : mahi;
+        const f2 l[2] = {u16x2_to_f2(lo[u].x & ml), u16x2_to_f2(lo[u].y & ml)};
+        const f2 h[2] = {u16x2_to_f2(hi[u].x & mh), u16x2_to_f2(hi[u].y & mh)};
+        int n0;
+        float w, val[kSXL];
+        plane_weight(aj, bk[u], v.linear, n0, w);
+        if (isB) {
+          fold_voxel(w, l, h, f.b, val);
+        } else {
+          fold_voxel(w, l, h, f.a, val);
+          if constexpr (SUM)
+            if (i < rows) {
+#pragma unroll
+              for (int c = 0; c < kSXL; ++c) f.s[c] += val[c];
+            }
+        }
+      }
+    }
+#pragma unroll
+    for (int d = XS; d < 32; d *= 2)
+#pragma unroll
+      for (int c = 0; c < kSXL; ++c) {
+        f.a[c] = fmaxf(f.a[c], __shfl_xor_sync(0xffffffffu, f.a[c], d));
+        if (BOTH) f.b[c] = fmaxf(f.b[c], __shfl_xor_sync(0xffffffffu, f.b[c], d));
+        if (SUM) f.s[c] += __shfl_xor_sync(0xffffffffu, f.s[c], d);
+      }
+  }
+  __shared__ float part[BOTH || SUM ? 2 : 1][cta_warps(S)][kSXW / G];
+  if (s > 0 && lane < XS)
+#pragma unroll
+    for (int c = 0; c < kSXL; ++c) {
+      part[0][warp][XS * c + lane] = f.a[c];
+      if (BOTH || SUM) part[1][warp][XS * c + lane] = BOTH ? f.b[c] : f.s[c];
+    }
+  __syncthreads();
+  if (s > 0 || lane >= XS) return;
+#pragma unroll 1
+  for (int q = 1; q < S; ++q)
+#pragma unroll
+    for (int c = 0; c < kSXL; ++c) {
+      f.a[c] = fmaxf(f.a[c], part[0][warp + q][XS * c + lane]);
+      if (BOTH) f.b[c] = fmaxf(f.b[c], part[1][warp + q][XS * c + lane]);
+      if (SUM) f.s[c] += part[1][warp + q][XS * c + lane];
+    }
+}
+
 // Row k: its columns in pair A (which come first) and pair B.
 template <bool VEC>
 __device__ __forceinline__ void fold_row(const PlanView& v, const Pair& A, const Pair& B, int k, int lane, int x0,
                                          int lim, Fold& f) {
   const Split b = v.B[k];
-  const int top = B.n != kNoPair ? B.n : A.n, bottom = A.n != kNoPair ? A.n : B.n;
-  auto lower = [&](int j) {
+  const int top = B.n != kNoPair ? B.n : A.n;
+  const float guess = (float)v.J0 + ((float)(A.n + b.i) + b.f - (v.linear ? 0.0f : 0.5f)) * v.rinv;
+  const int first = first_index(v.ny, lane, guess, [&](int j) {
     const Split a = v.A[j];
-    return a.i - b.i - (a.f - b.f < 0.0f);
-  };
+    return a.i - b.i - (a.f - b.f < 0.0f) >= A.n;
+  });
   const size_t o = (size_t)k * v.ncols + x0;
   f2 lo[2], hi[2];
   int held = kNoPair;
-  for (int j = first_index(v.ny, lane, [&](int i) { return lower(i) >= bottom; }); j < v.ny; ++j) {
-    int n0;
-    float w;
-    plane_weight(v.A[j], b, v.linear, n0, w);
-    if (n0 > top) break;
-    f.any = true;
-    const bool isB = n0 == B.n;
-    if (n0 != held) {
-      load_counts<VEC>(isB ? B.lo : A.lo, o, lim, lo);
-      load_counts<VEC>(isB ? B.hi : A.hi, o, lim, hi);
-      held = n0;
+  for (int jb = first; jb < v.ny; jb += 32) {
+    int nl;
+    float wl;
+    plane_weight(v.A[min(jb + lane, v.ny - 1)], b, v.linear, nl, wl);  // of 32 columns at once
+    const int columns = __popc(__ballot_sync(0xffffffffu, jb + lane < v.ny && nl <= top));
+    f.any |= columns > 0;
+#pragma unroll 1
+    for (int t = 0; t < columns; ++t) {
+      const int n0 = __shfl_sync(0xffffffffu, nl, t);
+      const float w = __shfl_sync(0xffffffffu, wl, t);
+      const bool isB = n0 == B.n;
+      if (n0 != held) {
+        load_counts<VEC>(isB ? B.lo : A.lo, o, lim, lo);
+        load_counts<VEC>(isB ? B.hi : A.hi, o, lim, hi);
+        held = n0;
+      }
+      float val[kSXL];
+      if (isB)
+        fold_voxel(w, lo, hi, f.b, val);
+      else
+        fold_voxel(w, lo, hi, f.a, val);
     }
-    float val[kSXL];
-    if (isB)
-      fold_voxel(w, lo, hi, f.b, val);
-    else
-      fold_voxel(w, lo, hi, f.a, val);
+    if (columns < 32) break;
   }
 }
 
-template <bool VEC>
+template <bool VEC, int XS>
 __device__ __forceinline__ void get(const float* p, int lim, float (&out)[kSXL]) {
   if constexpr (VEC) {
     const float4 q = *reinterpret_cast<const float4*>(p);
     out[0] = q.x, out[1] = q.y, out[2] = q.z, out[3] = q.w;
   } else {
 #pragma unroll
-    for (int c = 0; c < kSXL; ++c) out[c] = 32 * c < lim ? p[32 * c] : 0.0f;
+    for (int c = 0; c < kSXL; ++c) out[c] = XS * c < lim ? p[XS * c] : 0.0f;
   }
 }
-template <bool VEC>
+template <bool VEC, int XS>
 __device__ __forceinline__ void put(float* p, int lim, const float (&v)[kSXL]) {
   if constexpr (VEC) {
     *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
   } else {
 #pragma unroll
     for (int c = 0; c < kSXL; ++c)
-      if (32 * c < lim) p[32 * c] = v[c];
+      if (XS * c < lim) p[XS * c] = v[c];
   }
 }
 __device__ __forceinline__ void max_into(float (&a)[kSXL], const float (&b)[kSXL]) {
@@ -209,57 +324,102 @@ __device__ __forceinline__ void max_into(float (&a)[kSXL], const float (&b)[kSXL
   for (int c = 0; c < kSXL; ++c) a[c] = fmaxf(a[c], b[c]);
 }
 
-// Which column j or row k a warp owns, and its columns x.  Blocks: x-tiles
-// fastest, the columns [j0, j1) in groups of kSWarps, then the rows.
+// Blocks of a launch, x-tiles fastest in each part: columns [j0, j1), which may
+// hold voxels of the pairs, S warps to a column and kSXW / G columns x to a
+// tile; the other columns (a push only) and the rows, one warp and kSXW columns
+// x each.
+struct Parts {
+  int xtiles, xtiles_live;
+  int j0, j1;
+  unsigned live, idle;  // blocks of the first two parts
+  float rows;           // rows of a column in one pair, 1 / (rho cos theta)
+};
+
+// What a warp works on: column j or row k, and its lane's columns x.
 struct Place {
-  bool column, live;
+  bool ok;      // there is such a column or row
   int i;        // j or k
   int x0, lim;  // first column x of the lane, columns from there to the edge
 };
-template <bool VEC>
-__device__ __forceinline__ Place place(const PlanView& v, int xtiles, int j0, int j1) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int jgroups = (j1 - j0 + kSWarps - 1) / kSWarps;
-  const int g = blockIdx.x / xtiles, xb = (blockIdx.x - g * xtiles) * kSXW;
-  Place p;
-  p.column = g < jgroups;
-  p.i = (p.column ? j0 + g * kSWarps : (g - jgroups) * kSWarps) + warp;
-  p.live = p.i < (p.column ? j1 : v.nz);
-  p.x0 = xb + (VEC ? lane * kSXL : lane);
+template <bool VEC, int XS>
+__device__ __forceinline__ Place place(const PlanView& v, bool ok, int i, int xt) {
+  const int lane = (threadIdx.x & 31) % XS;
+  Place p{ok, i, xt * XS * kSXL + (VEC ? lane * kSXL : lane), 0};
   p.lim = v.nx - p.x0;
   if (VEC && p.lim <= 0) p.x0 = 0;  // reads something, writes nothing
   return p;
 }
+template <bool VEC, int S, int G>
+__device__ __forceinline__ Place live_column(const PlanView& v, const Parts& t) {
+  constexpr int C = cta_warps(S) / S;
+  const int g = blockIdx.x / t.xtiles_live, j = t.j0 + g * C + (int)(threadIdx.x >> 5) / S;
+  return place<VEC, 32 / G>(v, j < t.j1, j, blockIdx.x - g * t.xtiles_live);
+}
+template <bool VEC, int S>
+__device__ __forceinline__ Place idle_column(const PlanView& v, const Parts& t) {
+  const unsigned b = blockIdx.x - t.live;
+  const int g = b / t.xtiles, i = g * cta_warps(S) + (int)(threadIdx.x >> 5);
+  const int j = i < t.j0 ? i : i + (t.j1 - t.j0);
+  return place<VEC, 32>(v, j < v.ny, j, b - g * t.xtiles);
+}
+template <bool VEC, int S>
+__device__ __forceinline__ Place some_row(const PlanView& v, const Parts& t) {
+  const unsigned b = blockIdx.x - t.live - t.idle;
+  const int g = b / t.xtiles, k = g * cta_warps(S) + (int)(threadIdx.x >> 5);
+  return place<VEC, 32>(v, k < v.nz, k, b - g * t.xtiles);
+}
+
+// A column's voxels in the pairs; false for lanes that have nothing to write.
+template <bool VEC, bool SUM, bool BOTH, int S, int G>
+__device__ __forceinline__ bool fold_live(const PlanView& v, const Parts& t, const Pair& A, const Pair& B, const Place& p,
+                                          Fold& f) {
+  if constexpr (S == 1) {
+    static_assert(G == 1, "one row at a time");
+    if (p.ok) fold_column<VEC, SUM>(v, t.rows, A, B, p.i, threadIdx.x & 31, p.x0, p.lim, f);
+    return p.ok && p.lim > 0;
+  } else {
+    fold_long_column<VEC, SUM, BOTH, S, G>(v, t.rows, A, B, p.i, p.ok, p.x0, p.lim, f);
+    return p.ok && p.lim > 0 && (threadIdx.x >> 5) % S == 0 && (threadIdx.x & 31) < 32 / G;
+  }
+}
+
+// 64 registers where columns are shared, so that the rows (and the push's idle
+// columns) beside them find room for enough warps.
+template <int S>
+constexpr int min_ctas() { return S == 1 ? 1 : 32 / cta_warps(S); }
 
 // Pair A into the outputs (any of them NULL): columns [j0, j1) hold its voxels.
-template <bool VEC, bool SUM>
-__global__ void __launch_bounds__(32 * kSWarps)
-k_stream_pair(PlanView v, Pair A, int xtiles, int j0, int j1, float* zmip, float* zsum, float* ymip) {
-  const Place p = place<VEC>(v, xtiles, j0, j1);
-  if (!p.live) return;
-  const int lane = threadIdx.x & 31;
+template <bool VEC, bool SUM, int S, int G>
+__global__ void __launch_bounds__(32 * cta_warps(S), min_ctas<S>())
+k_stream_pair(PlanView v, Pair A, Parts t, float* zmip, float* zsum, float* ymip) {
   const Pair none{nullptr, nullptr, kNoPair};
   Fold f{};
-  if (p.column)
-    fold_column<VEC, SUM>(v, A, none, p.i, lane, p.x0, p.lim, f);
-  else
-    fold_row<VEC>(v, A, none, p.i, lane, p.x0, p.lim, f);
-  float* out = p.column ? zmip : ymip;
-  if (!f.any || p.lim <= 0) return;
-  const size_t o = (size_t)p.i * v.nx + p.x0;
   float old[kSXL];
-  if (out) {
-    get<VEC>(out + o, p.lim, old);
-    max_into(f.a, old);
-    put<VEC>(out + o, p.lim, f.a);
-  }
-  if constexpr (SUM) {
-    if (p.column) {
-      get<VEC>(zsum + o, p.lim, old);
+  if (blockIdx.x < t.live) {
+    constexpr int XS = 32 / G;
+    const Place p = live_column<VEC, S, G>(v, t);
+    if (!fold_live<VEC, SUM, false, S, G>(v, t, A, none, p, f) || !f.any) return;
+    const size_t o = (size_t)p.i * v.nx + p.x0;
+    if (zmip) {
+      get<VEC, XS>(zmip + o, p.lim, old);
+      max_into(f.a, old);
+      put<VEC, XS>(zmip + o, p.lim, f.a);
+    }
+    if constexpr (SUM) {
+      get<VEC, XS>(zsum + o, p.lim, old);
 #pragma unroll
       for (int c = 0; c < kSXL; ++c) old[c] += f.s[c];
-      put<VEC>(zsum + o, p.lim, old);
+      put<VEC, XS>(zsum + o, p.lim, old);
     }
+  } else {
+    const Place p = some_row<VEC, S>(v, t);
+    if (!p.ok) return;
+    fold_row<VEC>(v, A, none, p.i, threadIdx.x & 31, p.x0, p.lim, f);
+    if (!f.any || p.lim <= 0) return;
+    float* y = ymip + (size_t)p.i * v.nx + p.x0;
+    get<VEC, 32>(y, p.lim, old);
+    max_into(f.a, old);
+    put<VEC, 32>(y, p.lim, f.a);
   }
 }
 
@@ -277,32 +437,46 @@ struct Slide {
   bool fresh, last;
 };
 
-template <bool VEC>
-__global__ void __launch_bounds__(32 * kSWarps)
-k_sliding_push(PlanView v, Pair A, Pair B, Slide s, int xtiles) {
-  const Place p = place<VEC>(v, xtiles, 0, v.ny);
-  if (!p.live) return;
-  const int lane = threadIdx.x & 31;
-  const size_t o = (p.column ? (size_t)0 : (size_t)v.ny * v.nx) + (size_t)p.i * v.nx + p.x0;
-  float run[kSXL] = {}, next[kSXL] = {};
-  if (p.lim > 0) {  // on their way while the run is searched
-    if (!s.fresh) get<VEC>(s.run + o, p.lim, run);
-    if (s.next) get<VEC>(s.next + o, p.lim, next);
-  }
-  Fold f{};
-  if (p.column)
-    fold_column<VEC, false>(v, A, B, p.i, lane, p.x0, p.lim, f);
-  else
-    fold_row<VEC>(v, A, B, p.i, lane, p.x0, p.lim, f);
-  if (p.lim <= 0) return;
-  if (s.slotA) put<VEC>(s.slotA + o, p.lim, f.a);
-  if (s.slotB) put<VEC>(s.slotB + o, p.lim, f.b);
+template <bool VEC, int XS>
+__device__ __forceinline__ void slide_load(const Slide& s, size_t o, int lim, float (&run)[kSXL], float (&next)[kSXL]) {
+  if (!s.fresh) get<VEC, XS>(s.run + o, lim, run);
+  if (s.next) get<VEC, XS>(s.next + o, lim, next);
+}
+template <bool VEC, int XS>
+__device__ __forceinline__ void slide_store(const Slide& s, size_t o, int lim, const Fold& f, float (&run)[kSXL],
+                                            const float (&next)[kSXL]) {
+  if (s.slotA) put<VEC, XS>(s.slotA + o, lim, f.a);
+  if (s.slotB) put<VEC, XS>(s.slotB + o, lim, f.b);
   max_into(run, f.a);
   if (s.last) max_into(run, f.b);
-  if (f.any || s.fresh) put<VEC>(s.run + o, p.lim, run);
+  if (f.any || s.fresh) put<VEC, XS>(s.run + o, lim, run);
   max_into(run, next);
   max_into(run, f.b);
-  put<VEC>(s.view + o, p.lim, run);
+  put<VEC, XS>(s.view + o, lim, run);
+}
+
+template <bool VEC, int S, int G>
+__global__ void __launch_bounds__(32 * cta_warps(S), min_ctas<S>())
+k_sliding_push(PlanView v, Pair A, Pair B, Slide s, Parts t) {
+  float run[kSXL] = {}, next[kSXL] = {};
+  Fold f{};
+  if (blockIdx.x < t.live) {
+    constexpr int XS = 32 / G;
+    const Place p = live_column<VEC, S, G>(v, t);
+    const size_t o = (size_t)p.i * v.nx + p.x0;
+    if (S == 1 && p.ok && p.lim > 0) slide_load<VEC, XS>(s, o, p.lim, run, next);  // on their way during the search
+    if (!fold_live<VEC, false, true, S, G>(v, t, A, B, p, f)) return;
+    if (S > 1) slide_load<VEC, XS>(s, o, p.lim, run, next);
+    slide_store<VEC, XS>(s, o, p.lim, f, run, next);
+    return;
+  }
+  const bool row = blockIdx.x >= t.live + t.idle;
+  const Place p = row ? some_row<VEC, S>(v, t) : idle_column<VEC, S>(v, t);
+  if (!p.ok) return;
+  const size_t o = (row ? (size_t)v.ny * v.nx : (size_t)0) + (size_t)p.i * v.nx + p.x0;
+  if (p.lim > 0) slide_load<VEC, 32>(s, o, p.lim, run, next);
+  if (row) fold_row<VEC>(v, A, B, p.i, threadIdx.x & 31, p.x0, p.lim, f);
+  if (p.lim > 0) slide_store<VEC, 32>(s, o, p.lim, f, run, next);
 }
 
 // Suffix maxima of the slots: slot q = max(slot q, .., slot last), q = last - 1
@@ -377,36 +551,90 @@ static bool stream_vec(const PlanView& v, const void* f0, const void* f1, const 
 }
 static bool vec_out(const void* p) { return (uintptr_t)p % 16 == 0; }
 
-// Blocks for columns [j0, j1) and all rows; 0 when there are too many.
-static unsigned stream_blocks(const PlanView& v, long long columns, bool rows) {
-  const long long xtiles = (v.nx + kSXW - 1) / kSXW;
-  const long long groups = (columns + kSWarps - 1) / kSWarps + (rows ? (v.nz + kSWarps - 1) / kSWarps : 0);
-  return xtiles * groups <= 0x7fffffffLL ? (unsigned)(xtiles * groups) : 0u;
+// A way to share a column: S warps of G row groups.
+template <int S_, int G_>
+struct Share {
+  static constexpr int S = S_, G = G_;
+};
+
+// Rows of a column in one pair (all of them at 90 degrees).
+static double run_rows(const opm_plan* p) { return std::min((double)p->nz, 1.0 / std::max(p->rho * p->c, 1e-12)); }
+
+// Warps per column for runs of `run` rows; `warps`: columns x x-tiles, the warps
+// that one to a column would make.  One serves while they fill the GPU or the
+// runs are short; beyond that a run is walked by 4, 8 or 16 (x 4 row groups).
+// The lines lie where both sides cost the same on frames of 87 to 2048 rows.
+// us per pair (z + y) with 1 / 4 / 8 / 16 warps, and with the scatter before:
+//   512 x 2048, step 0.3, pixel 0.1, 75 deg (run 12, warps 2160)  6.3 / 9.5 / - / -        9.8
+//   ..., 85 deg (34, 768)                                       11.7 / 7.6 / 8.2 / 31      9.7
+//   ..., 89 deg (172, 192)                                        48 / 7.1 / 7.0 / 12      9.6
+//   ..., 90 deg (512, 48)                                        137 / 15 / 9.6 / 7.6      9.5
+//   87 x 1304, step 0.4, pixel 0.115, 90 deg (87, 55)              25 / 5.0 / 4.1 / 4.3    5.3
+//   1024 x 256, step 0.5, pixel 0.1, 90 deg (1024, 10)            275 / 27 / 15 / 6.0      5.6
+// Rows off 8 bytes cost four times the loads, which sharing hides as well:
+//   333 x 1001 with a z-sum, step 0.2, pixel 0.115, 75 deg (6.7, 704) 8.4 / 6.3 / - / 35   7.3
+static int column_share(double run, long long warps, bool vec) {
+  if (run >= 64.0 && (double)warps <= (vec ? 0.17 : 1.0) * run) return 16;
+  if (run >= 64.0 && (double)warps <= 1.5 * run) return 8;
+  return run * 1000.0 > (vec ? 12.0 : 5.0) * (double)warps ? 4 : 1;
+}
+
+// Calls go(Share) for the chosen one.
+template <typename Go>
+static void with_share(int S, const Go& go) {
+  if (S == 1)
+    go(Share<1, 1>{});
+  else if (S == 4)
+    go(Share<4, 1>{});
+  else if (S == 8)
+    go(Share<8, 1>{});
+  else
+    go(Share<16, 4>{});
+}
+
+// The blocks for columns [j0, j1), the others if `idle`, and all rows if `rows`;
+// their number, or 0 when there are none or too many.
+static unsigned stream_parts(const opm_plan* p, int S, int j0, int j1, bool idle, bool rows, Parts* t) {
+  const PlanView& v = p->view;
+  const auto up = [](long long a, long long b) { return (a + b - 1) / b; };
+  const int G = S == 16 ? Share<16, 4>::G : 1, W = cta_warps(S);
+  const long long xt = up(v.nx, kSXW), xl = up(v.nx, kSXW / G);
+  const long long live = xl * up(j1 - j0, W / S), off = idle ? xt * up(v.ny - (j1 - j0), W) : 0;
+  const long long all = live + off + (rows ? xt * up(v.nz, W) : 0);
+  if (all > 0x7fffffffLL) return 0;
+  *t = Parts{(int)xt, (int)xl, j0, j1, (unsigned)live, (unsigned)off, (float)run_rows(p)};
+  return (unsigned)all;
+}
+
+// Columns with a voxel in the pairs n .. last: n0 grows with j and falls with k.
+static void pair_columns(const opm_plan* p, int n, int last, int* j0, int* j1) {
+  const auto lower = [](const Split& a, const Split& b) { return a.i - b.i - (a.f - b.f < 0.0f ? 1 : 0); };
+  const auto first = [&](const Split& b, int least) {
+    return (int)(std::partition_point(p->hA.begin(), p->hA.end(), [&](const Split& a) { return lower(a, b) < least; }) -
+                 p->hA.begin());
+  };
+  *j0 = first(p->hB.front(), n);
+  *j1 = std::max(*j0, first(p->hB.back(), last + 1));
 }
 
 opm_status launch_stream_pair(const opm_plan* p, const uint16_t* lo, const uint16_t* hi, int n, float* zmip,
                               float* zsum, float* ymip, cudaStream_t s) {
   const PlanView& v = p->view;
   if (v.nz > 65535) return fail(OPM_ERR_UNSUPPORTED, "more than 65535 camera rows");
-  // columns with a voxel in the pair: n0 grows with j and falls with k
-  const Split b0 = p->hB.front(), b1 = p->hB.back();
-  const auto lower = [](const Split& a, const Split& b) { return a.i - b.i - (a.f - b.f < 0.0f ? 1 : 0); };
-  const auto first = [&](const Split& b, int least) {
-    return (int)(std::partition_point(p->hA.begin(), p->hA.end(), [&](const Split& a) { return lower(a, b) < least; }) -
-                 p->hA.begin());
-  };
-  int j0 = first(b0, n), j1 = first(b1, n + 1);
-  if ((!zmip && !zsum) || j1 < j0) j1 = j0;
-  const unsigned blocks = stream_blocks(v, j1 - j0, ymip != nullptr);
-  if (blocks == 0) {
-    if (j1 == j0 && !ymip) return OPM_OK;  // the pair has no voxel
-    return fail(OPM_ERR_UNSUPPORTED, "plane-pair grid exceeds launch limits");
-  }
+  int j0 = 0, j1 = 0;
+  if (zmip || zsum) pair_columns(p, n, n, &j0, &j1);
+  if (j1 == j0 && !ymip) return OPM_OK;  // the pair has no voxel
   const bool vec = stream_vec(v, lo, hi, nullptr) && vec_out(zmip) && vec_out(zsum) && vec_out(ymip);
-  const int xtiles = (v.nx + kSXW - 1) / kSXW;
-  const auto kern = zsum ? (vec ? k_stream_pair<true, true> : k_stream_pair<false, true>)
-                         : (vec ? k_stream_pair<true, false> : k_stream_pair<false, false>);
-  kern<<<blocks, 32 * kSWarps, 0, s>>>(v, Pair{lo, hi, n}, xtiles, j0, j1, zmip, zsum, ymip);
+  const int share = column_share(run_rows(p), (j1 - j0) * (long long)((v.nx + kSXW - 1) / kSXW), vec);
+  Parts t;
+  const unsigned blocks = stream_parts(p, share, j0, j1, false, ymip != nullptr, &t);
+  if (blocks == 0) return fail(OPM_ERR_UNSUPPORTED, "plane-pair grid exceeds launch limits");
+  with_share(share, [&](auto sh) {
+    constexpr int S = decltype(sh)::S, G = decltype(sh)::G;
+    const auto kern = zsum ? (vec ? k_stream_pair<true, true, S, G> : k_stream_pair<false, true, S, G>)
+                           : (vec ? k_stream_pair<true, false, S, G> : k_stream_pair<false, false, S, G>);
+    kern<<<blocks, 32 * cta_warps(S), 0, s>>>(v, Pair{lo, hi, n}, t, zmip, zsum, ymip);
+  });
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? OPM_OK : cuda_fail(e, "launch k_stream_pair");
 }
@@ -460,11 +688,17 @@ opm_status launch_sliding_push(const opm_plan* p, const uint16_t* stack, int m, 
   sl.view = view;
   sl.fresh = m == 0;
   sl.last = last;
-  const unsigned blocks = stream_blocks(v, v.ny, true);
-  if (blocks == 0) return fail(OPM_ERR_UNSUPPORTED, "sliding-view grid exceeds launch limits");
+  int j0, j1;
+  pair_columns(p, A.n, B.n, &j0, &j1);
   const bool vec = stream_vec(v, A.lo, A.hi, B.hi) && per % kSXL == 0 && vec_out(run) && vec_out(slots) && vec_out(view);
-  const int xtiles = (v.nx + kSXW - 1) / kSXW;
-  (vec ? k_sliding_push<true> : k_sliding_push<false>)<<<blocks, 32 * kSWarps, 0, s>>>(v, A, B, sl, xtiles);
+  const int share = column_share(run_rows(p), (j1 - j0) * (long long)((v.nx + kSXW - 1) / kSXW), vec);
+  Parts t;
+  const unsigned blocks = stream_parts(p, share, j0, j1, true, true, &t);
+  if (blocks == 0) return fail(OPM_ERR_UNSUPPORTED, "sliding-view grid exceeds launch limits");
+  with_share(share, [&](auto sh) {
+    constexpr int S = decltype(sh)::S, G = decltype(sh)::G;
+    (vec ? k_sliding_push<true, S, G> : k_sliding_push<false, S, G>)<<<blocks, 32 * cta_warps(S), 0, s>>>(v, A, B, sl, t);
+  });
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "launch k_sliding_push");
   if (last && N > 2) {  // the next stack's suffixes
