@@ -4,8 +4,8 @@
 // keeps the current pair of raw planes in registers, so a raw vector is
 // fetched once per plane step rather than once per voxel.  The run's planes
 // and weights are worked out by the warp's lanes side by side, one column
-// each, and handed round by shuffles; the plane after the current pair is
-// already on its way when the walk steps onto it.
+// each, and handed round by shuffles; where the walk next steps onto the plane
+// after the current pair, that plane is already on its way.
 // A lane owns NH vectors of H columns x, 32 H apart, so that every load and
 // store instruction of a warp covers one contiguous span.
 // Bounded by DRAM: the FP32 volume of 200 x 512 x 2048 (35 deg, step 0.3, pixel
@@ -141,7 +141,7 @@ k_deskew(PlanView v, const Tin* __restrict__ raw, Tout* __restrict__ vol, uint16
   };
 
   Acc a[NH][H], b[NH][H], d[NH][H];
-  RawVec<Tin, H> next[NH];  // plane ocur + 2
+  RawVec<Tin, H> next[NH];  // plane ocur + 2, when the next change steps onto plane ocur + 1
   int ocur = -0x40000000;   // plane index held in a[] (none yet)
 #pragma unroll
   for (int h = 0; h < NH; ++h)
@@ -170,7 +170,8 @@ k_deskew(PlanView v, const Tin* __restrict__ raw, Tout* __restrict__ vol, uint16
           widen<Tin, H, Acc>(r1[h], b[h]);
         }
       }
-      fetch(n0 + 2, next);
+      const unsigned later = jj < 31 ? change >> (jj + 1) : 0u;
+      if (later && __shfl_sync(0xffffffffu, nl, jj + __ffs(later)) == n0 + 1) fetch(n0 + 2, next);
 #pragma unroll
       for (int h = 0; h < NH; ++h)
 #pragma unroll
