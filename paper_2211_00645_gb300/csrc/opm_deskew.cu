@@ -25,23 +25,46 @@ constexpr int kThreadsX = 32;  // lanes along x
 constexpr int kThreadsY = 4;   // j-runs per CTA
 constexpr int kRunJ = 32;      // output columns per warp, one per lane for the plane table
 
-// H raw elements as loaded: 8 or 16 bytes, or a single element.
+// H raw elements as loaded, packed into words; VEC: one load of 8 or 16 bytes,
+// else element by element.
 template <typename T, int H>
 struct RawVec {
-  static_assert(H == 1 || sizeof(T) * H == 8 || sizeof(T) * H == 16, "8- or 16-byte vectors");
-  uint32_t w[(sizeof(T) * H + 3) / 4];
+  static_assert(sizeof(T) * H == 8 || sizeof(T) * H == 16, "8- or 16-byte vectors");
+  uint32_t w[sizeof(T) * H / 4];
+};
+template <typename T>
+struct RawVec<T, 1> {
+  T v;
 };
 
-template <typename T, int H>
+template <bool VEC, typename T, int H>
 __device__ __forceinline__ void load_raw(const T* __restrict__ p, RawVec<T, H>& out) {
-  if constexpr (sizeof(T) * H == 16) {
+  if constexpr (H == 1) {
+    out.v = __ldg(p);
+  } else if constexpr (!VEC) {
+#pragma unroll
+    for (int i = 0; i < (int)(sizeof(out.w) / 4); ++i) {
+      if constexpr (sizeof(T) == 2)
+        out.w[i] = (uint32_t)__ldg(p + 2 * i) | (uint32_t)__ldg(p + 2 * i + 1) << 16;
+      else
+        out.w[i] = __float_as_uint(__ldg(p + i));
+    }
+  } else if constexpr (sizeof(T) * H == 16) {
     const uint4 u = __ldg(reinterpret_cast<const uint4*>(p));
     out.w[0] = u.x, out.w[1] = u.y, out.w[2] = u.z, out.w[3] = u.w;
-  } else if constexpr (sizeof(T) * H == 8) {
+  } else {
     const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
     out.w[0] = u.x, out.w[1] = u.y;
+  }
+}
+
+template <typename T, int H>
+__device__ __forceinline__ void zero_raw(RawVec<T, H>& out) {
+  if constexpr (H == 1) {
+    out.v = T(0);
   } else {
-    *reinterpret_cast<T*>(out.w) = __ldg(p);
+#pragma unroll
+    for (int i = 0; i < (int)(sizeof(out.w) / 4); ++i) out.w[i] = 0u;
   }
 }
 
@@ -52,12 +75,20 @@ template <typename T, int H, typename Acc>
 __device__ __forceinline__ void widen(const RawVec<T, H>& r, Acc (&out)[H]) {
   if constexpr (std::is_same<T, uint16_t>::value) {
 #pragma unroll
-    for (int i = 0; i < H; ++i)
-      out[i] = __uint_as_float(__byte_perm(r.w[i / 2], 0x4B000000u, i % 2 ? 0x7632 : 0x7610)) - 8388608.0f;
+    for (int i = 0; i < H; ++i) {
+      uint32_t u;
+      if constexpr (H == 1)
+        u = 0x4B000000u | r.v;
+      else
+        u = __byte_perm(r.w[i / 2], 0x4B000000u, i % 2 ? 0x7632 : 0x7610);
+      out[i] = __uint_as_float(u) - 8388608.0f;
+    }
+  } else if constexpr (H == 1) {
+    out[0] = static_cast<Acc>(r.v);
   } else {
-    const T* e = reinterpret_cast<const T*>(r.w);
+    static_assert(std::is_same<T, float>::value, "vectors of uint16 or FP32");
 #pragma unroll
-    for (int i = 0; i < H; ++i) out[i] = static_cast<Acc>(e[i]);
+    for (int i = 0; i < H; ++i) out[i] = __uint_as_float(r.w[i]);
   }
 }
 
@@ -87,7 +118,8 @@ __device__ __forceinline__ void store_vec(Tout* op, const Acc (&val)[H]) {
     else
       asm volatile("st.global.cs.b32 [%0], %1;" ::"l"(op), "r"(q[0]) : "memory");
   } else if constexpr (std::is_same<Tout, uint16_t>::value) {
-    __stcs(op, to_u16_rn(val[0]));
+    const float c = INSIDE ? val[0] : fminf(fmaxf(val[0], 0.0f), 65535.0f);
+    __stcs(op, (uint16_t)__float_as_uint(c + 8388608.0f));
   } else if constexpr (std::is_same<Tout, float>::value && H == 4) {
     st_cs_v4(op, val[0], val[1], val[2], val[3]);
   } else if constexpr (std::is_same<Tout, float>::value && H == 2) {
@@ -100,7 +132,7 @@ __device__ __forceinline__ void store_vec(Tout* op, const Acc (&val)[H]) {
 
 // vol2 (uint16, may be NULL unless DUAL) receives the round-to-nearest-even
 // copy of the same values in the same pass.
-template <typename Tin, typename Tout, typename Acc, int H, int NH, bool DUAL>
+template <typename Tin, typename Tout, typename Acc, int H, int NH, bool DUAL, bool VEC>
 __global__ void __launch_bounds__(kThreadsX* kThreadsY)
 k_deskew(PlanView v, const Tin* __restrict__ raw, Tout* __restrict__ vol, uint16_t* __restrict__ vol2,
          int xtiles) {
@@ -131,12 +163,10 @@ k_deskew(PlanView v, const Tin* __restrict__ raw, Tout* __restrict__ vol, uint16
   auto fetch = [&](int n, RawVec<Tin, H>(&out)[NH]) {
 #pragma unroll
     for (int h = 0; h < NH; ++h) {
-      if (n >= 0 && n < v.nscan && lim[h] > 0) {
-        load_raw<Tin, H>(rowp + (size_t)n * plane + xh[h], out[h]);
-      } else {
-#pragma unroll
-        for (int i = 0; i < (int)sizeof(out[h].w) / 4; ++i) out[h].w[i] = 0u;
-      }
+      if (n >= 0 && n < v.nscan && lim[h] > 0)
+        load_raw<VEC, Tin, H>(rowp + (size_t)n * plane + xh[h], out[h]);
+      else
+        zero_raw(out[h]);
     }
   };
 
@@ -198,7 +228,7 @@ bool aligned(const void* q, int n) {
   return n % H == 0 && (uintptr_t)q % (sizeof(T) * H) == 0;
 }
 
-template <typename Tin, typename Tout, typename Acc, int H, int NH, bool DUAL>
+template <typename Tin, typename Tout, typename Acc, int H, int NH, bool DUAL, bool VEC>
 opm_status run(const opm_plan* p, const void* raw, void* vol, void* vol2, cudaStream_t s) {
   const PlanView& v = p->view;
   const int xtiles = (v.nx + kThreadsX * H * NH - 1) / (kThreadsX * H * NH);
@@ -208,23 +238,35 @@ opm_status run(const opm_plan* p, const void* raw, void* vol, void* vol2, cudaSt
     return fail(OPM_ERR_UNSUPPORTED, "deskew grid exceeds launch limits");
   dim3 block(kThreadsX, kThreadsY);
   dim3 grid((unsigned)gx, (unsigned)gy);
-  k_deskew<Tin, Tout, Acc, H, NH, DUAL><<<grid, block, 0, s>>>(v, static_cast<const Tin*>(raw), static_cast<Tout*>(vol),
-                                                               static_cast<uint16_t*>(vol2), xtiles);
+  k_deskew<Tin, Tout, Acc, H, NH, DUAL, VEC><<<grid, block, 0, s>>>(v, static_cast<const Tin*>(raw),
+                                                                    static_cast<Tout*>(vol),
+                                                                    static_cast<uint16_t*>(vol2), xtiles);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? OPM_OK : cuda_fail(e, "launch k_deskew");
 }
 
-// Vectors of H elements when the rows of every array start on one; else one
-// element per lane and instruction, kNH1 per lane: contiguous for the warp,
-// where element-wise vectors would leave strides of H between lanes (1001
-// columns, uint16 to FP32: 524 us element-wise, 353 us contiguous).
+// Vectors of H elements when the rows of every array start on one; FP32 input
+// that is only 8-byte aligned (an even width, a base off 16 bytes) in vectors of
+// two; aligned outputs alone keep their vector stores and take the raw elements
+// one by one.  Else one element per lane and instruction, contiguous for the
+// warp, where element-wise vectors would leave strides of H between lanes.  The
+// narrower forms hold 8 columns per lane where the row has them, since the walk's
+// own instructions bound them.  us, 100 x 256 x w at 45 deg, step 0.2, pixel
+// 0.115, element-wise half-vectors -> this: uint16 to FP32 w = 509 85 -> 38, raw
+// alone off 4 bytes 39 -> 34; FP32 to FP32 w = 509 52 -> 48 (55 with 4 per lane),
+// w = 506 49 -> 46; FP32 to uint16 w = 506 48 -> 42, w = 509 48 -> 49.
 template <typename Tin, typename Tout, typename Acc, int H, int NH, bool DUAL = false>
 opm_status run_aligned(const opm_plan* p, const void* raw, void* vol, void* vol2, cudaStream_t s) {
-  constexpr int kNH1 = 4;
   const int nx = p->view.nx;
-  if (aligned<Tin, H>(raw, nx) && aligned<Tout, H>(vol, nx) && (!DUAL || aligned<uint16_t, H>(vol2, nx)))
-    return run<Tin, Tout, Acc, H, NH, DUAL>(p, raw, vol, vol2, s);
-  return run<Tin, Tout, Acc, 1, kNH1, DUAL>(p, raw, vol, vol2, s);
+  const bool out = aligned<Tout, H>(vol, nx) && (!DUAL || aligned<uint16_t, H>(vol2, nx));
+  if (out && aligned<Tin, H>(raw, nx)) return run<Tin, Tout, Acc, H, NH, DUAL, true>(p, raw, vol, vol2, s);
+  if constexpr (sizeof(Tin) == 4)
+    if (aligned<Tin, 2>(raw, nx) && aligned<Tout, 2>(vol, nx) && (!DUAL || aligned<uint16_t, 2>(vol2, nx)))
+      return nx <= 4 * kThreadsX ? run<Tin, Tout, Acc, 2, 2, DUAL, true>(p, raw, vol, vol2, s)
+                                 : run<Tin, Tout, Acc, 2, 4, DUAL, true>(p, raw, vol, vol2, s);
+  if (out) return run<Tin, Tout, Acc, H, NH, DUAL, false>(p, raw, vol, vol2, s);
+  if (nx <= 4 * kThreadsX) return run<Tin, Tout, Acc, 1, 4, DUAL, true>(p, raw, vol, vol2, s);
+  return run<Tin, Tout, Acc, 1, 8, DUAL, true>(p, raw, vol, vol2, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -381,12 +423,12 @@ opm_status launch_deskew(const opm_plan* p, const void* raw, opm_dtype in_t, voi
   if (in_t == OPM_U16 && out_t == OPM_U16) {
     // 16-byte vectors where the rows allow them
     if (aligned<uint16_t, 8>(raw, p->view.nx) && aligned<uint16_t, 8>(vol, p->view.nx))
-      return run<uint16_t, uint16_t, float, 8, 1, false>(p, raw, vol, nullptr, s);
+      return run<uint16_t, uint16_t, float, 8, 1, false, true>(p, raw, vol, nullptr, s);
     return run_aligned<uint16_t, uint16_t, float, 4, 2>(p, raw, vol, nullptr, s);
   }
   if (in_t == OPM_F32 && out_t == OPM_F32) return run_aligned<float, float, float, 4, 1>(p, raw, vol, nullptr, s);
   if (in_t == OPM_F32 && out_t == OPM_U16) return run_aligned<float, uint16_t, float, 4, 1>(p, raw, vol, nullptr, s);
-  if (in_t == OPM_F64 && out_t == OPM_F64) return run<double, double, double, 1, 2, false>(p, raw, vol, nullptr, s);
+  if (in_t == OPM_F64 && out_t == OPM_F64) return run<double, double, double, 1, 2, false, true>(p, raw, vol, nullptr, s);
   return fail(OPM_ERR_UNSUPPORTED, "unsupported dtype pair");
 }
 
