@@ -72,16 +72,19 @@ struct Family {
 constexpr Family kFamilies[] = {{1, 3}, {1, 2}};
 constexpr int kNumFamilies = (int)(sizeof(kFamilies) / sizeof(kFamilies[0]));
 // Ring depth of the fast kernel for slab depth P: the deepest of 6 .. 3 stages
-// (two rows each) that still lets four of its CTAs into an SM's 228 KB of shared
-// memory (1 KB of it per CTA is the system's).  A fifth CTA's worth of rows in
-// flight is worth less than the fourth CTA: 200 x 512 x 2048 at 45 deg, step
-// 0.2, pixel 0.115 (21 planes), z + y: 203 us with 6 stages (3 CTAs per SM, the
-// schedule's fourth list a second wave), 162 with 4; 1024 columns at pixel / step 0.7 100 -> 77, 0.92 83 -> 68.
+// (two rows each) that still lets `ctas` of its CTAs into an SM's 228 KB of shared
+// memory (1 KB of it per CTA is the system's).  Alone it runs four, the
+// schedule's lists per SM, and a fifth CTA's worth of rows in flight is worth
+// less than the fourth CTA: 200 x 512 x 2048 at 45 deg, step 0.2, pixel 0.115 (21
+// planes), z + y: 203 us with 6 stages (3 CTAs per SM, the fourth list a second
+// wave), 162 with 4; 1024 columns at pixel / step 0.7 100 -> 77, 0.92 83 -> 68.
+// Beside a volume it runs one or two, with all 6: 300 x 512 x 2048 of the same
+// geometry, FP32 volume + z + y 1343 us with 4 stages, 1207 with 6; uint16 793, 722.
 constexpr int kFastStages[] = {6, 5, 4, 3};
 constexpr int fast_ring_bytes(int S, int P) { return S * (2 * P * 256 + 2 * 288 + 2 * 512 + 24) + 192; }
-constexpr int fast_stages(int P) {
+constexpr int fast_stages(int P, int ctas = 4) {
   for (int S : kFastStages)
-    if (4 * (fast_ring_bytes(S, P) + 1024) <= 228 * 1024) return S;
+    if (ctas * (fast_ring_bytes(S, P) + 1024) <= 228 * 1024) return S;
   return 3;
 }
 constexpr int kPerRun = 32;       // columns j per compute warp of the periodic kernel
@@ -145,8 +148,8 @@ struct opm_plan {
   int device;        // -1: created without a device
   void* dmem;        // one allocation holding every device table
   opm::PlanView view;
-  // opm_deskew_mip: the live view runs on `side` (highest priority, a
-  // quarter of the persistent grid) beside the volume on the caller's stream,
+  // opm_deskew_mip: the live view runs on `side` (highest priority, a quarter
+  // or half of the persistent grid) beside the volume on the caller's stream,
   // forked and joined through the two events; one_pass_fused selects the
   // single fused kernel instead (environment OPM_ONE_PASS_FUSED=1 at plan
   // creation).  `side` is NULL for a plan made without a device.
@@ -160,9 +163,9 @@ namespace opm {
 
 // Kernel launchers (one per translation unit).  Each returns OPM_OK or an
 // error already recorded with fail()/cuda_fail().
-// grid_div > 1 launches the persistent fast kernel with 1/grid_div of its
-// CTAs (each then walks grid_div of the schedule's lists), leaving room on
-// every SM for a kernel that runs beside it.
+// grid_div > 1 (a divisor of the plan's lists per SM) launches the persistent
+// fast kernel with 1/grid_div of its CTAs (each then walks grid_div of the
+// schedule's lists), leaving room on every SM for a kernel that runs beside it.
 opm_status launch_project(const opm_plan* p, const void* raw, opm_dtype in_t,
                           float* zmip, float* zsum, float* ymip, int32_t* argz,
                           cudaStream_t s, int grid_div = 1);

@@ -311,7 +311,7 @@ opm_status launch_fast(const opm_plan* p, const CUtensorMap& map, const ProjArgs
                        int grid_div) {
   if (p->family) return launch_per(p, map, args, s, grid_div);
   if (!p->view.units || !p->view.lists) return fail(OPM_ERR_INTERNAL, "plan has no fast-kernel schedule");
-  switch (fast_stages(args.P)) {
+  switch (fast_stages(args.P, p->lists_per_sm / std::max(1, grid_div))) {
     case 6: return launch_fast_s<6>(p, map, args, s, grid_div);
     case 5: return launch_fast_s<5>(p, map, args, s, grid_div);
     case 4: return launch_fast_s<4>(p, map, args, s, grid_div);
@@ -365,7 +365,7 @@ opm_status launch_project(const opm_plan* p, const void* raw, opm_dtype in_t, fl
   // the TMA kernels: uint16 rows on 16 bytes, z-MIP and / or y-MIP only
   const bool fast = u16 && !zsum && !argz && p->fast_ok && v.frow && !p->force_generic && encode_fn() != nullptr &&
                     (uintptr_t)raw % 16 == 0 && (size_t)v.ncols * 2 % 16 == 0 &&
-                    (int)(p->family ? per::total(kPerStages, P) : fast::total(fast_stages(P), P)) <= smax;
+                    (int)(p->family ? per::total(kPerStages, P) : fast::total(fast_stages(P, p->lists_per_sm / std::max(1, grid_div)), P)) <= smax;
 
   // initial values of the atomically combined outputs
   float* zinit = fast ? zmip : nullptr;
