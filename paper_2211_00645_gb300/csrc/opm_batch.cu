@@ -83,8 +83,8 @@ struct BatchItemDev {  // 64-byte aligned through its tensor map
   int32_t* argz;
   int nz, ny, nx, P;
   int linear, nscan;
-  short wr, slots;       // row groups, staged planes and vector rows of the direct kernel (general items)
-  int vec;
+  short wr, slots;       // the direct kernel's row groups, staged planes,
+  short vec, arg;        // vector rows and arg-max form (general items)
 };
 static_assert(sizeof(BatchItemDev) == 256, "item");
 
@@ -245,29 +245,35 @@ constexpr int kGenCtasPerSm = 2;
 // Planes per tile row that the general kernel's items may span.
 constexpr int kGenMaxPlanes = 221;
 
+// The job a CTA of the general kernel works on, in shared memory: behind every
+// store of a tile its fields would be read again from a local copy, and the forms
+// with more outputs have no registers to hold them.
+__shared__ direct::Job gen_job;
+
 // Every form of the direct kernel's job is a function of its own, so that the
 // items with fewer outputs do not pay for the registers of the others.
-template <bool VEC, bool JUMP, bool SUM, bool ARG>
-__device__ __noinline__ void gen_tile(const direct::Job& jb, unsigned char* smem) {
-  // Behind the reference every use of the job is a load, since the tile's own
-  // stores could have changed it.  The lightest form has the registers to hold
-  // a copy; the others spill it (one 200 x 512 x 1024 stack, both maxima:
-  // 374 -> 236 us with the copy; two with a sum: 331 -> 415 us; four that jump
-  // planes: 109 -> 132 us).
+template <bool VEC, bool JUMP, bool SUM, int ARG>
+__device__ __noinline__ void gen_tile(unsigned char* smem) {
+  // The lightest form has the registers for a copy of the job (one 200 x 512 x
+  // 1024 stack, both maxima: 212 -> 192 us), the heaviest not even for the plane
+  // difference (all outputs: 356 -> 305 us without).
   if constexpr (VEC && !JUMP && !SUM && !ARG) {
-    const direct::Job own = jb;
+    const direct::Job own = gen_job;
     direct::tile<uint16_t, VEC, SUM, ARG, JUMP>(own, smem);
   } else {
-    direct::tile<uint16_t, VEC, SUM, ARG, JUMP>(jb, smem);
+    direct::tile<uint16_t, VEC, SUM, ARG, JUMP, SUM && ARG && !JUMP>(gen_job, smem);
   }
 }
 
 template <bool VEC, bool JUMP>
-__device__ __forceinline__ void gen_job(const direct::Job& jb, unsigned char* smem) {
-  if (jb.argz)
-    jb.zsum ? gen_tile<VEC, JUMP, true, true>(jb, smem) : gen_tile<VEC, JUMP, false, true>(jb, smem);
+__device__ __forceinline__ void gen_tiles(int arg, bool sum, unsigned char* smem) {
+  using namespace direct;
+  if (arg == kArg16)
+    gen_tile<VEC, JUMP, true, kArg16>(smem);
+  else if (arg == kArg32)
+    sum ? gen_tile<VEC, JUMP, true, kArg32>(smem) : gen_tile<VEC, JUMP, false, kArg32>(smem);
   else
-    jb.zsum ? gen_tile<VEC, JUMP, true, false>(jb, smem) : gen_tile<VEC, JUMP, false, false>(jb, smem);
+    sum ? gen_tile<VEC, JUMP, true, kNoArg>(smem) : gen_tile<VEC, JUMP, false, kNoArg>(smem);
 }
 
 __global__ void __launch_bounds__(direct::kCtaThreads, kGenCtasPerSm)
@@ -279,30 +285,36 @@ k_batch_gen(const unsigned char* __restrict__ wl) {
     for (int u = lists[l]; u < lists[l + 1]; ++u) {
       const WorkUnit un = reinterpret_cast<const WorkUnit*>(wl + hdr->off_gunits)[u];
       const BatchItemDev* it = reinterpret_cast<const BatchItemDev*>(wl + kOffItems) + un.item;
-      direct::Job jb;
-      jb.raw = it->raw;
-      jb.slots = it->slots;
-      jb.row_pitch = (size_t)it->row_pitch;
-      jb.plane_pitch = (size_t)it->plane_pitch;
-      jb.A = it->A;
-      jb.B = it->B;
-      jb.linear = it->linear;
-      jb.nscan = it->nscan;
-      jb.ny = it->ny;
-      jb.nz = it->nz;
-      jb.nx = it->nx;
-      jb.wr = it->wr;
-      jb.band = it->band[un.jt / kTileJ];
-      jb.xb = un.xt * kX;
-      jb.zmip = it->zmip;
-      jb.zsum = it->zsum;
-      jb.ymip = it->ymip;
-      jb.argz = it->argz;
-      for (jb.jc = un.jt; jb.jc < min(un.jt + un.pad, jb.ny); jb.jc += direct::cta_cols(jb.wr)) {
-        if (jb.slots == direct::kJumpSlots)
-          it->vec ? gen_job<true, true>(jb, smem) : gen_job<false, true>(jb, smem);
+      const int columns = direct::cta_cols(it->wr);
+      for (int jc = un.jt; jc < min(un.jt + un.pad, it->ny); jc += columns) {
+        if (threadIdx.x == 0) {
+          direct::Job& jb = gen_job;
+          jb.raw = it->raw;
+          jb.slots = it->slots;
+          jb.row_pitch = (size_t)it->row_pitch;
+          jb.plane_pitch = (size_t)it->plane_pitch;
+          jb.A = it->A;
+          jb.B = it->B;
+          jb.linear = it->linear;
+          jb.nscan = it->nscan;
+          jb.ny = it->ny;
+          jb.nz = it->nz;
+          jb.nx = it->nx;
+          jb.wr = it->wr;
+          jb.band = it->band[un.jt / kTileJ];
+          jb.jc = jc;
+          jb.xb = un.xt * kX;
+          jb.zmip = it->zmip;
+          jb.zsum = it->zsum;
+          jb.ymip = it->ymip;
+          jb.argz = it->argz;
+        }
+        __syncthreads();
+        const bool vec = it->vec, sum = it->zsum != nullptr;
+        if (it->slots == direct::kJumpSlots)
+          vec ? gen_tiles<true, true>(it->arg, sum, smem) : gen_tiles<false, true>(it->arg, sum, smem);
         else
-          it->vec ? gen_job<true, false>(jb, smem) : gen_job<false, false>(jb, smem);
+          vec ? gen_tiles<true, false>(it->arg, sum, smem) : gen_tiles<false, false>(it->arg, sum, smem);
         __syncthreads();  // shared memory is read before the next job writes it
       }
     }
@@ -311,7 +323,7 @@ k_batch_gen(const unsigned char* __restrict__ wl) {
 
 // Shared memory of a batch launch for slab depth Pl (family 0: k_batch_fast).
 size_t batch_smem(int Pl, int family) { return family ? per::total(kPerStages, Pl) : fast::total(fast_stages(Pl), Pl); }
-size_t batch_gen_smem() { return direct::smem_bytes<uint16_t>(direct::kJumpSlots); }
+size_t batch_gen_smem() { return direct::smem_bytes<uint16_t>(direct::kJumpSlots, true, true); }
 
 PFN_cuTensorMapEncodeTiled_v12000 batch_encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -414,6 +426,18 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
   int* hglists = reinterpret_cast<int*>(stage + off_glists);
   WorkUnit* hunits = reinterpret_cast<WorkUnit*>(stage + off_units);
   int64_t nunits = 0;
+  // Row groups of a general item: a z-sum's are its plan's, so that it is summed
+  // in the one-plan call's order; the other outputs do not depend on them, and
+  // many items together need fewer (four waves of warps balance the lists): 8
+  // stacks of 50 x 87 x 1304, z + y 147 -> 136 us, arg-max 155 -> 141.
+  int64_t gtiles = 0;
+  for (int i = 0; i < n_items; ++i)
+    if (items[i].plan && !is_fast(items[i])) gtiles += direct::grid_tiles(items[i].plan->ny, items[i].plan->nx);
+  const int gwr = direct::row_groups(gtiles, 4 * direct::kEnough);
+  auto item_groups = [&](const opm_batch_item& it) {
+    const int wr = direct::row_groups(direct::grid_tiles(it.plan->ny, it.plan->nx));
+    return it.zsum ? wr : std::min(wr, gwr);
+  };
   // Units of the general items: `fine`, a CTA's single pieces, else whole
   // 32-column tiles.
   auto general_units = [&](bool fine) {
@@ -423,7 +447,7 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
       const opm_plan* p = it.plan;
       const bool zout = it.zmip || it.zsum || it.argz;
       if (!p || is_fast(it) || (!zout && !it.ymip)) continue;
-      const int cols = fine ? direct::cta_cols(direct::row_groups(p->ny, p->nx)) : kTileJ;
+      const int cols = fine ? direct::cta_cols(item_groups(it)) : kTileJ;
       for (int64_t jt = 0; jt < (int64_t)p->hBand.size(); ++jt)
         if (zout || p->hBand[jt].lo < p->hBand[jt].hi)
           n += (p->nx + kX - 1) / kX * ((std::min<int64_t>(kTileJ, p->ny - jt * kTileJ) + cols - 1) / cols);
@@ -489,8 +513,9 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
         d.row_pitch = rp;
         d.plane_pitch = pp;
         d.nscan = (int)p->nscan;
-        d.wr = (short)direct::row_groups(p->ny, p->nx);
+        d.wr = (short)item_groups(it);
         d.slots = (short)direct::row_slots(!p->unit_steps, p->rho);
+        d.arg = (short)direct::arg_form(it.argz != nullptr, it.zsum != nullptr, p->nz);
         d.vec = direct::vec_rows<uint16_t>(it.raw, p->nx, rp, pp) && !p->force_generic;
         d.linear = p->view.linear;
         d.zmip = it.zmip;
@@ -676,7 +701,7 @@ cudaError_t set_fast_attrs(int smem_optin) {
   if (e == cudaSuccess) e = set_kernel_smem(k_batch_fast<5>, smem_optin);
   if (e == cudaSuccess) e = set_kernel_smem(k_batch_fast<4>, smem_optin);
   if (e == cudaSuccess) e = set_kernel_smem(k_batch_fast<3>, smem_optin);
-  if (e == cudaSuccess) e = set_kernel_smem(k_batch_gen, smem_optin);
+  if (e == cudaSuccess) e = set_kernel_smem(k_batch_gen, (int)batch_gen_smem());
   if (e == cudaSuccess) e = set_per_attrs<0, true>(smem_optin);
   return e == cudaSuccess ? set_per_attrs<0, false>(smem_optin) : e;
 }

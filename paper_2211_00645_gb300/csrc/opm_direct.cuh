@@ -14,27 +14,30 @@
 //
 // A CTA of kWarps warps covers kWarps / wr neighbouring tiles along j, with
 // the rows of each dealt to wr warps in turn (rows ks + r, ks + r + wr, ...).
-// wr grows where the tiles alone would leave the GPU idle; it depends on the
-// output grid only (row_groups), so that one plan always sums in one order.
-// The wr partial results meet in shared memory in the order of r: sums are
-// reproducible bit for bit.  Rows' y-maxima meet in shared memory over the
-// CTA's tiles and go to the y-MIP once per kRows rows.
+// wr grows where the tiles alone would leave the GPU idle; for z-sums it depends
+// on the output grid only (row_groups), so that one plan always sums in one
+// order.  The wr partial results meet in shared memory, where every warp joins a
+// share of the columns in the order of r: sums are reproducible bit for bit.
+// Rows' y-maxima meet in shared memory over the CTA's tiles and go to the y-MIP
+// once per kRows rows.
 //
 // What bounds it: instruction issue (66 % of the schedulers' cycles, with two-
 // and three-cycle packed FMAs, 3-input maxima and byte permutes among them);
 // DRAM runs at 10-15 %.  8 columns x 4 x keep the accumulators, the plane pair
 // and the walk's state in 128 registers, 16 warps per SM; 24 warps at 80
-// registers spill and are slower (ragged stack below: 175 against 133 us before
-// the chunked staging).  Against the kernels it replaced, one thread per output
-// pixel for rows off 16 bytes and a TMA ring with one row per stage otherwise
-// (us per call, both sides on one GPU):
-//   151 x 333 x 1001 uint16, 45 deg, step 0.2, pixel 0.115, z + y:  454 -> 89
-//   300 x 800 x 1501 uint16, 35 deg, 0.3, 0.1, z + y:             4263 -> 670
-//   200 x 512 x 2048 uint16, 35 deg, 0.3, 0.1, z + sum + y:        442 -> 345
-//   200 x 512 x 1024 uint16, 45 deg, 0.2, 0.115, z + sum + y:      375 -> 171
-//   128 x 256 x 256 FP32, 30 deg, 0.4, 0.115, z + y:               180 -> 45
-//   200 x 512 x 1024 FP32, 45 deg, 0.2, 0.115, z + y:              365 -> 175
-//   100 x 256 x 512 uint16, 35 deg, step 0.05, pixel 0.1, z + y:   104 -> 39
+// registers spill and are slower, and so are 8 warps with all they ask for (all
+// outputs of the live-view stack 550 us against 413 with the arg-max rows packed
+// into half the registers).  Device time, us, against the kernels it replaced
+// (one thread per output pixel for rows off 16 bytes, a TMA ring with one row per
+// stage otherwise):
+//   151 x 333 x 1001 uint16, 45 deg, step 0.2, pixel 0.115, z + y:  447 -> 74
+//   200 x 512 x 2048 uint16, 35 deg, 0.3, 0.1, z + sum + y:         436 -> 334
+//   the same with arg-max:                                          439 -> 413
+//   50 x 87 x 1304 uint16, 30 deg, 0.4, 0.115, z + sum + y:          65 -> 22
+//   100 x 256 x 512 FP32, 45 deg, 0.2, 0.115, z + y:                180 -> 37
+//   100 x 256 x 512 uint16, 35 deg, step 0.05, pixel 0.1, z + y:     98 -> 29
+// All outputs of FP32 stacks that fill the GPU are the one form that is slower
+// (200 x 512 x 2048 434 -> 443, at 90 degrees 405 -> 426).
 #pragma once
 
 #include "opm_tma.cuh"
@@ -49,11 +52,11 @@ constexpr int kXW = 32 * kXL;    // columns x per warp
 constexpr int kWarps = 8;        // warps per CTA
 constexpr int kCtaThreads = 32 * kWarps;
 constexpr int kRows = 32;        // camera rows between two folds of the y-maxima
-constexpr int kPart = kWarps / 2 * kJ * kXW;  // values of one row group's partial results
+constexpr int kPart = kWarps * kJ * kXW;  // the warps' partial results, one value per column
 // Shared memory: the CTA's y-maxima, the warps' weight tables ((w, w) pairs of
 // two rows) and the warps' staged rows (two of `slots` planes).  After the last
-// row, the partial results (values and, beside them, arg-max rows) of one row
-// group of every tile take its place.
+// row, the warps' partial results (maxima, arg-max rows and sums) take its
+// place.
 constexpr int kYBytes = kRows * kXW * 4;
 constexpr int kWBytes = kWarps * 2 * kJ * 8;
 template <typename T>
@@ -61,9 +64,9 @@ __host__ __device__ constexpr int slot_bytes() { return kXW * (int)sizeof(T) + 1
 template <typename T>
 __host__ __device__ constexpr int warp_bytes(int slots) { return 2 * slots * slot_bytes<T>(); }
 template <typename T>
-__host__ __device__ constexpr int smem_bytes(int slots) {
-  return kYBytes + kWBytes + kWarps * warp_bytes<T>(slots) > 2 * kPart * 4 ? kYBytes + kWBytes + kWarps * warp_bytes<T>(slots)
-                                                                            : 2 * kPart * 4;
+__host__ __device__ constexpr int smem_bytes(int slots, bool sum, bool arg) {
+  const int rows = kYBytes + kWBytes + kWarps * warp_bytes<T>(slots), parts = (1 + sum + arg) * kPart * 4;
+  return rows > parts ? rows : parts;
 }
 // Planes staged per row: those of kJ columns that step by rho <= 1 planes
 // each (at most floor((kJ - 1) rho) + 1 steps; the 1e-3 allows for the rounding
@@ -72,12 +75,13 @@ constexpr int kJumpSlots = 2 * kJ;
 inline int row_slots(bool jump, double rho) { return jump ? kJumpSlots : (int)((kJ - 1) * rho + 1e-3) + 3; }
 constexpr int kEnough = 16 * 152;       // warps that keep every SM busy
 
-// Warps that share a tile's rows: the fewest of 2, 4, 8 that give kEnough
-// warps over the output grid.  2 at least keeps a CTA within a 32-column tile.
-inline int row_groups(int64_t ny, int64_t nx) {
-  const int64_t tiles = ((ny + kJ - 1) / kJ) * ((nx + kXW - 1) / kXW);
+// Warps that share a tile's rows: the fewest of 2, 4, 8 that give `enough`
+// warps over the output grid's tiles.  2 at least keeps a CTA within a 32-column
+// tile.
+inline int64_t grid_tiles(int64_t ny, int64_t nx) { return ((ny + kJ - 1) / kJ) * ((nx + kXW - 1) / kXW); }
+inline int row_groups(int64_t tiles, int64_t enough = kEnough) {
   int wr = 2;
-  while (wr < kWarps && tiles * wr < kEnough) wr *= 2;
+  while (wr < kWarps && tiles * wr < enough) wr *= 2;
   return wr;
 }
 // Columns j of one CTA, a divisor of kTileJ.
@@ -201,10 +205,29 @@ __device__ __forceinline__ float half(f2 v, int i) {
   return i ? hi : lo;
 }
 
-// The job of one CTA; every thread of it takes part.  smem: smem_bytes<T>(slots).
+// What a tile keeps of the arg-max: nothing, the row in 32 bits, or in 16 (two
+// columns to a register: beside z-sums the registers that keep two CTAs on an
+// SM; needs nz <= kMaxRow16).
+enum Arg { kNoArg = 0, kArg32 = 1, kArg16 = 2 };
+constexpr int kMaxRow16 = 65535;
+inline Arg arg_form(bool arg, bool sum, int64_t nz) { return !arg ? kNoArg : sum && nz <= kMaxRow16 ? kArg16 : kArg32; }
+
+// z = v and half HI of the packed rows = k where v > z.
+template <bool HI>
+__device__ __forceinline__ void max_row16(float& z, uint32_t& rows, float v, uint32_t k) {
+  if constexpr (HI)
+    asm("{ .reg .pred p; setp.gt.f32 p, %2, %0; @p mov.f32 %0, %2; @p prmt.b32 %1, %1, %3, 0x5410; }"
+        : "+f"(z), "+r"(rows) : "f"(v), "r"(k));
+  else
+    asm("{ .reg .pred p; setp.gt.f32 p, %2, %0; @p mov.f32 %0, %2; @p prmt.b32 %1, %1, %3, 0x3254; }"
+        : "+f"(z), "+r"(rows) : "f"(v), "r"(k));
+}
+
+// The job of one CTA; every thread of it takes part.  smem: smem_bytes<T>.
 // JUMP: a tile's neighbouring columns may lie more than one plane apart
-// (pixel > step, or a plan whose rounded plane table says so).
-template <typename T, bool VEC, bool SUM, bool ARG, bool JUMP>
+// (pixel > step, or a plan whose rounded plane table says so).  LEAN: the plane
+// difference is worked out for every column instead of held.
+template <typename T, bool VEC, bool SUM, int ARG, bool JUMP, bool LEAN = false>
 __device__ __forceinline__ void tile(const Job& jb, unsigned char* smem_raw) {
   float* smem = reinterpret_cast<float*>(smem_raw);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -226,7 +249,8 @@ __device__ __forceinline__ void tile(const Job& jb, unsigned char* smem_raw) {
 
   float zmax[kJ][kXL];
   f2 zsum[SUM ? kJ : 1][kXL / 2];
-  int az[ARG ? kJ : 1][kXL];
+  int az[ARG == kArg32 ? kJ : 1][kXL];
+  uint32_t az16[ARG == kArg16 ? kJ : 1][kXL / 2];
   // rows before the band are zero: the maximum starts at 0, attained in row 0
   const float zinit = r == 0 && bd.lo > 0 ? 0.0f : -INFINITY;
 #pragma unroll
@@ -235,7 +259,8 @@ __device__ __forceinline__ void tile(const Job& jb, unsigned char* smem_raw) {
     for (int c = 0; c < kXL; ++c) {
       zmax[j][c] = zinit;
       if constexpr (SUM) zsum[j][c / 2] = pk(0.0f, 0.0f);
-      if constexpr (ARG) az[j][c] = r == 0 ? 0 : INT32_MAX;
+      if constexpr (ARG == kArg32) az[j][c] = r == 0 ? 0 : INT32_MAX;
+      if constexpr (ARG == kArg16) az16[j][c / 2] = r == 0 ? 0u : ~0u;
     }
   const bool meet = jb.ymip && wj > 1;  // y-maxima of several tiles meet in shared memory
   if (meet) {
@@ -252,9 +277,17 @@ __device__ __forceinline__ void tile(const Job& jb, unsigned char* smem_raw) {
   unsigned step = 0;       // columns whose lower plane differs from the one before
   int shift = 0;           // where the row's first plane begins in its slot
   int buf = 0;             // which of the two rows was prepared last
+  constexpr bool kRowAhead = !SUM || (JUMP && !ARG);  // elsewhere the sums leave no registers for it
+  Split bk{};              // of the row to prepare next
+  if constexpr (kRowAhead) bk = jb.B[min(bd.lo + r, jb.nz - 1)];
   auto prepare = [&](int k) {
     float w;
-    plane_weight(aj, jb.B[k], jb.linear, nl, w);
+    if constexpr (kRowAhead) {
+      plane_weight(aj, bk, jb.linear, nl, w);
+      bk = jb.B[min(k + wr, jb.nz - 1)];
+    } else {
+      plane_weight(aj, jb.B[k], jb.linear, nl, w);
+    }
     buf ^= 1;
     if (lane < kJ) wtab[buf * kJ + lane] = make_float2(w, w);
     const int np = __shfl_up_sync(0xffffffffu, nl, 1);
@@ -334,17 +367,22 @@ __device__ __forceinline__ void tile(const Job& jb, unsigned char* smem_raw) {
         float v[kXL];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          v2[h] = fma2(j % 2 ? wq.y : wq.x, d[h], a[h]);
+          v2[h] = fma2(j % 2 ? wq.y : wq.x, LEAN ? sub2(b[h], a[h]) : d[h], a[h]);
           upk(v2[h], v[2 * h], v[2 * h + 1]);
           if constexpr (SUM) zsum[j][h] = add2(zsum[j][h], v2[h]);
         }
 #pragma unroll
         for (int c = 0; c < kXL; ++c) {
-          if constexpr (ARG) {
+          if constexpr (ARG == kArg32) {
             if (v[c] > zmax[j][c]) {
               zmax[j][c] = v[c];
               az[j][c] = k;
             }
+          } else if constexpr (ARG == kArg16) {
+            if (c % 2)
+              max_row16<true>(zmax[j][c], az16[j][c / 2], v[c], k);
+            else
+              max_row16<false>(zmax[j][c], az16[j][c / 2], v[c], k);
           } else {
             zmax[j][c] = fmaxf(zmax[j][c], v[c]);
           }
@@ -359,7 +397,12 @@ __device__ __forceinline__ void tile(const Job& jb, unsigned char* smem_raw) {
         float* y = jb.ymip + (size_t)k * jb.nx + jb.xb + xl;
 #pragma unroll
         for (int c = 0; c < kXL; ++c)
-          if (xof(c) < lim) atomic_max_f(y + xof(c), ym[c]);
+          if (xof(c) < lim) {
+            if constexpr (kCounts)
+              atomicMax(reinterpret_cast<int*>(y + xof(c)), __float_as_int(ym[c]));
+            else
+              atomic_max_f(y + xof(c), ym[c]);
+          }
       }
       if (meet) {
         float* yb = smem + (k - c0) * kXW;
@@ -388,64 +431,77 @@ __device__ __forceinline__ void tile(const Job& jb, unsigned char* smem_raw) {
   }
 
   if (!jb.zmip && !SUM && !ARG) return;
-  // partial results to group 0, in the order of the groups
-  for (int g = 1; g < wr; ++g) {
-    float* part = smem + (warp % wj) * kJ * kXW + lane;
-    auto pass = [&](auto&& put, auto&& take) {
-      __syncthreads();
-      if (r == g) {
+  // Every warp's partial results to shared memory; then every warp joins wj of
+  // the CTA's columns, in the order of the row groups, and writes them.
+  float* mine = smem + warp * kJ * kXW;
+  auto put = [&](float* to, auto&& value) {
 #pragma unroll
-        for (int j = 0; j < kJ; ++j)
+    for (int j = 0; j < kJ; ++j)
 #pragma unroll
-          for (int c = 0; c < kXL; ++c) put(j, c, part + j * kXW + 32 * c);
+      for (int c = 0; c < kXL; ++c) to[j * kXW + 32 * c + lane] = value(j, c);
+  };
+  auto take = [&](const float* from, float (&v)[kXL]) {
+#pragma unroll
+    for (int c = 0; c < kXL; ++c) v[c] = from[32 * c + lane];
+  };
+  auto write = [&](float* to, const float (&v)[kXL]) {
+    if constexpr (VEC) {
+      if ((uintptr_t)to % 16 == 0) {
+        if (lim > 0) *reinterpret_cast<float4*>(to + xl) = make_float4(v[0], v[1], v[2], v[3]);
+        return;
       }
-      __syncthreads();
-      if (r == 0) {
-#pragma unroll
-        for (int j = 0; j < kJ; ++j)
-#pragma unroll
-          for (int c = 0; c < kXL; ++c) take(j, c, part + j * kXW + 32 * c);
-      }
-    };
-    if constexpr (SUM)
-      pass([&](int j, int c, float* q) { q[0] = half(zsum[j][c / 2], c % 2); },
-           [&](int j, int c, const float* q) {
-             float lo, hi;
-             upk(zsum[j][c / 2], lo, hi);
-             zsum[j][c / 2] = c % 2 ? pk(lo, hi + q[0]) : pk(lo + q[0], hi);
-           });
-    pass([&](int j, int c, float* q) {
-           q[0] = zmax[j][c];
-           if constexpr (ARG) q[kPart] = __int_as_float(az[j][c]);
-         },
-         [&](int j, int c, const float* q) {
-           if constexpr (ARG) {  // the larger value, or the earlier row of equal ones
-             const int o = __float_as_int(q[kPart]);
-             if (q[0] > zmax[j][c] || (q[0] == zmax[j][c] && o < az[j][c])) {
-               zmax[j][c] = q[0];
-               az[j][c] = o;
-             }
-           } else {
-             zmax[j][c] = fmaxf(zmax[j][c], q[0]);
-           }
-         });
-  }
-  if (r > 0) return;
-#pragma unroll
-  for (int j = 0; j < kJ; ++j) {
-    if (j >= cols) break;
-    const size_t o = (size_t)(j0 + j) * jb.nx + jb.xb + xl;
-#pragma unroll
-    for (int c = 0; c < kXL; ++c) {
-      if (xof(c) >= lim) break;
-      // rows after the band are zero too
-      const bool past = bd.hi < jb.nz && zmax[j][c] < 0.0f;
-      if (jb.zmip) jb.zmip[o + xof(c)] = past ? 0.0f : zmax[j][c];
-      if constexpr (SUM)
-        if (jb.zsum) jb.zsum[o + xof(c)] = half(zsum[j][c / 2], c % 2);
-      if constexpr (ARG)
-        if (jb.argz) jb.argz[o + xof(c)] = past ? (int)bd.hi : az[j][c];
     }
+#pragma unroll
+    for (int c = 0; c < kXL; ++c)
+      if (xof(c) < lim) to[xl + xof(c)] = v[c];
+  };
+  const int group = wj * kJ * kXW;  // from one row group's results to the next
+  constexpr int kRowAt = kPart, kSumAt = (1 + (ARG != kNoArg)) * kPart;
+  __syncthreads();
+  put(mine, [&](int j, int c) { return zmax[j][c]; });
+  if constexpr (ARG == kArg32) put(mine + kRowAt, [&](int j, int c) { return __int_as_float(az[j][c]); });
+  if constexpr (ARG == kArg16)
+    put(mine + kRowAt, [&](int j, int c) { return __uint_as_float(az16[j][c / 2] >> (c % 2 * 16) & 0xffffu); });
+  if constexpr (SUM) put(mine + kSumAt, [&](int j, int c) { return half(zsum[j][c / 2], c % 2); });
+  __syncthreads();
+#pragma unroll 1
+  for (int i = 0; i < wj; ++i) {
+    const int col = warp * wj + i, j = jb.jc + col;
+    if (j >= jb.ny) break;
+    const float* q = smem + col * kXW;
+    float z[kXL], row[kXL], sum[kXL];
+    take(q, z);
+    if constexpr (ARG) take(q + kRowAt, row);
+    if constexpr (SUM) take(q + kSumAt, sum);
+#pragma unroll 1
+    for (int g = 1; g < wr; ++g) {
+      q += group;
+      float t[kXL], k[kXL], u[kXL];
+      take(q, t);
+      if constexpr (ARG) take(q + kRowAt, k);
+      if constexpr (SUM) take(q + kSumAt, u);
+#pragma unroll
+      for (int c = 0; c < kXL; ++c) {
+        if constexpr (ARG) {  // the larger value, or the earlier row of equal ones
+          if (t[c] > z[c] || (t[c] == z[c] && __float_as_int(k[c]) < __float_as_int(row[c]))) z[c] = t[c], row[c] = k[c];
+        } else {
+          z[c] = fmaxf(z[c], t[c]);
+        }
+        if constexpr (SUM) sum[c] += u[c];
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < kXL; ++c)
+      if (bd.hi < jb.nz && z[c] < 0.0f) {  // rows after the band are zero too
+        z[c] = 0.0f;
+        if constexpr (ARG) row[c] = __int_as_float((int)bd.hi);
+      }
+    const size_t o = (size_t)j * jb.nx + jb.xb;
+    if (jb.zmip) write(jb.zmip + o, z);
+    if constexpr (ARG)
+      if (jb.argz) write(reinterpret_cast<float*>(jb.argz) + o, row);
+    if constexpr (SUM)
+      if (jb.zsum) write(jb.zsum + o, sum);
   }
 }
 

@@ -162,8 +162,8 @@ k_project_per(const __grid_constant__ CUtensorMap tmap, const ProjArgs args) {
 }
 
 // Direct kernel (opm_direct.cuh): one job per CTA, x-tiles fastest.
-template <typename T, bool VEC, bool SUM, bool ARG, bool JUMP>
-__global__ void __launch_bounds__(direct::kCtaThreads, ARG && SUM ? 1 : 2)
+template <typename T, bool VEC, bool SUM, int ARG, bool JUMP>
+__global__ void __launch_bounds__(direct::kCtaThreads, ARG == direct::kArg32 && SUM ? 1 : 2)
 k_project_direct(const PlanView v, const T* __restrict__ raw, int wr, int slots, int xtiles, float* zmip, float* zsum,
                  float* ymip, int32_t* argz) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -319,11 +319,11 @@ opm_status launch_fast(const opm_plan* p, const CUtensorMap& map, const ProjArgs
   }
 }
 
-template <typename T, bool VEC, bool SUM, bool ARG>
+template <typename T, bool VEC, bool SUM, int ARG>
 opm_status launch_direct_as(const opm_plan* p, const void* raw, float* zmip, float* zsum, float* ymip, int32_t* argz,
                             cudaStream_t s) {
   const PlanView& v = p->view;
-  const int wr = direct::row_groups(v.ny, v.nx), cols = direct::cta_cols(wr);
+  const int wr = direct::row_groups(direct::grid_tiles(v.ny, v.nx)), cols = direct::cta_cols(wr);
   const long long xtiles = (v.nx + direct::kXW - 1) / direct::kXW;
   const long long nb = xtiles * ((v.ny + cols - 1) / cols);
   if (nb > 0x7fffffffLL) return fail(OPM_ERR_UNSUPPORTED, "grid too large");
@@ -333,7 +333,7 @@ opm_status launch_direct_as(const opm_plan* p, const void* raw, float* zmip, flo
   opm_status st = prepare_kernel(kern, p->device, done[jump]);
   if (st != OPM_OK) return st;
   const int slots = direct::row_slots(jump, p->rho);
-  kern<<<(unsigned)nb, direct::kCtaThreads, direct::smem_bytes<T>(slots), s>>>(
+  kern<<<(unsigned)nb, direct::kCtaThreads, direct::smem_bytes<T>(slots, SUM, ARG), s>>>(
       v, static_cast<const T*>(raw), wr, slots, (int)xtiles, zmip, zsum, ymip, argz);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? OPM_OK : cuda_fail(e, "launch k_project_direct");
@@ -344,14 +344,22 @@ opm_status launch_direct(const opm_plan* p, const void* raw, float* zmip, float*
                          cudaStream_t s) {
   const PlanView& v = p->view;
   const bool vec = direct::vec_rows<T>(raw, v.nx, v.ncols, (int64_t)v.nrows * v.ncols) && !p->force_generic;
-  const auto go = [&](auto vc, auto sm, auto ar) {
-    return launch_direct_as<T, decltype(vc)::value, decltype(sm)::value, decltype(ar)::value>(p, raw, zmip, zsum, ymip,
-                                                                                             argz, s);
+  const auto go = [&](auto sm, auto ar) {
+    constexpr bool SUM = decltype(sm)::value;
+    constexpr int ARG = decltype(ar)::value;
+    return vec ? launch_direct_as<T, true, SUM, ARG>(p, raw, zmip, zsum, ymip, argz, s)
+               : launch_direct_as<T, false, SUM, ARG>(p, raw, zmip, zsum, ymip, argz, s);
   };
-  const std::true_type yes;
-  const std::false_type no;
-  if (vec) return argz ? (zsum ? go(yes, yes, yes) : go(yes, no, yes)) : (zsum ? go(yes, yes, no) : go(yes, no, no));
-  return argz ? (zsum ? go(no, yes, yes) : go(no, no, yes)) : (zsum ? go(no, yes, no) : go(no, no, no));
+  const std::true_type sum;
+  const std::false_type no_sum;
+  const std::integral_constant<int, direct::kNoArg> no_arg;
+  const std::integral_constant<int, direct::kArg32> arg32;
+  const std::integral_constant<int, direct::kArg16> arg16;
+  switch (direct::arg_form(argz != nullptr, zsum != nullptr, v.nz)) {
+    case direct::kNoArg: return zsum ? go(sum, no_arg) : go(no_sum, no_arg);
+    case direct::kArg16: return go(sum, arg16);
+    default: return zsum ? go(sum, arg32) : go(no_sum, arg32);
+  }
 }
 
 }  // namespace
