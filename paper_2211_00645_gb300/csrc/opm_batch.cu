@@ -438,16 +438,19 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
     const int wr = direct::row_groups(direct::grid_tiles(it.plan->ny, it.plan->nx));
     return it.zsum ? wr : std::min(wr, gwr);
   };
-  // Units of the general items: `fine`, a CTA's single pieces, else whole
-  // 32-column tiles.
-  auto general_units = [&](bool fine) {
+  // Units of the general items cut into pieces of `piece` columns j, or of a CTA's
+  // where those are wider.
+  auto piece_columns = [&](const opm_batch_item& it, int piece) {
+    return std::max(piece, direct::cta_cols(item_groups(it)));
+  };
+  auto general_units = [&](int piece) {
     int64_t n = 0;
     for (int i = 0; i < n_items; ++i) {
       const opm_batch_item& it = items[i];
       const opm_plan* p = it.plan;
       const bool zout = it.zmip || it.zsum || it.argz;
       if (!p || is_fast(it) || (!zout && !it.ymip)) continue;
-      const int cols = fine ? direct::cta_cols(item_groups(it)) : kTileJ;
+      const int cols = piece_columns(it, piece);
       for (int64_t jt = 0; jt < (int64_t)p->hBand.size(); ++jt)
         if (zout || p->hBand[jt].lo < p->hBand[jt].hi)
           n += (p->nx + kX - 1) / kX * ((std::min<int64_t>(kTileJ, p->ny - jt * kTileJ) + cols - 1) / cols);
@@ -459,14 +462,14 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
   // fits the list does not depend on the pairing.
   bool pairs_fit = family > 0;
   if (family) {
-    int64_t n = general_units(false);
+    int64_t n = general_units(kTileJ);
     for (int i = 0; i < n_items; ++i)
       if (is_fast(items[i]))
         for (int jt = 0; jt < (int)items[i].plan->hBand.size(); ++jt)
           n += (items[i].plan->nx + kX - 1) / kX * pair_units(items[i].plan, jt, kchunk);
     pairs_fit = n <= max_units;
   }
-  bool fine = false;  // room for every general item's single pieces
+  int piece = kTileJ;  // columns j per unit of the general items
   int Pl = 2, Pg = 2, nseg = 0, nfast = 0;
   // first pass: fast items' units; second pass: general items' units after them
   for (int pass = 0; pass < 2; ++pass) {
@@ -540,18 +543,18 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
       if (it.ymip) hsegs[nseg++] = BatchSeg{it.ymip, (long long)(p->nz * p->nx)};
       const int xtiles = (int)((p->nx + kX - 1) / kX);
       const int jtiles = (int)((p->ny + kTileJ - 1) / kTileJ);
-      const int piece = fine ? direct::cta_cols(hitems[i].wr) : kTileJ;
+      const int cols = piece_columns(it, piece);
       for (int jt = 0; jt < jtiles; ++jt) {
         const Band bd = p->hBand[jt];
         const bool empty_unit = !fast && zout && bd.lo >= bd.hi;
         if (!fast) {
           if (bd.lo >= bd.hi && !empty_unit) continue;
-          for (int jc = jt * kTileJ; jc < std::min<int64_t>((jt + 1) * kTileJ, p->ny); jc += piece) {
+          for (int jc = jt * kTileJ; jc < std::min<int64_t>((jt + 1) * kTileJ, p->ny); jc += cols) {
             if (nunits + xtiles > max_units)
               return fail(OPM_ERR_UNSUPPORTED, std::string("the items need more than the ") + limit_what +
                                                    "'s limit of " + std::to_string(max_units) + " work units (split)");
             for (int xt = 0; xt < xtiles; ++xt)
-              hunits[nunits++] = WorkUnit{i, xt, jc, bd.lo, std::max(bd.lo, bd.hi), 0, 0, piece};
+              hunits[nunits++] = WorkUnit{i, xt, jc, bd.lo, std::max(bd.lo, bd.hi), 0, 0, cols};
           }
           continue;
         }
@@ -570,7 +573,10 @@ opm_status build_worklist(const opm_batch_item* items, int n_items, int kchunk, 
     }
     if (pass == 0) {
       nfast = (int)nunits;
-      fine = nunits + general_units(true) <= max_units;
+      // smaller pieces until every CTA has four, while the list has room: more
+      // of them balance little better and cost the host (2816 units 137 us, 1408 67)
+      while (piece > direct::kJ && general_units(piece) < 2 * nlists && nunits + general_units(piece / 2) <= max_units)
+        piece /= 2;
     }
   }
   const int ngen = (int)nunits - nfast;
