@@ -104,11 +104,11 @@ opm_status opm_plan_path(const opm_plan* plan, int* path, int* fam_p, int* fam_q
 /*
  * opm_plan_schedule - the live-view schedule of the fast and periodic kernels
  * (the live view of opm_project, Fig. 2d).  The work is cut into units of
- * *chunk_rows camera rows of one 32-column j-tile at one 128-column x-tile,
- * placed longest-first on *nlists lists, one per persistent CTA.  The plan
- * takes the largest of 256, 128, 64, 32 and 16 rows that gives at least 1.1
- * units per list, so that narrow stacks (an x-shard of one) still fill the
- * GPU.  All three are 0 for a plan without that schedule (the general
+ * *chunk_rows camera rows (rounded up to pairs of rows that step alike for the
+ * periodic kernel) of one 32-column j-tile at one 128-column x-tile, placed
+ * longest-first on *nlists lists, one per persistent CTA.  The plan takes the
+ * largest of 256, 128, 64, 32 and 16 rows that gives at least 1.1 units per
+ * list, so that narrow stacks (an x-shard of one) still fill the GPU.  All three are 0 for a plan without that schedule (the general
  * kernel's plans, and plans made with no CUDA device).  Any output pointer
  * may be NULL.  Errors: OPM_ERR_INVALID_ARG (plan NULL).
  */
@@ -330,7 +330,7 @@ opm_status opm_mip_backward(const opm_plan* plan, const float* g_zmip,
  * and that ask for z-MIP and/or y-MIP only run in one persistent launch of
  * the fast (or periodic) kernel over row chunks.  All other items (pixel >
  * step, ny < 32, or a z-sum or arg-max output) run in a second persistent
- * launch of the general kernel, one unit per tile and whole row band.
+ * launch of the general kernel, whole row bands per unit.
  * Results equal opm_project's for the same plan and outputs.
  */
 typedef struct opm_batch opm_batch; /* opaque; owns device + pinned work lists */
@@ -349,8 +349,9 @@ typedef struct {
 /*
  * opm_batch_create - work lists for up to max_items items and max_units
  * (<= 2^26) work units (a unit is one 32-column j-tile x 128-column x-tile x
- * row chunk of one item, or a whole row band for items of the general
- * kernel; 32 bytes of work list each).  Allocates device memory and pinned
+ * row chunk of one item, or a whole row band of a tile, or of a part of one
+ * where the list has room, for items of the general kernel; 32 bytes of work
+ * list each).  Allocates device memory and pinned
  * host memory once; the other batch calls allocate nothing except the CUDA
  * graph of opm_batch_launch_graph.
  * Errors: OPM_ERR_INVALID_ARG, OPM_ERR_OUT_OF_MEMORY, OPM_ERR_CUDA.

@@ -6,12 +6,13 @@
 // tiles into work units.  Items the fast kernels take (a fast-eligible plan,
 // z-MIP / y-MIP only) get one unit per (x-tile, j-tile, row chunk); all other
 // items (pixel > step, ny < 32, z-sum or arg-max outputs) get one unit per
-// (x-tile, j-tile) and whole row band, for the general kernel.  Each kind of
-// unit is sorted by decreasing length and dealt onto balanced lists, one per
-// persistent CTA of its kernel.  A CTA runs its kernel's producer and
-// consumer loops unit after unit on one mbarrier ring whose stage counter
-// carries on across units, so the next unit's slabs stream in while the
-// current one drains.  The fast items run in the kernel shape the caller
+// (x-tile, 8, 16 or 32 columns j) and whole row band, for the general kernel.
+// Each kind of unit is sorted by decreasing length and dealt onto balanced lists,
+// one per persistent CTA of its kernel.  A CTA of the fast kernels runs its
+// producer and consumer loops unit after unit on one mbarrier ring whose stage
+// counter carries on across units, so the next unit's slabs stream in while the
+// current one drains; a CTA of the general kernel runs the direct kernel's jobs
+// (opm_direct.cuh) one after another.  The fast items run in the kernel shape the caller
 // picks (opm_shape: periodic 32 x 2 or 16 x 2, fast 8 x 4) or all items in
 // the general kernel; the results are the same in every shape.
 //
@@ -242,7 +243,9 @@ k_batch_per(const unsigned char* __restrict__ wl, int Pl, unsigned* err) {
 // groups, or the 32-column j-tile's pieces one after another where the work
 // list has no room for single ones.
 constexpr int kGenCtasPerSm = 2;
-// Planes per tile row that the general kernel's items may span.
+// Planes per 32-column tile row that the general items may span: what lists have
+// accepted from the first version on (a slab of 221 planes filled the shared memory
+// of the kernel behind them then).  The direct kernel has no such bound.
 constexpr int kGenMaxPlanes = 221;
 
 // The job a CTA of the general kernel works on, in shared memory: behind every

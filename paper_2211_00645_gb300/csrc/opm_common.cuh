@@ -31,11 +31,6 @@ __device__ __forceinline__ void plane_weight_t(Split a, Split b, int linear, int
   }
 }
 
-template <typename T>
-__device__ __forceinline__ float to_f32(T v) {
-  return static_cast<float>(v);
-}
-
 // Load VEC consecutive elements starting at p as accumulator values.  `vec`
 // selects one aligned vector load; otherwise elements are loaded one by one
 // and those at or beyond `lim` read as zero.

@@ -94,7 +94,6 @@ __host__ __device__ constexpr int per_ofs(int p, int q, int ph, int t) { return 
 
 // Error bits recorded by kernels in the plan's device error word.
 enum : unsigned {
-  kErrSlabRange = 1u,   // a plane offset fell outside the staged slab
   kErrWaitTimeout = 2u, // an mbarrier wait gave up
   kErrOrder = 8u,       // the adjoint walk met a lower plane that decreased along j
 };

@@ -22,9 +22,9 @@
 //  * Only rows whose band can carry non-zero weight for the tile are visited;
 //    all other rows are exactly zero and enter the maxima as the value 0.
 //
-// Three kernels share that structure:
+// Two kernels share that structure, the third does without it:
 //  k_project_per   the periodic kernel (opm_periodic.cuh) for plans whose
-//                  pixel/step is a compiled ratio p/q (1/3): the fast
+//                  pixel/step is a compiled ratio p/q (1/3 or 1/2): the fast
 //                  kernel's producer and schedule, compute warps of 32
 //                  columns j x 2 columns x per lane with every plane step
 //                  at a compile-time position.
@@ -36,7 +36,8 @@
 //                  row band split into chunks (256 rows, fewer on narrow
 //                  stacks) whose z-maxima combine by atomic max, which
 //                  balances tiles of very different band length; a
-//                  persistent grid of 4 CTAs per SM walks the chunks.
+//                  persistent grid of 4 CTAs per SM (fewer beside a
+//                  volume) walks the chunks.
 //  k_project_direct  every other call: z-sum, first arg-max, FP32 input, rows
 //                  that are not a multiple of 16 bytes, any geometry
 //                  (opm_direct.cuh, shared with the batch).  It reads global

@@ -22,11 +22,11 @@ and exact, so the view is kept as three parts:
     nscan - 1 (built in one pass when that stack completed), until the new
     stack's pair p overwrites it with its own partial projection;
   * the mixed pair m, folded into the view directly.
-One opm_sliding_push call per frame does it in the library: two pair
-passes, one zeroing and two elementwise maxima instead of a whole
+One opm_sliding_push call per frame does it in the library: one kernel
+that folds both pairs and combines the parts, instead of a whole
 re-projection, and the view equals opm_project of the mixed stack bit for
-bit.  The completing frame also builds the next suffixes (nscan - 2
-maxima).  With a z-sum the mode re-projects the buffer after every frame
+bit.  The completing frame also builds the next suffixes (one pass over the
+slots).  With a z-sum the mode re-projects the buffer after every frame
 instead (sums would change their rounding order).
 """
 from __future__ import annotations

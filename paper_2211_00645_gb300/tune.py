@@ -8,8 +8,8 @@ results (bit for bit):
   kernel with 32 or 16 columns j per warp and 2 columns x per lane (plans
   whose pixel/step is a periodic family), ``fast_j8x4`` the fast kernel with
   8 columns j per warp, 4 columns x per lane and two rows per stage, and
-  ``gen_j8x4`` the general kernel (one row per stage, a whole row band per
-  unit);
+  ``gen_j8x4`` the general kernel (8 columns j per warp, 4 columns x per lane,
+  a whole row band per unit);
 * ``kchunk``: camera rows per work unit of the fast kernels (longer units
   stream more stages per ring fill but balance worse across CTAs);
 * ``ctas_per_sm``: persistent CTAs per SM (1..4; the general kernel takes
