@@ -23,8 +23,8 @@
 // What bounds it: L2 traffic (a push reads the run and one slot and writes a
 // slot and the view, 45 MB at 200 planes) and the latency of search and walk.
 // Device time back to back, 512 x 2048 frames, 35 deg, step 0.3, pixel 0.1: a
-// pair 7.1 us, with a z-sum 7.6; a push on 24 planes 12.5; 87 x 1304 frames of
-// 24 planes: pair 3.2, push 4.7.  (A scatter of shared and global atomic maxima
+// pair 7.2 us, with a z-sum 7.6; a push on 24 planes 11.4; 87 x 1304 frames of
+// 24 planes: pair 3.2, push 4.8.  (A scatter of shared and global atomic maxima
 // took 9.8 and 15; a push made of two of them, one zeroing and two elementwise
 // maxima 28, and 15 on the small frames.)
 // Four rows' loads ahead in a short run cost occupancy and were slower.
@@ -383,10 +383,12 @@ __device__ __forceinline__ bool fold_live(const PlanView& v, const Parts& t, con
   }
 }
 
-// 64 registers where columns are shared, so that the rows (and the push's idle
-// columns) beside them find room for enough warps.
+// Five CTAs per SM where a warp has a column (a push of 512 x 2048 frames 12.8 us
+// at the 56 registers it would take, 11.6 at 48); where columns are shared 64
+// registers, so that the rows and a push's idle columns beside them find room for
+// enough warps.
 template <int S>
-constexpr int min_ctas() { return S == 1 ? 1 : 32 / cta_warps(S); }
+constexpr int min_ctas() { return S == 1 ? 5 : 32 / cta_warps(S); }
 
 // Pair A into the outputs (any of them NULL): columns [j0, j1) hold its voxels.
 template <bool VEC, bool SUM, int S, int G>
@@ -574,6 +576,7 @@ static double run_rows(const opm_plan* p) { return std::min((double)p->nz, 1.0 /
 // Rows off 8 bytes cost four times the loads, which sharing hides as well:
 //   333 x 1001 with a z-sum, step 0.2, pixel 0.115, 75 deg (6.7, 704) 8.4 / 6.3 / - / 35   7.3
 static int column_share(double run, long long warps, bool vec) {
+  if (warps == 0) return 1;
   if (run >= 64.0 && (double)warps <= (vec ? 0.17 : 1.0) * run) return 16;
   if (run >= 64.0 && (double)warps <= 1.5 * run) return 8;
   return run * 1000.0 > (vec ? 12.0 : 5.0) * (double)warps ? 4 : 1;
