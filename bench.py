@@ -54,11 +54,11 @@ KERNEL_SOURCES = {
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per full-size
 # launch from ncu captures, keyed by the hash of the kernel's sources at
 # capture time (reported as null once a source has changed).  Both captured at
-# full size.  periodic: 448.36 MB read, 7.33 MB written, 70.2 M warp
-# instructions; volume_f32: 450.21 MB read, 4221.39 MB written.
+# full size.  periodic: 448.31 MB read, 6.75 MB written, 70.2 M warp
+# instructions; volume_f32: 449.15 MB read, 4221.44 MB written.
 NCU_TRAFFIC = {
-    "periodic": {"src_sha": "ded4b65b407e", "bytes_per_launch": 455692288, "warp_insts_per_launch": 70173217},
-    "volume_f32": {"src_sha": "10e9902e7130", "bytes_per_launch": 4671601408},
+    "periodic": {"src_sha": "9ebcf3423edf", "bytes_per_launch": 455053312, "warp_insts_per_launch": 70173184},
+    "volume_f32": {"src_sha": "894de42aa02a", "bytes_per_launch": 4670589440},
 }
 
 L2_BYTES = 129 * 10**6  # L2 of the GB300 (bytes)

@@ -26,18 +26,18 @@
 // DRAM runs at 10-15 %.  8 columns x 4 x keep the accumulators, the plane pair
 // and the walk's state in 128 registers, 16 warps per SM; 24 warps at 80
 // registers spill and are slower, and so are 8 warps with all they ask for (all
-// outputs of the live-view stack 550 us against 413 with the arg-max rows packed
+// outputs of the live-view stack 550 us against 413-422 with the arg-max rows packed
 // into half the registers).  Device time, us, against the kernels it replaced
 // (one thread per output pixel for rows off 16 bytes, a TMA ring with one row per
 // stage otherwise):
 //   151 x 333 x 1001 uint16, 45 deg, step 0.2, pixel 0.115, z + y:  447 -> 74
-//   200 x 512 x 2048 uint16, 35 deg, 0.3, 0.1, z + sum + y:         436 -> 334
-//   the same with arg-max:                                          439 -> 413
+//   200 x 512 x 2048 uint16, 35 deg, 0.3, 0.1, z + sum + y:         436 -> 332
+//   the same with arg-max:                                          439 -> 413-422
 //   50 x 87 x 1304 uint16, 30 deg, 0.4, 0.115, z + sum + y:          65 -> 22
 //   100 x 256 x 512 FP32, 45 deg, 0.2, 0.115, z + y:                180 -> 37
 //   100 x 256 x 512 uint16, 35 deg, step 0.05, pixel 0.1, z + y:     98 -> 29
 // All outputs of FP32 stacks that fill the GPU are the one form that is slower
-// (200 x 512 x 2048 434 -> 443, at 90 degrees 405 -> 426).
+// (200 x 512 x 2048 433 -> 442, at 90 degrees 405 -> 425).
 #pragma once
 
 #include "opm_tma.cuh"

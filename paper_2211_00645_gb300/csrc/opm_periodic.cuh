@@ -13,11 +13,12 @@
 // first and last column of each plane interval (along a row the voxels of
 // one interval are a + w (b - a) with w increasing in j, and a correctly
 // rounded FMA is monotone in w; the plan checks that the weights increase
-// inside every interval).  Every q-th column has the same weight, bit for bit
-// (the plan builds its column table from the exact ratio and checks it), so a
-// row's q weights stay in registers.  The arithmetic is that of every other
-// kernel of the library (the plan's weights, FMA on the exact plane
-// difference), so the outputs are the same bit for bit.
+// inside every interval).  Where pixel / step is p/q up to rounding every q-th
+// column has the same weight, bit for bit (the plan builds its tables from the
+// exact ratio), and a row's q weights stay in registers (REP); other plans that
+// step alike read every column's (131 us against 129 below).  The arithmetic is
+// that of every other kernel of the library (the plan's weights, FMA on the exact
+// plane difference), so the outputs are the same bit for bit.
 //
 // The two rows of a stage have the same phase: the plan pairs every tile's
 // rows by phase (RowPair), and a unit is a run of such pairs.  That leaves q
@@ -27,10 +28,10 @@
 // quarter to two thirds of it), and with rows paired in order six of nine 6 KB
 // bodies were in use.  What bounds it now is dispatch: packed FMAs, adds and
 // 3-input maxima take two to three cycles each, and more warps do not help (5
-// CTAs per SM: 145 us below).  us, rows in order with a weight pair per column
-// -> this: 200 x 512 x 2048 (35 deg, step 0.3, pixel 0.1) 149 -> 136, 1024 of
-// its columns 86 -> 79, 256 columns 40 -> 35; six two-channel stacks of the
-// serving mix 863 -> 754; 1/2 (step 0.2) 155.5 -> 155.
+// CTAs per SM were slower).  Device time, us, rows in order with a weight pair per
+// column -> this: 200 x 512 x 2048 (35 deg, step 0.3, pixel 0.1) 142 -> 129, 1024 of
+// its columns 79 -> 73, 256 columns 32 -> 30; step 0.2 (1/2) 151 -> 150, 80 -> 78,
+// 25 -> 24.
 //
 // CTA: one producer warp (TMA ring of two camera rows per stage, as in
 // opm_tma.cuh) and two compute warps.  Each compute warp owns all 32 columns

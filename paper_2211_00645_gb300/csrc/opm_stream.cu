@@ -20,13 +20,12 @@
 // together with the maxima it combines them with; columns outside both runs are
 // passed through unsearched.
 //
-// What bounds it: L2 traffic (a push reads the run and one slot and writes a
-// slot and the view, 45 MB at 200 planes) and the latency of search and walk.
-// Device time back to back, 512 x 2048 frames, 35 deg, step 0.3, pixel 0.1: a
-// pair 7.2 us, with a z-sum 7.6; a push on 24 planes 11.4; 87 x 1304 frames of
-// 24 planes: pair 3.2, push 4.8.  (A scatter of shared and global atomic maxima
-// took 9.8 and 15; a push made of two of them, one zeroing and two elementwise
-// maxima 28, and 15 on the small frames.)
+// What bounds it: the latency of search and walk, and issue (a push at 55 %; L2
+// and DRAM at 18 %); the suffix pass runs at 82 % of DRAM.  Device time back to
+// back, 512 x 2048 frames, 35 deg, step 0.3, pixel 0.1: a pair 7.2 us, with a z-sum
+// 7.6; a push on 200 planes 13.1; 87 x 1304 frames: pair 3.2, push 4.8.  (A scatter
+// of shared and global atomic maxima took 10 and 15; a push made of two of them, one
+// zeroing and two elementwise maxima 31, and 15 on the small frames.)
 // Four rows' loads ahead in a short run cost occupancy and were slower.
 #include <algorithm>
 
