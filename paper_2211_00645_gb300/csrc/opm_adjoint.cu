@@ -380,7 +380,8 @@ k_mip_tile(const __grid_constant__ CUtensorMap tmap, PlanView v, const float* __
       __syncwarp();
       if (lane == 0) tma_store_tile(&tmap, tile, xb, k0, na);
     } else if (xin) {
-      __syncwarp();
+      // a lane stores the columns it summed itself, so nothing is waited for here:
+      // the lanes past the grid's edge are already at the next tile's wait
       for (int t = 0; t < np; ++t)
         for (int kk = 0; kk < nk; ++kk)
           raw[((size_t)(na + t) * v.nrows + k0 + kk) * v.ncols + x] = tile[(t * kMipK + kk) * 32 + lane];
